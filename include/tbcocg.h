@@ -11,13 +11,17 @@
  * Eq. (GreensFunc), or their energy integral folded into Mulliken
  * populations.  H is the tight-binding Hamiltonian matrix and S the overlap
  * matrix of Section 2.2; both are real symmetric, S positive definite.
- * The solver is the generalized shifted COCG method of Section 3.3: one seed
- * system (Eq. shift-E) iterated by Eqs. (CGp:p), (CGp:x), (CGp:r) with
+ * The solver is the generalized shifted COCG method of Section 3.3 with
  * r' = S^-1 r from an inner solve (CG in FP64; with TB_MIXED, FP64
- * iterative refinement with FP32 corrections), every other shift carried by the scalar
- * recurrence Eq. (shift:pi) through the collinear residuals of
- * Eq. (collinear), and seed switching.  The generalized Lanczos process of
- * Section 3.2 (Eqs. 1.13, 1.18) is exported as well.
+ * iterative refinement with FP32 corrections).  With real H, S and e_j the
+ * collinear residuals of Eq. (collinear) are complex multiples of one real
+ * vector, so the iteration carries that real vector (the Lanczos vector of
+ * Section 3.2 in the residual space) and each shift the complex scalars of
+ * its own recurrence: the iterates of Eqs. (CGp:p), (CGp:x), (CGp:r) and
+ * (shift:pi) in real arithmetic.  The seed shift and its switching choose
+ * the real shift of the products and name the shift whose breakdown ends a
+ * column.  The generalized Lanczos process of Section 3.2 (Eqs. 1.13, 1.18)
+ * is exported as well.
  *
  * Conventions for every entry point
  *  - Return value: tb_status, TB_OK = 0.  tb_status_string() names it.
@@ -248,7 +252,7 @@ tb_status tb_shifted_cocg(tb_handle *h, int32_t K, const double *z, int32_t R, c
  * (tb_mulliken_orbital's work), every candidate of
  *   panel width P in {32, 64, 128, 256} (not above the orbital count),
  *   panels in flight (worker streams) in {2, 4}, and, on the mixed path
- *   with Chebyshev corrections, the Chebyshev-step form: 4 complex columns
+ *   with Chebyshev corrections, the Chebyshev-step form: 4 pairs of columns
  *   per thread at 3 resident CTAs per SM, or 2 at 4 CTAs per SM,
  * on P x (panels in flight) columns spread evenly over the system (an
  * untimed call first builds the graphs and the spectrum bounds; CUDA events
@@ -264,7 +268,7 @@ tb_status tb_shifted_cocg(tb_handle *h, int32_t K, const double *z, int32_t R, c
 typedef struct {
     int32_t panel;        /* right-hand sides per panel                          */
     int32_t streams;      /* panels in flight                                    */
-    int32_t cheb_cpt;     /* complex columns per thread of the Chebyshev step (0: not used) */
+    int32_t cheb_cpt;     /* pairs of columns per thread of the Chebyshev step (0: not used) */
     int32_t ctas_per_sm;  /* resident CTAs per SM of that step (0: not used)     */
     double rate;          /* measured shift*RHS*iterations per second            */
 } tb_tune;
@@ -554,9 +558,9 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle *h, int32_t j, int32_t n_step
 enum {
     TB_K_INNER_SPMV = 0,   /* w = S r and the inner-CG dot products        */
     TB_K_INNER_UPDATE = 1, /* inner-CG vector updates                      */
-    TB_K_OUTER_SPMM = 2,   /* q = (z_s S - H) r', A p and mu               */
-    TB_K_OUTER_UPDATE = 3, /* r_{n+1} = r_n - alpha A p                    */
-    TB_K_FINISH = 4,       /* rho_{n+1}                                    */
+    TB_K_OUTER_SPMM = 2,   /* W = (H - sigma S) u' and a_n                 */
+    TB_K_OUTER_UPDATE = 3, /* u_{n+1} from W, u_n, u_{n-1}                 */
+    TB_K_FINISH = 4,       /* t_{n+1} = u^T u'                             */
     TB_K_SHIFT_STEP = 5,   /* all shifts, projections, seed switching      */
     TB_K_FULL_UPDATE = 6,  /* full-mode x^k, p^k updates                   */
     TB_K_OTHER = 7,        /* set-up, outputs, Lanczos helpers             */

@@ -490,8 +490,8 @@ tb_status inner_cg32(View& v, const PanelDev& p, int inner_max, int& pred, int64
 // TB_DEBUG=1: the refinement state of the first real columns after a failed round
 void debug_inner32(View& v, const PanelDev& p, int round, cudaStream_t st) {
     if (!std::getenv("TB_DEBUG")) return;
-    std::vector<InnerState> is(2 * p.P);
-    cudaMemcpyAsync(is.data(), p.inner32, sizeof(InnerState) * 2 * p.P, cudaMemcpyDeviceToHost, st);
+    std::vector<InnerState> is(p.P);
+    cudaMemcpyAsync(is.data(), p.inner32, sizeof(InnerState) * p.P, cudaMemcpyDeviceToHost, st);
     cudaStreamSynchronize(st);
     std::fprintf(stderr, "[tb] round %d flags %d %d %d %d %d\n", round, v.flags_host[0], v.flags_host[1],
                  v.flags_host[2], v.flags_host[3], v.flags_host[4]);
@@ -502,7 +502,7 @@ void debug_inner32(View& v, const PanelDev& p, int round, cudaStream_t st) {
         std::fprintf(stderr, "[tb] breakdown it %g rc %g gam %.6e del %.6e den %.6e b2 %.6e gprev %.6e alpha %.6e\n",
                      dbg[0], dbg[1], dbg[2], dbg[3], dbg[4], dbg[5], dbg[6], dbg[7]);
     }
-    for (int i = 0; i < 2 * p.P && i < 8; ++i)
+    for (int i = 0; i < p.P && i < 8; ++i)
         std::fprintf(stderr, "[tb]   col %d: gprev %.3e alpha %.3e beta %.3e b2 %.3e conv %d skip %d scale %.3e\n",
                      i, is[i].gamma_prev, is[i].alpha, is[i].beta, is[i].bnorm2, is[i].conv, is[i].skip,
                      is[i].scale);
@@ -554,23 +554,23 @@ tb_status mixed_inner(View& v, const PanelDev& p, const double2* b, int inner_ma
         tb_status s = inner_cg32(v, p, inner_max, pred32, inner_total, st);
         if (s != TB_OK) return s;
         if (g_trace && p.hist) {
-            const size_t nh = (size_t)HIST_IT * 2 * p.P * 4;
+            const size_t nh = (size_t)HIST_IT * p.P * 4;
             std::vector<double> hv(nh);
             cudaMemcpyAsync(hv.data(), p.hist, sizeof(double) * nh, cudaMemcpyDeviceToHost, st);
             cudaStreamSynchronize(st);
-            for (int rc = 0; rc < 2 * p.P; ++rc) {
-                const double g0 = hv[((size_t)0 * 2 * p.P + rc) * 4];
+            for (int rc = 0; rc < p.P; ++rc) {
+                const double g0 = hv[((size_t)0 * p.P + rc) * 4];
                 double gmax = 0.0;
                 int itmax = 0;
                 for (int it = 0; it < HIST_IT; ++it) {
-                    const double g = hv[((size_t)it * 2 * p.P + rc) * 4];
+                    const double g = hv[((size_t)it * p.P + rc) * 4];
                     if (g > gmax) { gmax = g; itmax = it; }
                 }
                 if (g0 > 0.0 && gmax > 10.0 * g0) {
                     std::fprintf(stderr, "[tb] round %d col %d: gamma grows %.3e -> %.3e at it %d\n", round, rc, g0,
                                  gmax, itmax);
                     for (int it = 0; it < 30; ++it) {
-                        const double* e = &hv[((size_t)it * 2 * p.P + rc) * 4];
+                        const double* e = &hv[((size_t)it * p.P + rc) * 4];
                         std::fprintf(stderr, "[tb]     it %2d gam %.6e del %.6e alpha %.6e beta %.6e\n", it, e[0], e[1],
                                      e[2], e[3]);
                     }
@@ -593,8 +593,8 @@ tb_status mixed_inner(View& v, const PanelDev& p, const double2* b, int inner_ma
         if (g_trace) {
             cudaMemcpyAsync(v.flags_host, p.flags, NFLAGS * sizeof(int), cudaMemcpyDeviceToHost, st);
             cudaStreamSynchronize(st);
-            std::vector<InnerState> is(2 * p.P);
-            cudaMemcpyAsync(is.data(), p.inner32, sizeof(InnerState) * 2 * p.P, cudaMemcpyDeviceToHost, st);
+            std::vector<InnerState> is(p.P);
+            cudaMemcpyAsync(is.data(), p.inner32, sizeof(InnerState) * p.P, cudaMemcpyDeviceToHost, st);
             cudaStreamSynchronize(st);
             double smin = 1e300, smax = 0.0;
             for (auto& x : is)
@@ -624,7 +624,6 @@ struct InnerCtx {
     int64_t total = 0;
     int redo = 0;
     ChebPlan cheb;
-    bool res_exact = false;   // Rin holds b - S r' of the last solve (double-float refinement residual)
     // the Chebyshev steps of a full and of a last round as graphs, captured
     // on first use for the PanelDev of this context (its buffers stay fixed)
     cudaGraphExec_t cheb_graph[2] = {nullptr, nullptr};
@@ -655,17 +654,14 @@ tb_status inner_redo(View& v, const PanelDev& p, const double2* b, int inner_max
 // outer step) and their status said that more are needed.
 tb_status inner_solve(View& v, const PanelDev& p, const double2* b, int inner_max, InnerCtx& ic,
                       cudaStream_t st, int first_round = 0) {
-    ic.res_exact = false;
     if (!p.mixed) return inner_cg(v, p, inner_max, ic.pred, ic.total, st);
     tb_status s = mixed_inner(v, p, b, inner_max, ic.pred32, ic.rounds, ic.total, ic.cheb, ic.cheb_graph, st,
                               first_round);
-    if (s == TB_OK) ic.res_exact = b == p.Rcur;
     if (s != TB_ERR_BREAKDOWN && s != TB_ERR_NOT_CONVERGED) return s;
     return inner_redo(v, p, b, inner_max, ic, st);
 }
 
 tb_status inner_redo(View& v, const PanelDev& p, const double2* b, int inner_max, InnerCtx& ic, cudaStream_t st) {
-    ic.res_exact = false;
     ic.cheb.n = 0;   // the rest of this solve uses the FP32 CG corrections
     // The FP32 corrections failed to converge (or produced a non-finite
     // residual): redo this inner solve with the FP64 CG, on the device.
@@ -676,7 +672,7 @@ tb_status inner_redo(View& v, const PanelDev& p, const double2* b, int inner_max
     TB_CK(cudaStreamSynchronize(st));
     const int keep = v.flags_host[0] & ~ERR_INNER;
     TB_CK(cudaMemcpyAsync(p.flags, &keep, sizeof(int), cudaMemcpyHostToDevice, st));
-    TB_CK(cudaMemcpyAsync(p.Rin, b, sizeof(double2) * (size_t)p.npad * p.P, cudaMemcpyDeviceToDevice, st));
+    TB_CK(cudaMemcpyAsync(p.Rin, b, sizeof(double2) * (size_t)p.npad * p.C, cudaMemcpyDeviceToDevice, st));
     const tb_status s = inner_cg(v, p, inner_max, ic.pred, ic.total, st);
     if (s != TB_OK) return s;
     launch_split_panel(p, st);
@@ -687,10 +683,11 @@ tb_status inner_redo(View& v, const PanelDev& p, const double2* b, int inner_max
 
 // Device workspace of a panel's inner solves (FP64 CG; with p.mixed the FP32
 // CG and refinement buffers too) and of its grid reductions: everything but
-// the shift state.  p.P, p.npad, p.grid and p.mixed must be set.
+// the shift state.  p.P (even), p.npad, p.grid and p.mixed must be set.
 tb_status alloc_inner_workspace(Cleanup& cl, PanelDev& p, cudaStream_t st) {
     const int P = p.P;
-    const size_t nv = (size_t)p.npad * P;
+    p.C = P / 2;
+    const size_t nv = (size_t)p.npad * p.C;
     tb_status s;
     double2** vecs[] = {&p.Rcur, &p.Rprev, &p.Rp, &p.W, &p.Rin, &p.Pin, &p.Sin};
     for (double2** v : vecs) {
@@ -704,24 +701,24 @@ tb_status alloc_inner_workspace(Cleanup& cl, PanelDev& p, cudaStream_t st) {
         }
         if ((s = dalloc(cl, &p.RpS, nv)) != TB_OK) return s;
         TB_CK(cudaMemsetAsync(p.RpS, 0, sizeof(float4) * nv, st));
-        if ((s = dalloc(cl, &p.inner32, 3 * 2 * P)) != TB_OK) return s;
-        if ((s = dalloc(cl, &p.acc32, 8 * P)) != TB_OK) return s;
-        if ((s = dalloc(cl, &p.cgs, 4 * P)) != TB_OK) return s;
-        if ((s = dalloc(cl, &p.cgu, 2 * P)) != TB_OK) return s;
+        if ((s = dalloc(cl, &p.inner32, 3 * P)) != TB_OK) return s;
+        if ((s = dalloc(cl, &p.acc32, 4 * P)) != TB_OK) return s;
+        if ((s = dalloc(cl, &p.cgs, 2 * P)) != TB_OK) return s;
+        if ((s = dalloc(cl, &p.cgu, P)) != TB_OK) return s;
         if ((s = dalloc(cl, &p.ticket32, 1)) != TB_OK) return s;
         TB_CK(cudaMemsetAsync(p.ticket32, 0, sizeof(unsigned), st));
         if ((s = dalloc(cl, &p.dbg, 8)) != TB_OK) return s;
         if (std::getenv("TB_TRACE")) {
-            if ((s = dalloc(cl, &p.hist, (size_t)HIST_IT * 2 * P * 4)) != TB_OK) return s;
-            TB_CK(cudaMemsetAsync(p.hist, 0, sizeof(double) * HIST_IT * 2 * P * 4, st));
+            if ((s = dalloc(cl, &p.hist, (size_t)HIST_IT * P * 4)) != TB_OK) return s;
+            TB_CK(cudaMemsetAsync(p.hist, 0, sizeof(double) * HIST_IT * P * 4, st));
         }
         TB_CK(cudaMemsetAsync(p.dbg, 0, 8 * sizeof(double), st));
     }
     if ((s = dalloc(cl, &p.col, P)) != TB_OK) return s;
-    if ((s = dalloc(cl, &p.inner, 2 * P)) != TB_OK) return s;
-    if ((s = dalloc(cl, &p.partials, (size_t)p.grid * 4 * P)) != TB_OK) return s;
+    if ((s = dalloc(cl, &p.inner, P)) != TB_OK) return s;
+    if ((s = dalloc(cl, &p.partials, (size_t)p.grid * 4 * p.C)) != TB_OK) return s;
     if ((s = dalloc(cl, &p.counter, 1 + MAX_GROUPS)) != TB_OK) return s;
-    if ((s = dalloc(cl, &p.partials2, (size_t)MAX_GROUPS * 4 * std::max(p.P, 1))) != TB_OK) return s;
+    if ((s = dalloc(cl, &p.partials2, (size_t)MAX_GROUPS * 4 * p.C)) != TB_OK) return s;
     if ((s = dalloc(cl, &p.flags, NFLAGS)) != TB_OK) return s;
     return TB_OK;
 }
@@ -774,7 +771,7 @@ bool step_graph_build(View& v, PanelDev& p, InnerCtx& ic, int proj, int inner_ma
         launch_finish(v.ds, p, cs);
         launch_shift_step(v.ds, p, cs);
         if (proj == PROJ_NONE) launch_full_update(v.ds, p, cs);
-        launch_outer_spmm(v.ds, p, true, cs);
+        launch_outer_spmm(v.ds, p, cs);
         launch_outer_update(v.ds, p, cs);
         int pred32 = ic.pred32, rounds = ic.rounds;
         int64_t steps = 0;
@@ -809,6 +806,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
         // takes narrower panels)
         while (P > 1 && (double)K * npad * P * 32.0 > (double)state_budget(o)) P >>= 1;
     }
+    P = std::max(P, 2);   // the vector kernels take columns in pairs; a single column has an inactive partner
     int M = 0;
     if (q.proj == PROJ_ROWS) {
         for (int c = 0; c < R; ++c) M = std::max<int64_t>(M, q.row_ptr[c + 1] - q.row_ptr[c]);
@@ -832,17 +830,16 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     p.mixed = o->precision == TB_MIXED ? 1 : 0;
     p.inner_lo_tol = o->inner_lo_tol;
     p.cheb_cpt = q.cheb_cpt;
-    const size_t nv = (size_t)npad * P;
+    const size_t nv = (size_t)npad * P;   // x^k, p^k: complex, one per column
     tb_status s;
     if ((s = alloc_inner_workspace(cl, p, st)) != TB_OK) return s;
     if ((s = dalloc(cl, &p.z, K)) != TB_OK) return s;
-    if ((s = dalloc(cl, &p.pi, (size_t)P * K)) != TB_OK) return s;
-    if ((s = dalloc(cl, &p.pi_prev, (size_t)P * K)) != TB_OK) return s;
+    if ((s = dalloc(cl, &p.zeta, (size_t)P * K)) != TB_OK) return s;
+    if ((s = dalloc(cl, &p.pinv, (size_t)P * K)) != TB_OK) return s;
     if ((s = dalloc(cl, &p.conv_iter, (size_t)P * K)) != TB_OK) return s;
     if (q.proj == PROJ_NONE) {
         if ((s = dalloc(cl, &p.ak, (size_t)P * K)) != TB_OK) return s;
         if ((s = dalloc(cl, &p.bk, (size_t)P * K)) != TB_OK) return s;
-        if ((s = dalloc(cl, &p.ipi, (size_t)P * K)) != TB_OK) return s;
         if ((s = dalloc(cl, &p.X, nv * K)) != TB_OK) return s;
         if ((s = dalloc(cl, &p.Pk, nv * K)) != TB_OK) return s;
     } else {
@@ -853,8 +850,8 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
             p.deriv = 1;
             if ((s = dalloc(cl, &p.dt, (size_t)P * K * M)) != TB_OK) return s;
             if ((s = dalloc(cl, &p.du, (size_t)P * K * M)) != TB_OK) return s;
-            if ((s = dalloc(cl, &p.dpi, (size_t)P * K)) != TB_OK) return s;
-            if ((s = dalloc(cl, &p.dpi_prev, (size_t)P * K)) != TB_OK) return s;
+            if ((s = dalloc(cl, &p.dzeta, (size_t)P * K)) != TB_OK) return s;
+            if ((s = dalloc(cl, &p.dpinv, (size_t)P * K)) != TB_OK) return s;
         }
     }
     double2* w_dev = nullptr;
@@ -885,11 +882,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
         for (int c = 0; c < P; ++c) {
             ColState cs;
             std::memset(&cs, 0, sizeof(cs));
-            cs.zs = make_double2(q.z[2 * o->seed], q.z[2 * o->seed + 1]);
-            cs.alpha_prev = make_double2(1.0, 0.0);
-            cs.beta_prev = make_double2(0.0, 0.0);
-            cs.sc_cur = make_double2(1.0, 0.0);
-            cs.sc_prev = make_double2(1.0, 0.0);
+            cs.sigma = q.z[2 * o->seed];
             cs.seed = o->seed;
             cs.active = c < ncols ? 1 : 0;
             cs.row = c < ncols && !q.rhs ? v.o2p_h[q.cols[c0 + c]] : -1;
@@ -905,10 +898,10 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
             }
         }
         TB_CK(cudaMemcpyAsync(p.col, colh.data(), sizeof(ColState) * P, cudaMemcpyHostToDevice, st));
-        TB_CK(cudaMemsetAsync(p.inner, 0, sizeof(InnerState) * 2 * P, st));
+        TB_CK(cudaMemsetAsync(p.inner, 0, sizeof(InnerState) * P, st));
         if (p.mixed) {
-            TB_CK(cudaMemsetAsync(p.inner32, 0, sizeof(InnerState) * 3 * 2 * P, st));
-            TB_CK(cudaMemsetAsync(p.acc32, 0, sizeof(double) * 8 * P, st));
+            TB_CK(cudaMemsetAsync(p.inner32, 0, sizeof(InnerState) * 3 * P, st));
+            TB_CK(cudaMemsetAsync(p.acc32, 0, sizeof(double) * 4 * P, st));
         }
         TB_CK(cudaMemsetAsync(p.flags, 0, sizeof(int) * NFLAGS, st));
         if (q.proj == PROJ_ROWS)
@@ -932,7 +925,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
         bool tail_pending = false;
         for (int n = 0; n < o->max_iter; ++n) {
             const bool use_graph = tail_pending && g_graphs && g_step_graphs && !g_trace && p.mixed &&
-                                   ic.cheb.n > 0 && ic.cheb.chebyshev(ic.rounds - 1) && ic.res_exact && !sg.failed;
+                                   ic.cheb.n > 0 && ic.cheb.chebyshev(ic.rounds - 1) && !sg.failed;
             if (use_graph && (!sg.exec || sg.rounds != ic.rounds))
                 step_graph_build(v, p, ic, q.proj, o->inner_max_iter, sg);
             if (use_graph && sg.exec) {
@@ -946,10 +939,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
                 // rounds while some real column is above inner_tol)
                 if (v.flags_host[0] & ERR_INNER) s = inner_redo(v, p, p.Rcur, o->inner_max_iter, ic, st);
                 else if (v.flags_host[4] > 0) s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st, ic.rounds);
-                else {
-                    ic.res_exact = true;
-                    s = TB_OK;
-                }
+                else s = TB_OK;
                 if (s != TB_OK) return s;
             } else {
                 if (tail_pending) {
@@ -957,7 +947,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
                     launch_shift_step(v.ds, p, st);
                     if (q.proj == PROJ_NONE) launch_full_update(v.ds, p, st);
                 }
-                launch_outer_spmm(v.ds, p, ic.res_exact, st);
+                launch_outer_spmm(v.ds, p, st);
                 launch_outer_update(v.ds, p, st);
                 s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st);
                 if (s != TB_OK) return s;
@@ -2655,7 +2645,7 @@ tb_status tb_generalized_lanczos_batch(tb_handle* h, int32_t R, const int32_t* c
     if ((s = check_cols(h, R, cols)) != TB_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int npad = h->ds.npad;
-    const int P = std::min(opts->panel ? opts->panel : 64, next_pow2(R));
+    const int P = std::max(2, std::min(opts->panel ? opts->panel : 64, next_pow2(R)));
     Cleanup cl_out;
     cl_out.st = st;
     OutBuf oa, ob, on;
@@ -2676,7 +2666,7 @@ tb_status tb_generalized_lanczos_batch(tb_handle* h, int32_t R, const int32_t* c
         p.mixed = opts->precision == TB_MIXED ? 1 : 0;
         p.inner_lo_tol = opts->inner_lo_tol;
         if ((s = alloc_inner_workspace(cl, p, st)) != TB_OK) return s;
-        const size_t nv = (size_t)npad * P;
+        const size_t nv = (size_t)npad * p.C;
         double2 *U, *Uprev, *Wv;
         if ((s = dalloc(cl, &U, nv)) != TB_OK) return s;
         if ((s = dalloc(cl, &Uprev, nv)) != TB_OK) return s;
@@ -2696,10 +2686,10 @@ tb_status tb_generalized_lanczos_batch(tb_handle* h, int32_t R, const int32_t* c
             colh[c].row = c < ncols ? h->orb2pad_h[cols[c0 + c]] : -1;
         }
         TB_CK(cudaMemcpyAsync(p.col, colh.data(), sizeof(ColState) * P, cudaMemcpyHostToDevice, st));
-        TB_CK(cudaMemsetAsync(p.inner, 0, 2 * P * sizeof(InnerState), st));
+        TB_CK(cudaMemsetAsync(p.inner, 0, P * sizeof(InnerState), st));
         if (p.mixed) {
-            TB_CK(cudaMemsetAsync(p.inner32, 0, sizeof(InnerState) * 3 * 2 * P, st));
-            TB_CK(cudaMemsetAsync(p.acc32, 0, sizeof(double) * 8 * P, st));
+            TB_CK(cudaMemsetAsync(p.inner32, 0, sizeof(InnerState) * 3 * P, st));
+            TB_CK(cudaMemsetAsync(p.acc32, 0, sizeof(double) * 4 * P, st));
         }
         TB_CK(cudaMemsetAsync(p.flags, 0, NFLAGS * sizeof(int), st));
         TB_CK(cudaMemsetAsync(p.counter, 0, sizeof(unsigned) * (1 + MAX_GROUPS), st));
@@ -2714,13 +2704,13 @@ tb_status tb_generalized_lanczos_batch(tb_handle* h, int32_t R, const int32_t* c
         if ((s = inner_solve(v, p, p.Rcur, opts->inner_max_iter, ic, st)) != TB_OK) return s;
         launch_lz_start(p, p.Rp, U, np_, st);
         for (int n = 0; n < n_steps; ++n) {
-            launch_lz_spmv(h->ds, h->ds.H, U, p.W, P, st);                        // H u^n
+            launch_lz_spmv(h->ds, h->ds.H, U, p.W, p.C, st);                      // H u^n
             launch_lz_dot(p, U, p.W, ap + n, n_steps, 0, st);                     // a_n = u^T H u
             TB_CK(cudaMemcpyAsync(p.Rin, p.W, sizeof(double2) * nv, cudaMemcpyDeviceToDevice, st));
             TB_CK(cudaMemcpyAsync(p.Rcur, p.W, sizeof(double2) * nv, cudaMemcpyDeviceToDevice, st));
             if ((s = inner_solve(v, p, p.Rcur, opts->inner_max_iter, ic, st)) != TB_OK) return s;  // S^-1 H u^n
             launch_lz_combine(p, p.Rp, U, Uprev, Wv, ap + n, bp + n, n_steps, n_steps + 1, st);
-            launch_lz_spmv(h->ds, h->ds.S, Wv, p.W, P, st);                      // S w
+            launch_lz_spmv(h->ds, h->ds.S, Wv, p.W, p.C, st);                    // S w
             launch_lz_dot(p, Wv, p.W, bp + n + 1, n_steps + 1, 1, st);            // b_{n+1} = ||w||_S
             launch_lz_scale(p, Wv, U, Uprev, bp + n + 1, n_steps + 1, st);
             TB_CK(cudaGetLastError());
@@ -2776,7 +2766,8 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int npad = h->ds.npad;
     PanelDev p;
-    p.P = 1;
+    p.P = 2;   // the column and an inactive partner
+    p.C = 1;
     p.K = 1;
     p.npad = npad;
     p.grid = max_grid();
@@ -2784,15 +2775,15 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     // size check before any device work: everything must fit in the fixed array
     ScratchCarver dry(nullptr, TB_NOALLOC_SCRATCH_BYTES);
     for (int v = 0; v < 10; ++v) dry.take<double2>(npad);
-    dry.take<ColState>(1);
+    dry.take<ColState>(2);
     dry.take<InnerState>(2);
     dry.take<double>((size_t)p.grid * 4);
     dry.take<double>((size_t)MAX_GROUPS * 4);
     dry.take<unsigned>(1 + MAX_GROUPS);
     dry.take<int>(NFLAGS);
-    dry.take<double>(n_steps);
-    dry.take<double>((size_t)n_steps + 1);
-    dry.take<double>(1);
+    dry.take<double>((size_t)2 * n_steps);
+    dry.take<double>((size_t)2 * (n_steps + 1));
+    dry.take<double>(2);
     if (!dry.ok) return TB_ERR_TOO_LARGE;
     // the handle's device must be current: the scratch address and the
     // kernels were placed there by tb_create
@@ -2809,29 +2800,30 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     double2* U = sc.take<double2>(npad);
     double2* Uprev = sc.take<double2>(npad);
     double2* Wv = sc.take<double2>(npad);
-    p.col = sc.take<ColState>(1);
+    p.col = sc.take<ColState>(2);
     p.inner = sc.take<InnerState>(2);
     p.partials = sc.take<double>((size_t)p.grid * 4);
     p.partials2 = sc.take<double>((size_t)MAX_GROUPS * 4);
     p.counter = sc.take<unsigned>(1 + MAX_GROUPS);
     p.flags = sc.take<int>(NFLAGS);
-    double* ad = sc.take<double>(n_steps);
-    double* bd = sc.take<double>((size_t)n_steps + 1);
-    double* nd = sc.take<double>(1);
+    double* ad = sc.take<double>((size_t)2 * n_steps);          // [column][n_steps]
+    double* bd = sc.take<double>((size_t)2 * (n_steps + 1));
+    double* nd = sc.take<double>(2);
     if (!sc.ok) return TB_ERR_TOO_LARGE;
     // the array keeps the previous call's contents: clear everything that
     // the step loop reads before writing
-    ColState cs;
-    std::memset(&cs, 0, sizeof(cs));
-    cs.active = 1;
-    cs.row = h->orb2pad_h[j];
-    TB_CK(cudaMemcpyAsync(p.col, &cs, sizeof(cs), cudaMemcpyHostToDevice, st));
+    ColState cs[2];
+    std::memset(cs, 0, sizeof(cs));
+    cs[0].active = 1;
+    cs[0].row = h->orb2pad_h[j];
+    cs[1].row = -1;
+    TB_CK(cudaMemcpyAsync(p.col, cs, sizeof(cs), cudaMemcpyHostToDevice, st));
     TB_CK(cudaMemsetAsync(p.inner, 0, 2 * sizeof(InnerState), st));
     TB_CK(cudaMemsetAsync(p.flags, 0, NFLAGS * sizeof(int), st));
     TB_CK(cudaMemsetAsync(p.counter, 0, sizeof(unsigned) * (1 + MAX_GROUPS), st));
     TB_CK(cudaMemsetAsync(Uprev, 0, sizeof(double2) * npad, st));
-    TB_CK(cudaMemsetAsync(ad, 0, sizeof(double) * n_steps, st));
-    TB_CK(cudaMemsetAsync(bd, 0, sizeof(double) * (n_steps + 1), st));
+    TB_CK(cudaMemsetAsync(ad, 0, sizeof(double) * 2 * n_steps, st));
+    TB_CK(cudaMemsetAsync(bd, 0, sizeof(double) * 2 * (n_steps + 1), st));
     int pred = 64;
     int64_t inner_total = 0;
     const int inner_max = 1000;
@@ -2841,13 +2833,13 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     launch_lz_start(p, p.Rp, U, nd, st);
     for (int n = 0; n < n_steps; ++n) {
         launch_lz_spmv(h->ds, h->ds.H, U, p.W, 1, st);
-        launch_lz_dot(p, U, p.W, ad + n, 1, 0, st);
+        launch_lz_dot(p, U, p.W, ad + n, n_steps, 0, st);
         TB_CK(cudaMemcpyAsync(p.Rin, p.W, sizeof(double2) * npad, cudaMemcpyDeviceToDevice, st));
         if ((s = inner_cg(hv, p, inner_max, pred, inner_total, st)) != TB_OK) return s;
-        launch_lz_combine(p, p.Rp, U, Uprev, Wv, ad + n, bd + n, 1, 1, st);
+        launch_lz_combine(p, p.Rp, U, Uprev, Wv, ad + n, bd + n, n_steps, n_steps + 1, st);
         launch_lz_spmv(h->ds, h->ds.S, Wv, p.W, 1, st);
-        launch_lz_dot(p, Wv, p.W, bd + n + 1, 1, 1, st);
-        launch_lz_scale(p, Wv, U, Uprev, bd + n + 1, 1, st);
+        launch_lz_dot(p, Wv, p.W, bd + n + 1, n_steps + 1, 1, st);
+        launch_lz_scale(p, Wv, U, Uprev, bd + n + 1, n_steps + 1, st);
         TB_CK(cudaGetLastError());
     }
     if (h->flags_host[0] & ERR_NOT_SPD) return TB_ERR_S_NOT_SPD;

@@ -77,17 +77,20 @@ struct DevSystem {
 };
 size_t inner32_grp_smem(const DevSystem& s);   // dynamic shared memory of the grouped SpMV
 
-// Per right-hand side (complex column) state of a panel.
+// Per right-hand side (column) state of a panel.  The Krylov vectors are real
+// (see k_outer_spmm), so every scalar of the recurrence but the seed shift's
+// pivot is real.
 struct ColState {
-    double2 zs;          // seed shift z_s
-    double2 alpha;       // alpha_n of the current step
-    double2 alpha_prev;  // alpha_{n-1}
-    double2 beta_prev;   // beta_{n-1}
-    double2 rho;         // rho_n = r_n^T r'_n
-    double2 rho_new;     // rho_{n+1}
-    double2 sc_cur;      // pending scale of r_n and r'_n (seed switch)
-    double2 sc_prev;     // pending scale of r_{n-1}
-    double rnorm;        // ||r_{n+1}||_2
+    double sigma;        // real part of the seed shift: W = (H - sigma S) u'
+    double asig;         // a_n - sigma of the current step
+    double g, f, s;      // u_{n+1} = g (W - asig u_n) - f u_{n-1}; s: the step's scale (nu_{n+1} = B_{n+1} / s)
+    double t;            // t_n = u_n^T u'_n
+    double t_new;        // t_{n+1}
+    double nu, nu_prev;  // sqrt(t_n), sqrt(t_{n-1})
+    double inv_nu;       // 1 / nu of the latest vector (0 when it vanishes)
+    double B;            // B_n, the off-diagonal of T between steps n-1 and n
+    double rnorm;        // ||u_{n+1}||_2
+    double2 sinv;        // 1 / D_{n-1} of the seed shift
     int32_t seed;        // index of the seed shift
     int32_t active;      // 1 while some shift of the column is unconverged
     int32_t iters;       // outer steps run
@@ -98,7 +101,7 @@ struct ColState {
     int32_t pad_;
 };
 
-// Per real column (two per complex column) state of the inner CG.
+// Per column state of the inner solve (CG, refinement).
 struct InnerState {
     double gamma_prev;
     double alpha;
@@ -112,40 +115,43 @@ struct InnerState {
 };
 
 struct PanelDev {
-    int P = 0, K = 0, npad = 0, M = 0, proj = PROJ_NONE;
+    int P = 0;                    // columns (right-hand sides), even
+    int C = 0;                    // pairs of columns, P / 2: the unit of the vector kernels
+    int K = 0, npad = 0, M = 0, proj = PROJ_NONE;
     int grid = 0;                 // CTAs of the grid-stride kernels
     int mixed = 0;                // 1: inner S^-1 by FP32 corrections inside FP64 refinement
-    int cheb_cpt = 0;             // host side: columns per thread of the Chebyshev step (2 or 4; 0 = default)
+    int cheb_cpt = 0;             // host side: pairs of columns per thread of the Chebyshev step (2 or 4; 0 = default)
     double tol = 1e-10, inner_tol = 1e-13, inner_lo_tol = 1e-6;
     int switching = 1, force_switch_every = 0;
-    // panel vectors, [npad][P] complex
+    // panel vectors, [npad][C] pairs of columns: u_n, u_{n-1}, u'_n, W (and the
+    // inner CG's w), the inner solve's right-hand side and residual, its p and s
     double2 *Rcur = nullptr, *Rprev = nullptr, *Rp = nullptr, *W = nullptr;
     double2 *Rin = nullptr, *Pin = nullptr, *Sin = nullptr;
-    float4* RpS = nullptr;        // mixed: r' split (re_hi, re_lo, im_hi, im_lo) for double-float SpMVs
-    // FP32 inner CG of the mixed-precision solve, [npad][P] complex floats
+    float4* RpS = nullptr;        // mixed: u' split (hi, hi', lo, lo' of the pair) for double-float SpMVs
+    // FP32 vectors of the mixed-precision inner solve, [npad][C] pairs
     float2 *r32 = nullptr, *p32 = nullptr, *s32 = nullptr, *w32 = nullptr, *x32 = nullptr;
-    InnerState* inner32 = nullptr; // [3][2P]: refinement state, CG state slots 0 and 1
-    double* acc32 = nullptr;       // [2][4][P]: FP32 CG sums (gamma, delta per real column), two slots
-    double* cgs = nullptr;         // [2][2P]: alpha, beta of the current FP32 CG iteration
-    unsigned char* cgu = nullptr;  // [2P]: real column updated in the current FP32 CG iteration
+    InnerState* inner32 = nullptr; // [3][P]: refinement state, CG state slots 0 and 1
+    double* acc32 = nullptr;       // [2][4][C]: FP32 CG sums (gamma, delta per column), two slots
+    double* cgs = nullptr;         // [2][P]: alpha, beta of the current FP32 CG iteration
+    unsigned char* cgu = nullptr;  // [P]: column updated in the current FP32 CG iteration
     unsigned* ticket32 = nullptr;  // [1]: completion ticket of the FP32 SpMV (0 between launches)
     ColState* col = nullptr;       // [P]
-    InnerState* inner = nullptr;   // [2P]
+    InnerState* inner = nullptr;   // [P]
     double2* z = nullptr;          // [K]
-    double2 *pi = nullptr, *pi_prev = nullptr;   // [P][K]
+    double2 *zeta = nullptr, *pinv = nullptr;    // [P][K] zeta^k_n and 1 / D^k_{n-1} (see shift_coef)
     int32_t* conv_iter = nullptr;                // [P][K]
-    double2 *ak = nullptr, *bk = nullptr, *ipi = nullptr;  // [P][K] this step (full mode)
+    double2 *ak = nullptr, *bk = nullptr;        // [P][K] alpha^k, l^k of this step (full mode; alpha 0: no update)
     int32_t* frow = nullptr;       // [P][M] padded rows (PROJ_ROWS)
     double2 *t = nullptr, *u = nullptr;          // [P][K][M] projected x, p
     int deriv = 0;                               // 1: also d/dz_k of the projections (PROJ_ROWS)
-    double2 *dpi = nullptr, *dpi_prev = nullptr; // [P][K] d pi^k / d z_k
+    double2 *dzeta = nullptr, *dpinv = nullptr;  // [P][K] d/dz_k of zeta and pinv
     double2 *dt = nullptr, *du = nullptr;        // [P][K][M] d/dz_k of t, u
     double2 *X = nullptr, *Pk = nullptr;         // [K][npad][P] full mode x, p
-    double* partials = nullptr;    // [grid][4][P] per-CTA sums
-    double* partials2 = nullptr;   // [MAX_GROUPS][4][P] per-group sums
+    double* partials = nullptr;    // [grid][4][C] per-CTA sums
+    double* partials2 = nullptr;   // [MAX_GROUPS][4][C] per-group sums
     unsigned* counter = nullptr;   // [1 + MAX_GROUPS] arrival tickets of the grid reductions
     double* dbg = nullptr;         // [8] record of the first inner-CG breakdown (diagnostics)
-    double* hist = nullptr;        // trace only: [HIST_IT][2P][4] gamma, delta, alpha, beta per FP32 CG iteration
+    double* hist = nullptr;        // trace only: [HIST_IT][P][4] gamma, delta, alpha, beta per FP32 CG iteration
     int* flags = nullptr;          // [NFLAGS]: 0 errors, 1 inner active, 2 active columns,
                                    // 3 inner iterations used, 4 refinement: unconverged real columns,
                                    // 5 FP32 CG rounds stopped early by a rounding breakdown,
@@ -188,8 +194,7 @@ void launch_panel_rhs(const PanelDev& p, const double* rhs, const int32_t* orb2p
 void launch_vjp_accumulate(const double2* X, const double2* Y, int K, int Rc, int64_t N, const int32_t* cpos,
                            const double* vc, const int32_t* ea, const int32_t* eb, int64_t ne,
                            const double2* z, const double2* w, double g_s, double* gH, double* gS, cudaStream_t st);
-// sx_from_residual (mixed path): Rin holds r_n - S r'_n from the refinement
-void launch_outer_spmm(const DevSystem& s, const PanelDev& p, bool sx_from_residual, cudaStream_t st);
+void launch_outer_spmm(const DevSystem& s, const PanelDev& p, cudaStream_t st);   // Rin: u_n - S u'_n of the inner solve
 void launch_outer_update(const DevSystem& s, const PanelDev& p, cudaStream_t st);
 void launch_inner_spmv(const DevSystem& s, const PanelDev& p, int it, cudaStream_t st);
 void launch_inner_update(const DevSystem& s, const PanelDev& p, int it, cudaStream_t st);
@@ -256,7 +261,7 @@ void launch_lanczos_green(const double* a, const double* b, const double* norm, 
                           const double2* z, double2* G, cudaStream_t st);
 
 // generalized Lanczos on a panel of P independent columns (Section 3.2)
-void launch_lz_spmv(const DevSystem& s, const double* M, const double2* x, double2* y, int P, cudaStream_t st);
+void launch_lz_spmv(const DevSystem& s, const double* M, const double2* x, double2* y, int C, cudaStream_t st);
 void launch_lz_dot(const PanelDev& p, const double2* x, const double2* y, double* out, int stride, int mode,
                    cudaStream_t st);
 void launch_lz_combine(const PanelDev& p, const double2* y, double2* u, double2* u_prev, double2* w,

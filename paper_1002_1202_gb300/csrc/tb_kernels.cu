@@ -3,10 +3,13 @@
 // Data layout (device, HBM):
 //   * S and H: block-sparse rows over atoms, every block padded to 4x4
 //     (row-major doubles), block row I covering padded orbitals 4I..4I+3;
-//   * panel vectors: [npad][P] complex doubles (double2), the P right-hand
-//     sides of a panel interleaved per orbital row, so one atom's 4 rows of a
-//     panel are 4*P*16 contiguous bytes and a CTA's loads are coalesced along
-//     the column index.
+//   * panel vectors: [npad][P] doubles, the P right-hand sides of a panel
+//     interleaved per orbital row.  H, S and every right-hand side are real, so
+//     the Krylov vectors are real whatever the shifts (the complex residual of
+//     each shift is a complex number times the same real vector); the kernels
+//     take the columns in pairs, one double2 of columns 2c and 2c + 1 per
+//     orbital row (C = P / 2 pairs), so one atom's 4 rows of a panel are
+//     4*C*16 contiguous bytes and a CTA's loads are coalesced along the pairs.
 //
 // Reductions are deterministic: each CTA writes per-column partial sums, the
 // last CTA to arrive (atomic ticket) adds the partials in CTA order and
@@ -223,25 +226,37 @@ __global__ void k_compact_blocks(int n_atoms, const int* __restrict__ brow, cons
 }
 
 __global__ void k_panel_init(PanelDev p) {
-    const long long items = (long long)p.npad * p.P;
+    const int C = p.C;
+    const long long items = (long long)p.npad * C;
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
-        const int c = (int)(idx % p.P), i = (int)(idx / p.P);
-        const double2 v = cmk(i == p.col[c].row ? 1.0 : 0.0, 0.0);
+        const int c = (int)(idx % C), i = (int)(idx / C);
+        const double2 v = make_double2(i == p.col[2 * c].row ? 1.0 : 0.0, i == p.col[2 * c + 1].row ? 1.0 : 0.0);
         p.Rcur[idx] = v;
         p.Rin[idx] = v;
-        p.Rprev[idx] = cmk(0.0, 0.0);
+        p.Rprev[idx] = make_double2(0.0, 0.0);
     }
 }
 
+// a pair works while one of its two columns is active
+__device__ __forceinline__ bool pair_active(const PanelDev& p, int c) {
+    return p.col[2 * c].active != 0 || p.col[2 * c + 1].active != 0;
+}
+
 // ---------------------------------------------------------------------------
-// a1 + a2: q = A(z_s) r'_n = z_s S r'_n - H r'_n in one pass over the blocks,
-// A p_n = q + (beta_{n-1}/alpha_{n-1}) (r_{n-1} - r_n), mu = r'_n^T A p_n,
-// alpha_n = rho_n / mu (Eqs. CGp:p, CGp:r and the alpha_n of Section 3.3).
-// Pending seed-switch scales of r_n, r'_n, r_{n-1} are applied on the fly.
-// SX (mixed path): S r'_n is taken as r_n - res, res = r_n - S r'_n being
-// the refinement's last double-float residual (in Rin), so only H r'_n is
-// formed here -- half the double-float products.
+// a1 + a2 in real arithmetic.  With real H, S and b the residuals of every
+// shift are complex multiples of one real sequence u_n (Eq. collinear; the
+// seed residual r_n too), the Lanczos vectors of S^-1 H (Eqs. 1.13, 1.18)
+// in the residual space:
+//     nu_n B_{n+1} u^_{n+1} = H u'_n - a_n u_n - (nu_n B_n / nu_{n-1}) u_{n-1},
+//     u'_n = S^-1 u_n,  nu_n^2 = t_n = u_n^T u'_n,  a_n = u'_n^T H u'_n / t_n,
+// u^_n = u_n / nu_n.  One real vector per right-hand side carries all shifts,
+// where the complex seed system (Eqs. CGp:p, CGp:x, CGp:r) needs two: half
+// the products with S and H and half the vector traffic for the same
+// iterates.  The product is formed with the real part sigma of the seed
+// shift, W = H u' - sigma S u', S u' = u - res with res = u - S u' the inner
+// solve's residual (in Rin), so that an inexact u' enters as in the seed
+// system.  asig = a_n - sigma.
 // ---------------------------------------------------------------------------
 // One block row of a double-float SpMV (M = Mh + Ml, FP32 hi / lo blocks,
 // times the split r') with exact orbital counts (systems with s-only atoms):
@@ -280,55 +295,63 @@ __device__ __forceinline__ void df_row_ragged(const DevSystem& s, const float* _
     }
 }
 
-template <bool DF, bool SX = false, bool RAG = false>
+// Scalars of outer step n of one column from m = u'_n^T W (one thread):
+// asig = m / t_n, and the factors of the update
+//     u_{n+1} = g (W - asig u_n) - f u_{n-1},  g = 1 / (nu_n s), f = B_n / (nu_{n-1} s),
+// scaled by s = B_n (1 at the first step), so that nu_{n+1} = B_{n+1} / s stays
+// near one however the residuals shrink.  False (and the column is
+// deactivated) when t_n is not positive and finite, or when the seed shift
+// z_s makes the pivot of its own recurrence vanish (a real shift on a level):
+// D_n = z_s - a_n - B_n^2 / D_{n-1}.
+__device__ __forceinline__ bool lanczos_step_scalars(ColState& cs, double m, double2 zs) {
+    const double asig = m / cs.t;
+    double2 D = make_double2((zs.x - cs.sigma) - asig, zs.y);
+    if (cs.iters > 0) {
+        D.x -= cs.B * cs.B * cs.sinv.x;
+        D.y -= cs.B * cs.B * cs.sinv.y;
+    }
+    if (!(cs.t > 0.0) || !isfinite(m) || !isfinite(cs.t) || (D.x == 0.0 && D.y == 0.0)) {
+        cs.active = 0;
+        return false;
+    }
+    const double s = cs.iters > 0 ? cs.B : 1.0;
+    cs.asig = asig;
+    cs.s = s;
+    cs.g = 1.0 / (cs.nu * s);
+    cs.f = cs.iters > 0 ? cs.B / (cs.nu_prev * s) : 0.0;
+    return true;
+}
+
+template <bool DF, bool RAG = false>
 __global__ void __launch_bounds__(THREADS) k_outer_spmm(DevSystem s, PanelDev p) {
     __shared__ double smem[2 * THREADS];
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    const ColState cs = p.col[c];
-    const bool act = cs.active != 0;
-    const double2 sc = cs.sc_cur, scp = cs.sc_prev;
-    const double2 coef = act ? cdiv(cs.beta_prev, cs.alpha_prev) : cmk(0.0, 0.0);
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    const double sg0 = p.col[2 * c].sigma, sg1 = p.col[2 * c + 1].sigma;
     double mu[2] = {0.0, 0.0};
-    const long long items = (long long)s.n_atoms * P;
-    if (act) {
+    const long long items = (long long)s.n_atoms * C;
+    if (pair_active(p, c)) {
         for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
              idx += (long long)gridDim.x * THREADS) {
-            const int I = (int)(idx / P);
-            double2 aS[4], aH[4];
+            const int I = (int)(idx / C);
+            double2 aH[4];
             if (DF) {
-                // double-float products: S_hi/S_lo, H_hi/H_lo times the split r',
-                // the real and imaginary parts in the two lanes of packed FP32 ops
-                float2 sh[4], sl[4], hh[4], hl[4];
+                // double-float products: H_hi/H_lo times the split u', the two
+                // columns of the pair in the two lanes of packed FP32 ops
+                float2 hh[4], hl[4];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    sh[a] = sl[a] = hh[a] = hl[a] = make_float2(0.f, 0.f);
-                }
-                if (RAG) {
-                    const int ni = s.norb[I];
-                    df_row_ragged(s, s.H32hi, s.H32lo, I, ni, p.RpS, P, c, hh, hl);
-                    if (!SX) df_row_ragged(s, s.S32, s.S32lo, I, ni, p.RpS, P, c, sh, sl);
-                }
+                for (int a = 0; a < 4; ++a) hh[a] = hl[a] = make_float2(0.f, 0.f);
+                if (RAG) df_row_ragged(s, s.H32hi, s.H32lo, I, s.norb[I], p.RpS, C, c, hh, hl);
                 for (int b = RAG ? s.brow[I + 1] : s.brow[I]; b < s.brow[I + 1]; ++b) {
                     const int J = s.bcol[b];
-                    const float4* xr = p.RpS + (size_t)4 * J * P + c;
-                    const float4 x[4] = {xr[0], xr[P], xr[2 * P], xr[3 * P]};
-                    const float4* Sh = reinterpret_cast<const float4*>(s.S32 + 16 * (size_t)b);
-                    const float4* Sl = reinterpret_cast<const float4*>(s.S32lo + 16 * (size_t)b);
+                    const float4* xr = p.RpS + (size_t)4 * J * C + c;
+                    const float4 x[4] = {xr[0], xr[C], xr[2 * C], xr[3 * C]};
                     const float4* Hh = reinterpret_cast<const float4*>(s.H32hi + 16 * (size_t)b);
                     const float4* Hl = reinterpret_cast<const float4*>(s.H32lo + 16 * (size_t)b);
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
                         const float4 h4h = __ldg(Hh + a), h4l = __ldg(Hl + a);
                         const float hvh[4] = {h4h.x, h4h.y, h4h.z, h4h.w}, hvl[4] = {h4l.x, h4l.y, h4l.z, h4l.w};
-                        if (!SX) {
-                            const float4 s4h = __ldg(Sh + a), s4l = __ldg(Sl + a);
-                            const float svh[4] = {s4h.x, s4h.y, s4h.z, s4h.w}, svl[4] = {s4l.x, s4l.y, s4l.z, s4l.w};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                df_mac2(sh[a], sl[a], svh[e], svl[e], make_float2(x[e].x, x[e].y),
-                                        make_float2(x[e].z, x[e].w));
-                        }
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
                             df_mac2(hh[a], hl[a], hvh[e], hvl[e], make_float2(x[e].x, x[e].y),
@@ -336,30 +359,19 @@ __global__ void __launch_bounds__(THREADS) k_outer_spmm(DevSystem s, PanelDev p)
                     }
                 }
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    if (SX) {
-                        const size_t e = (size_t)(4 * I + a) * P + c;
-                        aS[a] = csub(p.Rcur[e], p.Rin[e]);
-                    } else {
-                        aS[a] = cmk((double)sh[a].x + (double)sl[a].x, (double)sh[a].y + (double)sl[a].y);
-                    }
-                    aH[a] = cmk((double)hh[a].x + (double)hl[a].x, (double)hh[a].y + (double)hl[a].y);
-                }
+                for (int a = 0; a < 4; ++a)
+                    aH[a] = make_double2((double)hh[a].x + (double)hl[a].x, (double)hh[a].y + (double)hl[a].y);
             } else {
 #pragma unroll
-                for (int a = 0; a < 4; ++a) { aS[a] = cmk(0.0, 0.0); aH[a] = cmk(0.0, 0.0); }
+                for (int a = 0; a < 4; ++a) aH[a] = make_double2(0.0, 0.0);
                 for (int b = s.brow[I]; b < s.brow[I + 1]; ++b) {
                     const int J = s.bcol[b];
-                    const double2* xr = p.Rp + (size_t)4 * J * P + c;
-                    const double2 x0 = xr[0], x1 = xr[P], x2 = xr[2 * P], x3 = xr[3 * P];
-                    const double2* Sb = reinterpret_cast<const double2*>(s.S + 16 * (size_t)b);
+                    const double2* xr = p.Rp + (size_t)4 * J * C + c;
+                    const double2 x0 = xr[0], x1 = xr[C], x2 = xr[2 * C], x3 = xr[3 * C];
                     const double2* Hb = reinterpret_cast<const double2*>(s.H + 16 * (size_t)b);
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
-                        const double2 s01 = __ldg(Sb + 2 * a), s23 = __ldg(Sb + 2 * a + 1);
                         const double2 h01 = __ldg(Hb + 2 * a), h23 = __ldg(Hb + 2 * a + 1);
-                        aS[a].x += s01.x * x0.x + s01.y * x1.x + s23.x * x2.x + s23.y * x3.x;
-                        aS[a].y += s01.x * x0.y + s01.y * x1.y + s23.x * x2.y + s23.y * x3.y;
                         aH[a].x += h01.x * x0.x + h01.y * x1.x + h23.x * x2.x + h23.y * x3.x;
                         aH[a].y += h01.x * x0.y + h01.y * x1.y + h23.x * x2.y + h23.y * x3.y;
                     }
@@ -367,55 +379,52 @@ __global__ void __launch_bounds__(THREADS) k_outer_spmm(DevSystem s, PanelDev p)
             }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                const size_t e = (size_t)(4 * I + a) * P + c;
-                const double2 q = cmul(sc, csub(cmul(cs.zs, aS[a]), aH[a]));
-                const double2 rc = cmul(sc, p.Rcur[e]);
-                const double2 rpv = cmul(scp, p.Rprev[e]);
-                const double2 Ap = cadd(q, cmul(coef, csub(rpv, rc)));
-                p.W[e] = Ap;
-                const double2 m = cmul(cmul(sc, p.Rp[e]), Ap);
-                mu[0] += m.x;
-                mu[1] += m.y;
+                const size_t e = (size_t)(4 * I + a) * C + c;
+                const double2 u = p.Rcur[e], res = p.Rin[e], x = p.Rp[e];
+                const double2 w = make_double2(aH[a].x - sg0 * (u.x - res.x), aH[a].y - sg1 * (u.y - res.y));
+                p.W[e] = w;
+                mu[0] += x.x * w.x;
+                mu[1] += x.y * w.y;
             }
         }
     }
-    if (grid_reduce_cols<2>(mu, P, p, smem)) {
-        const int t = threadIdx.x;
-        if (t < P && p.col[t].active) {
-            const double2 m = cmk(smem[t], smem[THREADS + t]);
-            const double2 rho = p.col[t].rho;
-            if ((m.x == 0.0 && m.y == 0.0) || (rho.x == 0.0 && rho.y == 0.0) || !isfinite(m.x) ||
-                !isfinite(m.y)) {
-                atomicOr(&p.flags[0], ERR_BREAKDOWN);
-                p.col[t].active = 0;
-            } else {
-                p.col[t].alpha = cdiv(rho, m);
-            }
+    if (grid_reduce_cols<2>(mu, C, p, smem)) {
+        for (int t = threadIdx.x; t < p.P; t += THREADS) {
+            ColState& cs = p.col[t];
+            if (!cs.active) continue;
+            const double m = smem[(t & 1) * THREADS + (t >> 1)];
+            if (!lanczos_step_scalars(cs, m, p.z[cs.seed])) atomicOr(&p.flags[0], ERR_BREAKDOWN);
         }
     }
 }
 
-// r_{n+1} = r_n - alpha_n A p_n; r_n becomes r_{n-1}; the inner CG starts
-// from b = r_{n+1}.
+// u_{n+1} = g_n (W - asig u_n) - f_n u_{n-1}; u_n becomes u_{n-1}; the FP64
+// inner CG starts from b = u_{n+1} in Rin (the refinement of the mixed path
+// takes it from Rcur).  An inactive column keeps its vectors.
 __global__ void k_outer_update(PanelDev p) {
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    const ColState cs = p.col[c];
-    if (!cs.active) return;
-    const long long items = (long long)p.npad * P;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    if (!pair_active(p, c)) return;
+    const ColState& c0 = p.col[2 * c];
+    const ColState& c1 = p.col[2 * c + 1];
+    const bool a0 = c0.active != 0, a1 = c1.active != 0;
+    const double as0 = c0.asig, as1 = c1.asig, g0 = c0.g, g1 = c1.g, f0 = c0.f, f1 = c1.f;
+    const long long items = (long long)p.npad * C;
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
-        const double2 rc = cmul(cs.sc_cur, p.Rcur[idx]);
-        const double2 rn = csub(rc, cmul(cs.alpha, p.W[idx]));
-        p.Rprev[idx] = rc;
-        p.Rcur[idx] = rn;
-        p.Rin[idx] = rn;
+        const double2 u = p.Rcur[idx], up = p.Rprev[idx], w = p.W[idx];
+        double2 un = u, um = up;
+        if (a0) { un.x = g0 * (w.x - as0 * u.x) - f0 * up.x; um.x = u.x; }
+        if (a1) { un.y = g1 * (w.y - as1 * u.y) - f1 * up.y; um.y = u.y; }
+        p.Rprev[idx] = um;
+        p.Rcur[idx] = un;
+        if (!p.mixed) p.Rin[idx] = un;
     }
 }
 
 // ---------------------------------------------------------------------------
-// a3 + a4: inner CG for S r' = r (Section 3.3), both real parts of every
-// complex column, Chronopoulos-Gear form (one reduction per iteration):
+// a3 + a4: inner CG for S u' = u (Section 3.3), both columns of every
+// pair, Chronopoulos-Gear form (one reduction per iteration):
 //   w_i = S r_i, gamma_i = r_i.r_i, delta_i = w_i.r_i,
 //   beta_i = gamma_i/gamma_{i-1}, alpha_i = gamma_i/(delta_i - beta_i gamma_i/alpha_{i-1}),
 //   p_i = r_i + beta_i p_{i-1}, s_i = w_i + beta_i s_{i-1},
@@ -424,23 +433,23 @@ __global__ void k_outer_update(PanelDev p) {
 __global__ void __launch_bounds__(THREADS) k_inner_spmv(DevSystem s, PanelDev p, int it) {
     __shared__ double smem[4 * THREADS];
     if (it > 0 && *(volatile int*)&p.flags[1] == 0) return;
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    const bool act = p.col[c].active != 0;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    const bool act = pair_active(p, c);
     const bool live = act && !(p.inner[2 * c].conv && p.inner[2 * c + 1].conv && it > 0);
     double v[4] = {0.0, 0.0, 0.0, 0.0};   // gamma_re, gamma_im, delta_re, delta_im
-    const long long items = (long long)s.n_atoms * P;
+    const long long items = (long long)s.n_atoms * C;
     if (live) {
         for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
              idx += (long long)gridDim.x * THREADS) {
-            const int I = (int)(idx / P);
+            const int I = (int)(idx / C);
             double2 acc[4];
 #pragma unroll
             for (int a = 0; a < 4; ++a) acc[a] = cmk(0.0, 0.0);
             for (int b = s.brow[I]; b < s.brow[I + 1]; ++b) {
                 const int J = s.bcol[b];
-                const double2* xr = p.Rin + (size_t)4 * J * P + c;
-                const double2 x0 = xr[0], x1 = xr[P], x2 = xr[2 * P], x3 = xr[3 * P];
+                const double2* xr = p.Rin + (size_t)4 * J * C + c;
+                const double2 x0 = xr[0], x1 = xr[C], x2 = xr[2 * C], x3 = xr[3 * C];
                 const double2* Sb = reinterpret_cast<const double2*>(s.S + 16 * (size_t)b);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
@@ -451,7 +460,7 @@ __global__ void __launch_bounds__(THREADS) k_inner_spmv(DevSystem s, PanelDev p,
             }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                const size_t e = (size_t)(4 * I + a) * P + c;
+                const size_t e = (size_t)(4 * I + a) * C + c;
                 const double2 r = p.Rin[e];
                 p.W[e] = acc[a];
                 v[0] += r.x * r.x;
@@ -461,13 +470,13 @@ __global__ void __launch_bounds__(THREADS) k_inner_spmv(DevSystem s, PanelDev p,
             }
         }
     }
-    if (grid_reduce_cols<4>(v, P, p, smem)) {
+    if (grid_reduce_cols<4>(v, C, p, smem)) {
         const int t = threadIdx.x;
         int nact = 0;
-        if (t < P) {
-            const bool cact = p.col[t].active != 0;
-            if (it == 0 && cact) p.col[t].rnorm = sqrt(smem[t] + smem[THREADS + t]);
+        if (t < C) {
             for (int part = 0; part < 2; ++part) {
+                const bool cact = p.col[2 * t + part].active != 0;
+                if (it == 0 && cact) p.col[2 * t + part].rnorm = sqrt(smem[part * THREADS + t]);
                 InnerState st = p.inner[2 * t + part];
                 const double gam = smem[part * THREADS + t];
                 const double del = smem[(2 + part) * THREADS + t];
@@ -510,12 +519,12 @@ __global__ void __launch_bounds__(THREADS) k_inner_spmv(DevSystem s, PanelDev p,
 
 __global__ void k_inner_update(PanelDev p, int it) {
     if (it > 0 && *(volatile int*)&p.flags[1] == 0) return;
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    if (!p.col[c].active) return;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    if (!pair_active(p, c)) return;
     const InnerState s0 = p.inner[2 * c], s1 = p.inner[2 * c + 1];
     if (s0.conv && s1.conv && it > 0) return;
-    const long long items = (long long)p.npad * P;
+    const long long items = (long long)p.npad * C;
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
         const double2 r = p.Rin[idx], w = p.W[idx];
@@ -567,11 +576,11 @@ __device__ void refine_finish_counts(PanelDev& p, int nact) {
 // round 0: ||b||, x = 0
 __global__ void __launch_bounds__(THREADS) k_refine_start(PanelDev p, const double2* __restrict__ b) {
     __shared__ double smem[2 * THREADS];
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    const bool act = p.col[c].active != 0;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    const bool act = pair_active(p, c);
     double v[2] = {0.0, 0.0};
-    const long long items = (long long)p.npad * P;
+    const long long items = (long long)p.npad * C;
     if (act) {
         for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
              idx += (long long)gridDim.x * THREADS) {
@@ -582,13 +591,13 @@ __global__ void __launch_bounds__(THREADS) k_refine_start(PanelDev p, const doub
             v[1] += bv.y * bv.y;
         }
     }
-    if (grid_reduce_cols<2>(v, P, p, smem)) {
+    if (grid_reduce_cols<2>(v, C, p, smem)) {
         const int t = threadIdx.x;
         int nact = 0;
-        if (t < P) {
-            const bool cact = p.col[t].active != 0;
-            if (cact) p.col[t].rnorm = sqrt(smem[t] + smem[THREADS + t]);
+        if (t < C) {
             for (int part = 0; part < 2; ++part) {
+                const bool cact = p.col[2 * t + part].active != 0;
+                if (cact) p.col[2 * t + part].rnorm = sqrt(smem[part * THREADS + t]);
                 const double b2 = smem[part * THREADS + t];
                 p.inner[2 * t + part].bnorm2 = b2;
                 InnerState st = p.inner32[2 * t + part];
@@ -608,25 +617,25 @@ __global__ void __launch_bounds__(THREADS) k_refine_start(PanelDev p, const doub
 template <bool DF, bool RAG = false>
 __global__ void __launch_bounds__(THREADS) k_refine_residual(DevSystem s, PanelDev p, const double2* __restrict__ b) {
     __shared__ double smem[2 * THREADS];
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    const bool act = p.col[c].active != 0 && !(p.inner32[2 * c].skip && p.inner32[2 * c + 1].skip);
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    const bool act = pair_active(p, c) && !(p.inner32[2 * c].skip && p.inner32[2 * c + 1].skip);
     double v[2] = {0.0, 0.0};
-    const long long items = (long long)s.n_atoms * P;
+    const long long items = (long long)s.n_atoms * C;
     if (act) {
         for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
              idx += (long long)gridDim.x * THREADS) {
-            const int I = (int)(idx / P);
+            const int I = (int)(idx / C);
             double2 acc[4];
             if (DF) {
                 float2 ah[4], al[4];
 #pragma unroll
                 for (int a = 0; a < 4; ++a) ah[a] = al[a] = make_float2(0.f, 0.f);
-                if (RAG) df_row_ragged(s, s.S32, s.S32lo, I, s.norb[I], p.RpS, P, c, ah, al);
+                if (RAG) df_row_ragged(s, s.S32, s.S32lo, I, s.norb[I], p.RpS, C, c, ah, al);
                 for (int bb = RAG ? s.brow[I + 1] : s.brow[I]; bb < s.brow[I + 1]; ++bb) {
                     const int J = s.bcol[bb];
-                    const float4* xr = p.RpS + (size_t)4 * J * P + c;
-                    const float4 x[4] = {xr[0], xr[P], xr[2 * P], xr[3 * P]};
+                    const float4* xr = p.RpS + (size_t)4 * J * C + c;
+                    const float4 x[4] = {xr[0], xr[C], xr[2 * C], xr[3 * C]};
                     const float4* Sh = reinterpret_cast<const float4*>(s.S32 + 16 * (size_t)bb);
                     const float4* Sl = reinterpret_cast<const float4*>(s.S32lo + 16 * (size_t)bb);
 #pragma unroll
@@ -647,8 +656,8 @@ __global__ void __launch_bounds__(THREADS) k_refine_residual(DevSystem s, PanelD
                 for (int a = 0; a < 4; ++a) acc[a] = cmk(0.0, 0.0);
                 for (int bb = s.brow[I]; bb < s.brow[I + 1]; ++bb) {
                     const int J = s.bcol[bb];
-                    const double2* xr = p.Rp + (size_t)4 * J * P + c;
-                    const double2 x0 = xr[0], x1 = xr[P], x2 = xr[2 * P], x3 = xr[3 * P];
+                    const double2* xr = p.Rp + (size_t)4 * J * C + c;
+                    const double2 x0 = xr[0], x1 = xr[C], x2 = xr[2 * C], x3 = xr[3 * C];
                     const double2* Sb = reinterpret_cast<const double2*>(s.S + 16 * (size_t)bb);
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
@@ -660,7 +669,7 @@ __global__ void __launch_bounds__(THREADS) k_refine_residual(DevSystem s, PanelD
             }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                const size_t e = (size_t)(4 * I + a) * P + c;
+                const size_t e = (size_t)(4 * I + a) * C + c;
                 const double2 r = csub(b[e], acc[a]);
                 p.Rin[e] = r;
                 v[0] += r.x * r.x;
@@ -668,12 +677,12 @@ __global__ void __launch_bounds__(THREADS) k_refine_residual(DevSystem s, PanelD
             }
         }
     }
-    if (grid_reduce_cols<2>(v, P, p, smem)) {
+    if (grid_reduce_cols<2>(v, C, p, smem)) {
         const int t = threadIdx.x;
         int nact = 0;
-        if (t < P) {
-            const bool cact = p.col[t].active != 0;
+        if (t < C) {
             for (int part = 0; part < 2; ++part) {
+                const bool cact = p.col[2 * t + part].active != 0;
                 InnerState st = p.inner32[2 * t + part];
                 if (!st.skip) {
                     const double r2 = smem[part * THREADS + t];
@@ -704,17 +713,17 @@ __global__ void __launch_bounds__(THREADS) k_refine_residual(DevSystem s, PanelD
 // round reads them).  cheb_gamma > 0: also the first Chebyshev iterate
 // d_1 = gamma f into x32 (the next round makes Chebyshev corrections).
 __global__ void k_refine_scale(PanelDev p, const double2* __restrict__ src, float cheb_gamma) {
-    const int P = p.P;
-    const int c = threadIdx.x % P;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
     if (blockIdx.x == 0) {
-        for (int q = threadIdx.x; q < 8 * P; q += THREADS) p.acc32[q] = 0.0;   // both CG sum slots
+        for (int q = threadIdx.x; q < 8 * C; q += THREADS) p.acc32[q] = 0.0;   // both CG sum slots
         if (threadIdx.x == 0) p.flags[7] = -1;                                  // no CG scalars yet
     }
-    if (!p.col[c].active) return;
+    if (!pair_active(p, c)) return;
     const InnerState i0 = p.inner32[2 * c], i1 = p.inner32[2 * c + 1];
     if (i0.skip && i1.skip) return;
     const double s0 = i0.scale, s1 = i1.scale;
-    const long long items = (long long)p.npad * P;
+    const long long items = (long long)p.npad * C;
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
         const double2 v = src[idx];
@@ -727,10 +736,10 @@ __global__ void k_refine_scale(PanelDev p, const double2* __restrict__ src, floa
 // r' copied into the FP64 inner right-hand side slot and split for the
 // double-float products (after an FP64 redo of a mixed inner solve)
 __global__ void k_split_panel(PanelDev p) {
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    if (!p.col[c].active) return;
-    const long long items = (long long)p.npad * P;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    if (!pair_active(p, c)) return;
+    const long long items = (long long)p.npad * C;
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS)
         p.RpS[idx] = df_split(p.Rp[idx]);
@@ -738,14 +747,14 @@ __global__ void k_split_panel(PanelDev p) {
 
 // x += d / scale (FP32 correction added in FP64) for the columns that took the round
 __global__ void k_refine_add(PanelDev p) {
-    const int P = p.P;
-    const int c = threadIdx.x % P;
-    if (!p.col[c].active) return;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
+    if (!pair_active(p, c)) return;
     const InnerState i0 = p.inner32[2 * c], i1 = p.inner32[2 * c + 1];
     const bool u0 = !i0.skip, u1 = !i1.skip;
     if (!u0 && !u1) return;
     const double f0 = u0 ? i0.unscale : 0.0, f1 = u1 ? i1.unscale : 0.0;
-    const long long items = (long long)p.npad * P;
+    const long long items = (long long)p.npad * C;
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
         const float2 d = p.x32[idx];
@@ -765,15 +774,14 @@ __global__ void k_refine_add(PanelDev p) {
 // derives the same alpha, beta and convergence flags from them (identical
 // inputs, identical arithmetic).  The CG state is double-buffered as well:
 // update(it) reads slot it&1 and CTA 0 writes slot (it+1)&1.
-//   inner32[0 .. 2P)        refinement state (skip, scale), written by k_refine_*
-//   inner32[2P .. 4P)       CG state slot 0
-//   inner32[4P .. 6P)       CG state slot 1
-//   acc32[(slot*4 + q)*P + c]  gamma_re, gamma_im, delta_re, delta_im of column c
+//   inner32[0 .. P)        refinement state (skip, scale), written by k_refine_*
+//   inner32[P .. 2P)       CG state slot 0
+//   inner32[2P .. 3P)       CG state slot 1
+//   acc32[(slot*4 + q)*C + c]  gamma, gamma', delta, delta' of the two columns of pair c
 
 // Packed FP32 FMA of Blackwell (two lanes per instruction): d = a * b + c
 // elementwise on float2.  The block products below broadcast one S entry
-// into both lanes, so one instruction updates the real and imaginary parts
-// of one complex column.
+// into both lanes, so one instruction updates the two columns of one pair.
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
     unsigned long long ra, rb, rc, rd;
     asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
@@ -788,24 +796,24 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
 // CG scalars of iteration it, once, by the last CTA of the SpMV to finish
 // (every thread of that CTA calls this): FP64 alpha, beta and the
 // convergence of every real column from the accumulated sums; the update
-// kernel that follows only reads them (cgs[0..2P) alpha, [2P..4P) beta,
-// upd flags in cgu[0..2P)).  The sums are read through L2 (__ldcg): other
+// kernel that follows only reads them (cgs[0..P) alpha, [P..2P) beta,
+// upd flags in cgu[0..P)).  The sums are read through L2 (__ldcg): other
 // CTAs added them with device-scope atomics before their fence and ticket.
 __device__ void inner32_scalars_cta(const PanelDev& p, int it) {
     __shared__ int s_cnt, s_err;
-    const int P = p.P;
+    const int C = p.C;
     const InnerState* base = p.inner32;
-    const InnerState* prev = p.inner32 + (size_t)(1 + (it & 1)) * 2 * P;
-    InnerState* next = p.inner32 + (size_t)(1 + ((it + 1) & 1)) * 2 * P;
-    const double* acc_slot = p.acc32 + (size_t)(it & 1) * 4 * P;
+    const InnerState* prev = p.inner32 + (size_t)(1 + (it & 1)) * 2 * C;
+    InnerState* next = p.inner32 + (size_t)(1 + ((it + 1) & 1)) * 2 * C;
+    const double* acc_slot = p.acc32 + (size_t)(it & 1) * 4 * C;
     if (threadIdx.x == 0) { s_cnt = 0; s_err = 0; }
     __syncthreads();
-    for (int rc = threadIdx.x; rc < 2 * P; rc += blockDim.x) {
+    for (int rc = threadIdx.x; rc < 2 * C; rc += blockDim.x) {
         const int c = rc >> 1, part = rc & 1;
-        const bool cact = p.col[c].active != 0;
+        const bool cact = p.col[rc].active != 0;
         InnerState st = prev[rc];
-        const double gam = __ldcg(acc_slot + (size_t)part * P + c);
-        const double del = __ldcg(acc_slot + (size_t)(2 + part) * P + c);
+        const double gam = __ldcg(acc_slot + (size_t)part * C + c);
+        const double del = __ldcg(acc_slot + (size_t)(2 + part) * C + c);
         if (it == 0) {
             st.bnorm2 = gam;
             st.conv = (!cact || base[rc].skip || gam == 0.0) ? 1 : 0;
@@ -838,17 +846,17 @@ __device__ void inner32_scalars_cta(const PanelDev& p, int it) {
             }
         }
         p.cgs[rc] = st.alpha;
-        p.cgs[2 * P + rc] = st.beta;
+        p.cgs[2 * C + rc] = st.beta;
         p.cgu[rc] = st.conv ? 0 : 1;
         if (!st.conv) atomicAdd(&s_cnt, 1);
         next[rc] = st;
         if (p.hist && it < HIST_IT) {
-            double* hh = p.hist + ((size_t)it * 2 * P + rc) * 4;
+            double* hh = p.hist + ((size_t)it * 2 * C + rc) * 4;
             hh[0] = gam; hh[1] = del; hh[2] = st.conv ? 0.0 : st.alpha; hh[3] = st.conv ? 0.0 : st.beta;
         }
     }
-    double* acc_next = p.acc32 + (size_t)((it + 1) & 1) * 4 * P;
-    for (int q = threadIdx.x; q < 4 * P; q += blockDim.x) acc_next[q] = 0.0;
+    double* acc_next = p.acc32 + (size_t)((it + 1) & 1) * 4 * C;
+    for (int q = threadIdx.x; q < 4 * C; q += blockDim.x) acc_next[q] = 0.0;
     __syncthreads();
     if (threadIdx.x == 0) {
         p.flags[1] = s_cnt;
@@ -876,27 +884,27 @@ __device__ void inner32_ticket_tail(const PanelDev& p, int it) {
 }
 
 // w = S r (FP32) and the sums gamma = r.r, delta = w.r of every real column.
-// CPT complex columns per thread (2: one float4 per orbital row), P / CPT
+// CPT column pairs per thread (2: one float4 per orbital row), C / CPT
 // threads per block row; the block-column index of the next block is loaded
 // one block ahead so the panel-row gathers do not wait on it.
-// PW: the panel width as a compile-time constant (4 ... 256: row strides
-// fold into the load offsets; measured 4 % faster at 256 columns), 0 for
+// PW: the panel's pair count as a compile-time constant (4 ... 128: row strides
+// fold into the load offsets; measured 4 % faster at 256 pairs), 0 for
 // any width at run time.
 template <int CPT, int PW = 0>
 __global__ void __launch_bounds__(THREADS, 4) k_inner32_spmv(DevSystem s, PanelDev p, int it) {
     __shared__ double smem[4 * CPT * THREADS];
     if (*(volatile int*)&p.flags[1] == 0) return;
-    const int P = PW > 0 ? PW : p.P;
-    const int TPR = P / CPT;                    // threads per block row
+    const int C = PW > 0 ? PW : p.C;
+    const int TPR = C / CPT;                    // threads per block row
     const int t0 = threadIdx.x % TPR;
     const int c0 = t0 * CPT;
     const InnerState* base = p.inner32;
-    const InnerState* cgp = p.inner32 + (size_t)(1 + (it & 1)) * 2 * P;
+    const InnerState* cgp = p.inner32 + (size_t)(1 + (it & 1)) * 2 * C;
     bool live = false;
 #pragma unroll
     for (int j = 0; j < CPT; ++j) {
         const int c = c0 + j;
-        live |= p.col[c].active && (it == 0 ? !(base[2 * c].skip && base[2 * c + 1].skip)
+        live |= pair_active(p, c) && (it == 0 ? !(base[2 * c].skip && base[2 * c + 1].skip)
                                             : !(cgp[2 * c].conv && cgp[2 * c + 1].conv));
     }
     float v32[4 * CPT];
@@ -918,10 +926,10 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_spmv(DevSystem s, PanelD
                 const int J = Jn;
                 if (bb + 1 < b1) Jn = __ldg(s.bcol + bb + 1);
                 float xv[4][2 * CPT];
-                const float2* xb = p.r32 + (size_t)(4 * J) * P + c0;
+                const float2* xb = p.r32 + (size_t)(4 * J) * C + c0;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float2* xr = xb + e * P;
+                    const float2* xr = xb + e * C;
                     if (CPT == 2) {
                         const float4 q4 = *reinterpret_cast<const float4*>(xr);
                         xv[e][0] = q4.x; xv[e][1] = q4.y; xv[e][2] = q4.z; xv[e][3] = q4.w;
@@ -941,7 +949,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_spmv(DevSystem s, PanelD
             }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                const size_t e = (size_t)(4 * I + a) * P + c0;
+                const size_t e = (size_t)(4 * I + a) * C + c0;
                 float r[2 * CPT];
                 if (CPT == 2) {
                     const float4 r4 = *reinterpret_cast<const float4*>(p.r32 + e);
@@ -967,14 +975,14 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_spmv(DevSystem s, PanelD
     for (int q = 0; q < 4 * CPT; ++q) v[q] = v32[q];
     block_reduce_cols<4 * CPT>(v, TPR, smem);
     if (threadIdx.x < TPR) {
-        double* acc_slot = p.acc32 + (size_t)(it & 1) * 4 * P;
+        double* acc_slot = p.acc32 + (size_t)(it & 1) * 4 * C;
 #pragma unroll
         for (int j = 0; j < CPT; ++j) {
             const int c = threadIdx.x * CPT + j;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const double val = smem[(4 * j + q) * THREADS + threadIdx.x];
-                if (val != 0.0) atomicAdd(acc_slot + (size_t)q * P + c, val);
+                if (val != 0.0) atomicAdd(acc_slot + (size_t)q * C + c, val);
             }
         }
     }
@@ -986,14 +994,14 @@ __device__ __forceinline__ uint32_t smem_u32(const void* ptr) {
 }
 
 // Grouped form: CTA (g, slice) computes the 4G rows of the G consecutive
-// atoms of group g for the PC complex columns of one panel slice.  The panel
+// atoms of group g for the PC column pairs of one panel slice.  The panel
 // rows of the distinct block columns of the group (its neighbour union, built
 // on the host when the system is created) and the group's FP32 S blocks are
 // staged once in shared memory by 16-byte asynchronous copies; every block
 // product then reads shared memory.  The union of 16 neighbouring atoms is
 // ~3x smaller than the sum of their neighbour lists, so the L2 -> SM gather
-// traffic drops by that factor.  PC / 2 threads per atom, two complex
-// columns each; the block products pair (S[a][e], S[a][e+1]), two adjacent
+// traffic drops by that factor.  PC / 2 threads per atom, two
+// pairs each; the block products pair (S[a][e], S[a][e+1]), two adjacent
 // lanes of a loaded S row, against (x[e][q], x[e+1][q]) in packed FP32 FMAs.
 constexpr int PC = 32;
 constexpr int GRP_HDR = 128;   // reserved head of the dynamic shared memory
@@ -1001,8 +1009,8 @@ constexpr int GRP_HDR = 128;   // reserved head of the dynamic shared memory
 __global__ void __launch_bounds__(256) k_inner32_spmv_grp(DevSystem s, PanelDev p, int it) {
     extern __shared__ __align__(128) unsigned char gsm[];
     if (*(volatile int*)&p.flags[1] == 0) return;
-    const int P = p.P;
-    const int nslices = P / PC;
+    const int C = p.C;
+    const int nslices = C / PC;
     const int g = blockIdx.x / nslices;
     const int slice = blockIdx.x - g * nslices;
     const int a0 = g * s.grpG;
@@ -1017,13 +1025,13 @@ __global__ void __launch_bounds__(256) k_inner32_spmv_grp(DevSystem s, PanelDev 
     const int tc = t % TPA;
     const int c0 = slice * PC + 2 * tc;
     const InnerState* base = p.inner32;
-    const InnerState* cgp = p.inner32 + (size_t)(1 + (it & 1)) * 2 * P;
+    const InnerState* cgp = p.inner32 + (size_t)(1 + (it & 1)) * 2 * C;
     bool live = false;
     if (I < a1) {
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const int c = c0 + j;
-            live |= p.col[c].active && (it == 0 ? !(base[2 * c].skip && base[2 * c + 1].skip)
+            live |= pair_active(p, c) && (it == 0 ? !(base[2 * c].skip && base[2 * c + 1].skip)
                                                 : !(cgp[2 * c].conv && cgp[2 * c + 1].conv));
         }
     }
@@ -1041,7 +1049,7 @@ __global__ void __launch_bounds__(256) k_inner32_spmv_grp(DevSystem s, PanelDev 
         for (int k = t; k < nx; k += blockDim.x) {
             const int row = k / TPA, q4 = k - row * TPA;
             const int J = __ldg(s.grp_cols + u0 + row / 4);
-            const float2* src = p.r32 + (size_t)(4 * J + (row & 3)) * P + slice * PC + 2 * q4;
+            const float2* src = p.r32 + (size_t)(4 * J + (row & 3)) * C + slice * PC + 2 * q4;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(xs_a + 16u * (uint32_t)k), "l"(src));
         }
         const uint32_t ss_a = smem_u32(ss);
@@ -1096,7 +1104,7 @@ __global__ void __launch_bounds__(256) k_inner32_spmv_grp(DevSystem s, PanelDev 
             for (int q = 0; q < 4; ++q) acc[a][q] = acc2[a][q].x + acc2[a][q].y;
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
-            const size_t e = (size_t)(4 * I + a) * P + c0;
+            const size_t e = (size_t)(4 * I + a) * C + c0;
             const float4 r4 = *reinterpret_cast<const float4*>(p.r32 + e);
             *reinterpret_cast<float4*>(p.w32 + e) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
             const float r[4] = {r4.x, r4.y, r4.z, r4.w};
@@ -1125,7 +1133,7 @@ __global__ void __launch_bounds__(256) k_inner32_spmv_grp(DevSystem s, PanelDev 
         double sum = 0.0;
         for (int w = 0; w < (int)(blockDim.x / 32); ++w) sum += red[((size_t)w * TPA + tcol) * 8 + q];
         const int c = slice * PC + 2 * tcol + q / 4;
-        if (sum != 0.0) atomicAdd(p.acc32 + (size_t)(it & 1) * 4 * P + (size_t)(q % 4) * P + c, sum);
+        if (sum != 0.0) atomicAdd(p.acc32 + (size_t)(it & 1) * 4 * C + (size_t)(q % 4) * C + c, sum);
     }
     inner32_ticket_tail(p, it);
 }
@@ -1136,12 +1144,12 @@ __global__ void __launch_bounds__(256) k_inner32_spmv_grp(DevSystem s, PanelDev 
 // is initialised.
 template <int V>
 __global__ void k_inner32_update(PanelDev p, int it) {
-    // V complex columns per thread (V = 2: one float4 of each vector)
+    // V column pairs per thread (V = 2: one float4 of each vector)
     using vec = typename std::conditional<V == 2, float4, float2>::type;
-    const int P = p.P;
+    const int C = p.C;
     if (*(volatile int*)&p.flags[7] != it) return;      // no scalars for this iteration (the SpMV exited early)
-    const int c0 = (V * threadIdx.x) % P;
-    // per real column q: act (the complex column is active: at it == 0 its
+    const int c0 = (V * threadIdx.x) % C;
+    // per column q: act (the column is active: at it == 0 its
     // p, s, x start at zero) and upd (this iteration updates it); inactive
     // columns keep their vectors
     float a[2 * V], b[2 * V];
@@ -1150,19 +1158,19 @@ __global__ void k_inner32_update(PanelDev p, int it) {
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         const int c = c0 + j;
-        const bool ac = p.col[c].active != 0;
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
             const int q = 2 * j + part, rc = 2 * c + part;
+            const bool ac = p.col[rc].active != 0;
             act[q] = ac;
             upd[q] = ac && p.cgu[rc] != 0;
             a[q] = upd[q] ? (float)p.cgs[rc] : 0.f;
-            b[q] = upd[q] ? (float)p.cgs[2 * P + rc] : 0.f;
+            b[q] = upd[q] ? (float)p.cgs[2 * C + rc] : 0.f;
             any |= (it == 0) ? act[q] : upd[q];
         }
     }
     if (!any) return;
-    const long long items = (long long)p.npad * P / V;
+    const long long items = (long long)p.npad * C / V;
     vec* r32 = reinterpret_cast<vec*>(p.r32);
     vec* w32 = reinterpret_cast<vec*>(p.w32);
     vec* p32 = reinterpret_cast<vec*>(p.p32);
@@ -1217,12 +1225,12 @@ __global__ void k_inner32_update(PanelDev p, int it) {
 // and the gather reads d_k alone).  f is the round's right-hand side r32.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool cheb_live(const PanelDev& p, int c) {
-    return p.col[c].active && !(p.inner32[2 * c].skip && p.inner32[2 * c + 1].skip);
+    return pair_active(p, c) && !(p.inner32[2 * c].skip && p.inner32[2 * c + 1].skip);
 }
 
 // One Chebyshev step: io <- io + omega (gamma (f - S cur) + cur - io) on the
-// own rows, with S cur gathered as in k_inner32_spmv (CPT complex columns
-// per thread, P / CPT threads per block row, PW the panel width when it is
+// own rows, with S cur gathered as in k_inner32_spmv (CPT column pairs
+// per thread, C / CPT threads per block row, PW the pair count when it is
 // a compile-time constant).  mode 1: the first step (d_0 = 0, io is not
 // read).  mode 2 (the LAST instance): the last step, which adds its result
 // to the FP64 solution of the refinement instead of storing it
@@ -1235,8 +1243,8 @@ template <int CPT, int PW = 0, bool LAST = false>
 __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelDev p, const float2* __restrict__ cur,
                                                             float2* io, float omega, float gamma, int mode) {
     if (*(volatile int*)&p.flags[4] == 0) return;
-    const int P = PW > 0 ? PW : p.P;
-    const int TPR = P / CPT;
+    const int C = PW > 0 ? PW : p.C;
+    const int TPR = C / CPT;
     const int t0 = threadIdx.x % TPR;
     const int c0 = t0 * CPT;
     bool live = false;
@@ -1259,10 +1267,10 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelD
             if (bb + 1 < b1) Jn = __ldg(s.bcol + bb + 1);
             if (s.unit_diag && J == I) continue;   // S_II = 1: d_I is added in the update
             float xv[4][2 * CPT];
-            const float2* xb = cur + (size_t)(4 * J) * P + c0;
+            const float2* xb = cur + (size_t)(4 * J) * C + c0;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float2* xr = xb + e * P;
+                const float2* xr = xb + e * C;
                 if (CPT == 2) {
                     const float4 q4 = *reinterpret_cast<const float4*>(xr);
                     xv[e][0] = q4.x; xv[e][1] = q4.y; xv[e][2] = q4.z; xv[e][3] = q4.w;
@@ -1282,7 +1290,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelD
         }
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
-            const size_t e = (size_t)(4 * I + a) * P + c0;
+            const size_t e = (size_t)(4 * I + a) * C + c0;
             float f[2 * CPT], dc[2 * CPT], dp[2 * CPT];
             if (CPT == 2) {
                 const float4 f4 = *reinterpret_cast<const float4*>(p.r32 + e);
@@ -1303,10 +1311,9 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelD
                 for (int j = 0; j < CPT; ++j) {
                     // 1 / scale of the real columns that took the round (0: skipped)
                     const InnerState i0 = p.inner32[2 * (c0 + j)], i1 = p.inner32[2 * (c0 + j) + 1];
-                    const bool ca = p.col[c0 + j].active != 0;
                     double2 x = p.Rp[e + j];
-                    if (ca && !i0.skip && isfinite(dn[2 * j])) x.x += (double)dn[2 * j] * i0.unscale;
-                    if (ca && !i1.skip && isfinite(dn[2 * j + 1])) x.y += (double)dn[2 * j + 1] * i1.unscale;
+                    if (!i0.skip && isfinite(dn[2 * j])) x.x += (double)dn[2 * j] * i0.unscale;
+                    if (!i1.skip && isfinite(dn[2 * j + 1])) x.y += (double)dn[2 * j + 1] * i1.unscale;
                     p.Rp[e + j] = x;
                     p.RpS[e + j] = df_split(x);
                 }
@@ -1319,22 +1326,19 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelD
     }
 }
 
-// The same Chebyshev step with four complex columns per thread and packed
-// FP32 FMAs: thread t0 of a block row (P / 4 threads per row) takes the
-// column pairs (2 t0, 2 t0 + 1) and (P/2 + 2 t0, P/2 + 2 t0 + 1), so each of
+// The same Chebyshev step with four column pairs per thread and packed
+// FP32 FMAs: thread t0 of a block row (C / 4 threads per row) takes the
+// pairs (2 t0, 2 t0 + 1) and (C/2 + 2 t0, C/2 + 2 t0 + 1), so each of
 // its two loads per gathered row is part of a contiguous 512-byte warp
 // access.  The block product runs over the rows e of the gathered d_k: row e
 // of the transposed block (column e of S_IJ, from S32T) gives S[a][e] for
 // the four output rows a, each broadcast into both lanes of a packed FMA
-// against the (re, im) pairs of the thread's columns.  Against two columns
-// per thread this halves the S loads and the FMA instructions per column
-// (ncu at P = 128: 7.3 M instead of 15.5 M warp instructions per launch).
-// Compiled for three CTAs per SM (80 registers): at four (64 registers) the
-// 32 accumulators spill.  Measured on the benchmark workload, four panels in
-// flight: 17.2 M shift*RHS*iterations/s against 15.8 M with two columns per
-// thread; eight columns per thread (two CTAs per SM), staging the next
-// block's rows in shared memory, and L1 / L2 prefetches of them all measured
-// slower.
+// against the two columns of a pair.  Against two pairs per thread this
+// halves the S loads and the FMA instructions per column (ncu at 128 pairs:
+// 7.3 M instead of 15.5 M warp instructions per launch).  Compiled for three
+// CTAs per SM (80 registers): at four (64 registers) the 32 accumulators
+// spill.  Eight pairs per thread (two CTAs per SM), staging the next block's
+// rows in shared memory, and L1 / L2 prefetches of them all measured slower.
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
@@ -1343,9 +1347,9 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4(DevSystem s, Panel
                                                              float2* io, float omega, float gamma, int mode) {
     constexpr int CPT = 4, NP = 2;   // columns, column pairs per thread
     if (*(volatile int*)&p.flags[4] == 0) return;
-    const int P = PW > 0 ? PW : p.P;
-    const int TPR = P / CPT;
-    const int pstride = P / NP;
+    const int C = PW > 0 ? PW : p.C;
+    const int TPR = C / CPT;
+    const int pstride = C / NP;
     const int t0 = threadIdx.x % TPR;
     bool live = false;
 #pragma unroll
@@ -1366,13 +1370,13 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4(DevSystem s, Panel
             const int J = Jn;
             if (bb + 1 < b1) Jn = __ldg(s.bcol + bb + 1);
             if (s.unit_diag && J == I) continue;   // S_II = 1: d_I is added in the update
-            const float2* xb = cur + (size_t)(4 * J) * P + 2 * t0;
+            const float2* xb = cur + (size_t)(4 * J) * C + 2 * t0;
             const float4* St = reinterpret_cast<const float4*>(s.S32T + 16 * (size_t)bb);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 float4 xq[NP];
 #pragma unroll
-                for (int k = 0; k < NP; ++k) xq[k] = *reinterpret_cast<const float4*>(xb + (size_t)e * P + k * pstride);
+                for (int k = 0; k < NP; ++k) xq[k] = *reinterpret_cast<const float4*>(xb + (size_t)e * C + k * pstride);
                 const float4 sc = __ldg(St + e);     // S[0][e], S[1][e], S[2][e], S[3][e]
                 const float sv[4] = {sc.x, sc.y, sc.z, sc.w};
 #pragma unroll
@@ -1388,7 +1392,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4(DevSystem s, Panel
         }
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
-            const size_t row = (size_t)(4 * I + a) * P;
+            const size_t row = (size_t)(4 * I + a) * C;
 #pragma unroll
             for (int k = 0; k < NP; ++k) {
                 const int c = k * pstride + 2 * t0;
@@ -1406,10 +1410,9 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4(DevSystem s, Panel
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const InnerState i0 = p.inner32[2 * (c + j)], i1 = p.inner32[2 * (c + j) + 1];
-                        const bool ca = p.col[c + j].active != 0;
                         double2 x = p.Rp[e + j];
-                        if (ca && !i0.skip && isfinite(dn[2 * j])) x.x += (double)dn[2 * j] * i0.unscale;
-                        if (ca && !i1.skip && isfinite(dn[2 * j + 1])) x.y += (double)dn[2 * j + 1] * i1.unscale;
+                        if (!i0.skip && isfinite(dn[2 * j])) x.x += (double)dn[2 * j] * i0.unscale;
+                        if (!i1.skip && isfinite(dn[2 * j + 1])) x.y += (double)dn[2 * j + 1] * i1.unscale;
                         p.Rp[e + j] = x;
                         p.RpS[e + j] = df_split(x);
                     }
@@ -1432,9 +1435,9 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4r(DevSystem s, Pane
                                                               float2* io, float omega, float gamma, int mode) {
     constexpr int NP = 2;
     if (*(volatile int*)&p.flags[4] == 0) return;
-    const int P = PW > 0 ? PW : p.P;
-    const int TPR = P / 4;
-    const int pstride = P / NP;
+    const int C = PW > 0 ? PW : p.C;
+    const int TPR = C / 4;
+    const int pstride = C / NP;
     const int t0 = threadIdx.x % TPR;
     bool live = false;
 #pragma unroll
@@ -1460,7 +1463,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4r(DevSystem s, Pane
             const int J = m.x;
             const int nj = (m.y < 0) ? 1 : 4;
             if (s.unit_diag && J == I) continue;   // S_II = 1: d_I is added in the update
-            const float2* xb = cur + (size_t)(4 * J) * P + 2 * t0;
+            const float2* xb = cur + (size_t)(4 * J) * C + 2 * t0;
             const float4* Sr = reinterpret_cast<const float4*>(s.S32r) + (m.y & 0x7fffffff);
             if (ni == 4) {
                 // nj rows e of the gathered d_k, column e of the block as four
@@ -1469,8 +1472,8 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4r(DevSystem s, Pane
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     if (e >= nj) break;
-                    const float4 xa = *reinterpret_cast<const float4*>(xb + (size_t)e * P);
-                    const float4 xq = *reinterpret_cast<const float4*>(xb + (size_t)e * P + pstride);
+                    const float4 xa = *reinterpret_cast<const float4*>(xb + (size_t)e * C);
+                    const float4 xq = *reinterpret_cast<const float4*>(xb + (size_t)e * C + pstride);
                     const float4 sc = __ldg(Sr + e);
                     const float sv[4] = {sc.x, sc.y, sc.z, sc.w};
 #pragma unroll
@@ -1489,8 +1492,8 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4r(DevSystem s, Pane
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     if (e >= nj) break;
-                    const float4 xa = *reinterpret_cast<const float4*>(xb + (size_t)e * P);
-                    const float4 xq = *reinterpret_cast<const float4*>(xb + (size_t)e * P + pstride);
+                    const float4 xa = *reinterpret_cast<const float4*>(xb + (size_t)e * C);
+                    const float4 xq = *reinterpret_cast<const float4*>(xb + (size_t)e * C + pstride);
                     const float2 s2 = make_float2(sv[e], sv[e]);
                     acc[0][0] = __ffma2_rn(s2, lo2(xa), acc[0][0]);
                     acc[0][1] = __ffma2_rn(s2, hi2(xa), acc[0][1]);
@@ -1502,7 +1505,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4r(DevSystem s, Pane
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             if (a >= ni) break;
-            const size_t row = (size_t)(4 * I + a) * P;
+            const size_t row = (size_t)(4 * I + a) * C;
 #pragma unroll
             for (int k = 0; k < NP; ++k) {
                 const int c = k * pstride + 2 * t0;
@@ -1520,10 +1523,9 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4r(DevSystem s, Pane
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const InnerState i0 = p.inner32[2 * (c + j)], i1 = p.inner32[2 * (c + j) + 1];
-                        const bool ca = p.col[c + j].active != 0;
                         double2 x = p.Rp[e + j];
-                        if (ca && !i0.skip && isfinite(dn[2 * j])) x.x += (double)dn[2 * j] * i0.unscale;
-                        if (ca && !i1.skip && isfinite(dn[2 * j + 1])) x.y += (double)dn[2 * j + 1] * i1.unscale;
+                        if (!i0.skip && isfinite(dn[2 * j])) x.x += (double)dn[2 * j] * i0.unscale;
+                        if (!i1.skip && isfinite(dn[2 * j + 1])) x.y += (double)dn[2 * j + 1] * i1.unscale;
                         p.Rp[e + j] = x;
                         p.RpS[e + j] = df_split(x);
                     }
@@ -1535,76 +1537,71 @@ __global__ void __launch_bounds__(THREADS, 3) k_inner32_cheb4r(DevSystem s, Pane
     }
 }
 
-// rho_{n+1} = r_{n+1}^T r'_{n+1} (unconjugated); also clears the count of
-// active columns that the shift step rebuilds.
+// t_{n+1} = u_{n+1}^T u'_{n+1}; also clears the count of active columns that
+// the shift step rebuilds.
 __global__ void __launch_bounds__(THREADS) k_finish(PanelDev p) {
     __shared__ double smem[2 * THREADS];
-    const int P = p.P;
-    const int c = threadIdx.x % P;
+    const int C = p.C;
+    const int c = threadIdx.x % C;
     double v[2] = {0.0, 0.0};
-    if (p.col[c].active) {
-        const long long items = (long long)p.npad * P;
+    if (pair_active(p, c)) {
+        const long long items = (long long)p.npad * C;
         for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
              idx += (long long)gridDim.x * THREADS) {
-            const double2 m = cmul(p.Rcur[idx], p.Rp[idx]);
-            v[0] += m.x;
-            v[1] += m.y;
+            const double2 u = p.Rcur[idx], x = p.Rp[idx];
+            v[0] += u.x * x.x;
+            v[1] += u.y * x.y;
         }
     }
-    if (grid_reduce_cols<2>(v, P, p, smem)) {
-        const int t = threadIdx.x;
-        if (t < P && p.col[t].active) p.col[t].rho_new = cmk(smem[t], smem[THREADS + t]);
-        if (t == 0) p.flags[2] = 0;
+    if (grid_reduce_cols<2>(v, C, p, smem)) {
+        for (int t = threadIdx.x; t < p.P; t += THREADS)
+            if (p.col[t].active) p.col[t].t_new = smem[(t & 1) * THREADS + (t >> 1)];
+        if (threadIdx.x == 0) p.flags[2] = 0;
     }
 }
 
-// Projected functionals f_m^T r' of column c into d[0..nfun).
-__device__ void eval_functionals(const DevSystem& s, const PanelDev& p, int c, int nfun, double2* d,
-                                 double* red) {
+// Projected functionals f_m^T u' of column c into d[0..nfun).
+__device__ void eval_functionals(const DevSystem& s, const PanelDev& p, int c, int nfun, double* d, double* red) {
     const int tid = threadIdx.x;
+    const double* Rp = reinterpret_cast<const double*>(p.Rp);
     if (p.proj == PROJ_ROWS) {
-        for (int m = tid; m < nfun; m += THREADS) d[m] = p.Rp[(size_t)p.frow[(size_t)c * p.M + m] * p.P + c];
+        for (int m = tid; m < nfun; m += THREADS) d[m] = Rp[(size_t)p.frow[(size_t)c * p.M + m] * p.P + c];
     } else if (p.proj == PROJ_SROW) {
-        // s_j^T r' = sum over row j of S (S symmetric)
+        // s_j^T u' = sum over row j of S (S symmetric)
         const int row = p.col[c].row, I = row >> 2, a = row & 3;
         const int b0 = s.brow[I], nbl = s.brow[I + 1] - b0;
-        double re = 0.0, im = 0.0;
+        double acc = 0.0;
         for (int e = tid; e < 4 * nbl; e += THREADS) {
             const int b = b0 + e / 4, be = e % 4;
-            const double sv = s.S[16 * (size_t)b + 4 * a + be];
-            const double2 x = p.Rp[(size_t)(4 * s.bcol[b] + be) * p.P + c];
-            re += sv * x.x;
-            im += sv * x.y;
+            acc += s.S[16 * (size_t)b + 4 * a + be] * Rp[(size_t)(4 * s.bcol[b] + be) * p.P + c];
         }
-        red[tid] = re;
-        red[THREADS + tid] = im;
+        red[tid] = acc;
         __syncthreads();
         for (int st = THREADS / 2; st >= 1; st >>= 1) {
-            if (tid < st) {
-                red[tid] += red[tid + st];
-                red[THREADS + tid] += red[THREADS + tid + st];
-            }
+            if (tid < st) red[tid] += red[tid + st];
             __syncthreads();
         }
-        if (tid == 0) d[0] = cmk(red[0], red[THREADS]);
+        if (tid == 0) d[0] = red[0];
     }
     __syncthreads();
 }
 
-// Initial shift state: pi_0 = pi_{-1} = 1, x^k_0 = 0, p^k_0 = r'_0 (projected:
-// u^k = f^T r'_0), rho_0 = r_0^T r'_0.
+// Initial shift state of column c: zeta^k_0 = nu_0, no pivot yet, x^k_0 = 0,
+// q^k_0 = u'_0 / nu_0 (projected: F u'_0 / nu_0).
 __global__ void k_shift_init(DevSystem s, PanelDev p) {
-    extern __shared__ double2 dyn[];
-    __shared__ double red[2 * THREADS];
+    extern __shared__ double dyn_init[];
+    __shared__ double red[THREADS];
     const int c = blockIdx.x, K = p.K;
-    ColState cs = p.col[c];
+    const ColState cs = p.col[c];
     if (!cs.active) return;
     const int nfun = cs.nfun;
-    double2* d = dyn;
+    double* d = dyn_init;
     if (p.proj != PROJ_NONE) eval_functionals(s, p, c, nfun, d, red);
+    const double nu = sqrt(cs.t_new);
+    const double inv_nu = nu > 0.0 ? 1.0 / nu : 0.0;
     for (int k = threadIdx.x; k < K; k += THREADS) {
-        p.pi[(size_t)c * K + k] = cmk(1.0, 0.0);
-        p.pi_prev[(size_t)c * K + k] = cmk(1.0, 0.0);
+        p.zeta[(size_t)c * K + k] = cmk(nu, 0.0);
+        p.pinv[(size_t)c * K + k] = cmk(0.0, 0.0);
         p.conv_iter[(size_t)c * K + k] = -1;
     }
     if (p.proj != PROJ_NONE) {
@@ -1612,23 +1609,25 @@ __global__ void k_shift_init(DevSystem s, PanelDev p) {
             const int k = e / nfun, m = e % nfun;
             const size_t o = ((size_t)c * K + k) * p.M + m;
             p.t[o] = cmk(0.0, 0.0);
-            p.u[o] = d[m];
+            p.u[o] = cmk(d[m] * inv_nu, 0.0);
             if (p.deriv) {
                 p.dt[o] = cmk(0.0, 0.0);
-                p.du[o] = cmk(0.0, 0.0);      // u_0 = F r'_0 does not depend on z_k
+                p.du[o] = cmk(0.0, 0.0);      // q_0 does not depend on z_k
             }
         }
     }
     if (p.deriv)
         for (int k = threadIdx.x; k < K; k += THREADS) {
-            p.dpi[(size_t)c * K + k] = cmk(0.0, 0.0);
-            p.dpi_prev[(size_t)c * K + k] = cmk(0.0, 0.0);
+            p.dzeta[(size_t)c * K + k] = cmk(0.0, 0.0);
+            p.dpinv[(size_t)c * K + k] = cmk(0.0, 0.0);
         }
     __syncthreads();
     if (threadIdx.x == 0) {
-        cs.rho = cs.rho_new;
-        cs.n_unconv = K;
-        p.col[c] = cs;
+        ColState& out = p.col[c];
+        out.t = cs.t_new;
+        out.nu = nu;
+        out.inv_nu = inv_nu;
+        out.n_unconv = K;
         atomicAdd(&p.flags[2], 1);
     }
 }
@@ -1636,47 +1635,99 @@ __global__ void k_shift_init(DevSystem s, PanelDev p) {
 __global__ void k_full_init(PanelDev p) {
     const long long per = (long long)p.npad * p.P;
     const long long items = per * p.K;
+    const double* Rp = reinterpret_cast<const double*>(p.Rp);
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
         p.X[idx] = cmk(0.0, 0.0);
-        p.Pk[idx] = p.Rp[idx % per];
+        p.Pk[idx] = cmk(Rp[idx % per] * p.col[idx % p.P].inv_nu, 0.0);
     }
 }
 
+// Shift k of a column at outer step n: the pivot of the tridiagonal z_k - T,
+//     D_n = z_k - a_n - B_n^2 / D_{n-1},
+// the step's coefficients alpha = zeta_n / D_n and l = B_{n+1} / D_n, and
+// zeta_{n+1} = l zeta_n, |zeta_{n+1}| ||u^_{n+1}|| being the residual of
+// shift k (the collinear residual of Eq. collinear): the COCG iterates of
+// shift k for whatever seed, with one complex division per shift and step.
+// Im D_n has the sign of Im z_k and at least its size, so no pivot vanishes
+// off the real axis.
+struct ShiftCoef {
+    double2 inv, al, l, zeta;
+};
+__device__ __forceinline__ ShiftCoef shift_coef(double2 z, double sigma, double asig, double B, double Bn,
+                                                double2 pinv, double2 zeta) {
+    const double B2 = B * B;
+    const double2 D = cmk((z.x - sigma) - asig - B2 * pinv.x, z.y - B2 * pinv.y);
+    ShiftCoef c;
+    const double den = D.x * D.x + D.y * D.y;
+    const double id = 1.0 / den;
+    c.inv = cmk(D.x * id, -D.y * id);
+    c.al = cmul(zeta, c.inv);
+    c.l = cmk(Bn * c.inv.x, Bn * c.inv.y);
+    c.zeta = cmk(Bn * c.al.x, Bn * c.al.y);
+    return c;
+}
+
+// End of a column's shift step (one thread): the next step's scalars, the
+// column's activity, and the seed switch.
+__device__ void shift_step_finish(const PanelDev& p, int c, const ColState& cs, int n_unconv, int worst, double nu,
+                                  double inv_nu, double Bn) {
+    ColState out = cs;
+    const int K = p.K;
+    out.iters = cs.iters + 1;
+    out.n_unconv = n_unconv;
+    if (n_unconv == 0) out.active = 0;
+    out.t = cs.t_new;
+    out.nu_prev = cs.nu;
+    out.nu = nu;
+    out.inv_nu = inv_nu;
+    out.B = Bn;
+    if (out.active && p.switching) {
+        const bool seed_conv = p.conv_iter[(size_t)c * K + cs.seed] >= 0;
+        const bool forced = p.force_switch_every > 0 && (out.iters % p.force_switch_every == 0);
+        if ((seed_conv || forced) && worst < K && worst != cs.seed) {
+            out.seed = worst;
+            out.sigma = p.z[worst].x;
+            out.switches += 1;
+        }
+    }
+    out.sinv = p.pinv[(size_t)c * K + out.seed];
+    p.col[c] = out;
+    if (out.active) atomicAdd(&p.flags[2], 1);
+}
+
 // ---------------------------------------------------------------------------
-// a5 + a6: every shift of column c in one pass (Eq. shift:pi, Eq. collinear),
-// projected updates, convergence, and seed switching on the device.
+// a5 + a6: every shift of column c in one pass, projected updates,
+// convergence, and seed switching on the device.  The seed shift (initially
+// opts->seed, then the unconverged shift of the largest residual once the
+// seed has converged) sets sigma of the next steps and the breakdown test;
+// the shifts' own recurrences do not depend on it.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(THREADS) k_shift_step(DevSystem s, PanelDev p) {
     extern __shared__ double2 dyn[];
-    __shared__ double red[2 * THREADS];
+    __shared__ double red[THREADS];
     __shared__ int s_cnt[THREADS];
     __shared__ double s_best[THREADS];
     __shared__ int s_bestk[THREADS];
-    __shared__ int s_sw;
-    __shared__ double2 s_c1, s_c0;
     const int c = blockIdx.x, K = p.K, tid = threadIdx.x;
     const ColState cs = p.col[c];
     if (!cs.active) {
         if (p.proj == PROJ_NONE)
-            for (int k = tid; k < K; k += THREADS) p.ipi[(size_t)c * K + k] = cmk(0.0, 0.0);
+            for (int k = tid; k < K; k += THREADS) p.ak[(size_t)c * K + k] = cmk(0.0, 0.0);
         return;
     }
     const int nfun = cs.nfun;
-    double2* d = dyn;                       // [M]
-    double2* sak = d + p.M;                 // [K]
-    double2* sbk = sak + K;                 // [K]
-    double2* sip = sbk + K;                 // [K]
-    double2* sdak = sip + K;                // [K] derivative mode: d alpha^k, d beta^k, d (1/pi^k)
+    double2* sak = dyn;                     // [K] alpha^k
+    double2* sbk = sak + K;                 // [K] l^k
+    double2* sdak = sbk + K;                // [K] derivative mode: d alpha^k, d l^k
     double2* sdbk = sdak + K;
-    double2* sdip = sdbk + K;
+    double* d = reinterpret_cast<double*>(dyn + (p.deriv ? 4 : 2) * (size_t)K);   // [M]
     if (p.proj != PROJ_NONE) eval_functionals(s, p, c, nfun, d, red);
 
-    const double2 one = cmk(1.0, 0.0);
-    const double2 alpha = cs.alpha;
-    const double2 beta = cdiv(cs.rho_new, cs.rho);
-    const double2 c2 = cdiv(cmul(cs.beta_prev, alpha), cs.alpha_prev);
-    const double rnorm = cs.rnorm;
+    const double nu = sqrt(cs.t_new);
+    const double inv_nu = nu > 0.0 ? 1.0 / nu : 0.0;
+    const double Bn = cs.s * nu;                                   // B_{n+1}
+    const double rhat = nu > 0.0 ? cs.rnorm * inv_nu : 0.0;        // ||u^_{n+1}||
     const int it = cs.iters;
     int nunc = 0;
     double best = -1.0;
@@ -1684,40 +1735,33 @@ __global__ void __launch_bounds__(THREADS) k_shift_step(DevSystem s, PanelDev p)
     for (int k = tid; k < K; k += THREADS) {
         const size_t o = (size_t)c * K + k;
         if (p.conv_iter[o] >= 0) {
-            sip[k] = cmk(0.0, 0.0);
-            if (p.proj == PROJ_NONE) p.ipi[o] = cmk(0.0, 0.0);
+            sak[k] = cmk(0.0, 0.0);
+            if (p.proj == PROJ_NONE) p.ak[o] = cmk(0.0, 0.0);
             continue;
         }
-        const double2 pk = p.pi[o], pp = p.pi_prev[o];
-        const double2 dl = csub(p.z[k], cs.zs);
-        const double2 pin = cadd(cmul(cadd(one, cmul(alpha, dl)), pk), cmul(c2, csub(pk, pp)));
-        const double2 ratio = cdiv(pk, pin);
-        const double2 ak = cmul(alpha, ratio);
-        const double2 bk = cmul(beta, cmul(ratio, ratio));
-        const double2 ip = cdiv(one, pin);
-        const double res = rnorm / cabs2(pin);
-        p.pi_prev[o] = pk;
-        p.pi[o] = pin;
+        const double2 pinv = p.pinv[o], zeta = p.zeta[o];
+        const ShiftCoef f = shift_coef(p.z[k], cs.sigma, cs.asig, cs.B, Bn, pinv, zeta);
+        const double res = sqrt(f.zeta.x * f.zeta.x + f.zeta.y * f.zeta.y) * rhat;
+        p.pinv[o] = f.inv;
+        p.zeta[o] = f.zeta;
         if (p.deriv) {
-            // d/dz_k with the seed quantities fixed (d Delta_k / d z_k = 1)
-            const double2 dpk = p.dpi[o], dpp = p.dpi_prev[o];
-            const double2 dpin = cadd(cadd(cmul(alpha, pk), cmul(cadd(one, cmul(alpha, dl)), dpk)),
-                                      cmul(c2, csub(dpk, dpp)));
-            const double2 ip2 = cmul(ip, ip);
-            const double2 num = cmul(csub(cmul(dpk, pin), cmul(pk, dpin)), ip2);
-            sdak[k] = cmul(alpha, num);
-            sdbk[k] = cmul(cmk(2.0 * beta.x, 2.0 * beta.y), cmul(ratio, num));
-            sdip[k] = cmk(-cmul(dpin, ip2).x, -cmul(dpin, ip2).y);
-            p.dpi_prev[o] = dpk;
-            p.dpi[o] = dpin;
+            // d/dz_k: dD_n = 1 - B_n^2 d(1/D_{n-1})
+            const double2 dp = p.dpinv[o], dz = p.dzeta[o];
+            const double B2 = cs.B * cs.B;
+            const double2 dD = cmk(1.0 - B2 * dp.x, -B2 * dp.y);
+            const double2 i2 = cmul(f.inv, f.inv), id = cmul(i2, dD);
+            const double2 dinv = cmk(-id.x, -id.y);
+            const double2 dal = cadd(cmul(zeta, dinv), cmul(dz, f.inv));
+            sdak[k] = dal;
+            sdbk[k] = cmk(Bn * dinv.x, Bn * dinv.y);
+            p.dpinv[o] = dinv;
+            p.dzeta[o] = cmk(Bn * dal.x, Bn * dal.y);
         }
-        sak[k] = ak;
-        sbk[k] = bk;
-        sip[k] = ip;
+        sak[k] = f.al;
+        sbk[k] = f.l;
         if (p.proj == PROJ_NONE) {
-            p.ak[o] = ak;
-            p.bk[o] = bk;
-            p.ipi[o] = ip;
+            p.ak[o] = f.al;
+            p.bk[o] = f.l;
         }
         if (res <= p.tol) {
             p.conv_iter[o] = it + 1;
@@ -1730,17 +1774,18 @@ __global__ void __launch_bounds__(THREADS) k_shift_step(DevSystem s, PanelDev p)
     if (p.proj != PROJ_NONE) {
         for (int e = tid; e < K * nfun; e += THREADS) {
             const int k = e / nfun, m = e % nfun;
-            const double2 ip = sip[k];
-            if (ip.x == 0.0 && ip.y == 0.0) continue;
+            const double2 al = sak[k];
+            if (al.x == 0.0 && al.y == 0.0) continue;
             const size_t o = ((size_t)c * K + k) * p.M + m;
             const double2 u = p.u[o];
+            const double2 un = cmul(sbk[k], u);
             if (p.deriv) {
                 const double2 du = p.du[o];
-                p.dt[o] = cadd(p.dt[o], cadd(cmul(sdak[k], u), cmul(sak[k], du)));
-                p.du[o] = cadd(cadd(cmul(d[m], sdip[k]), cmul(sdbk[k], u)), cmul(sbk[k], du));
+                p.dt[o] = cadd(p.dt[o], cadd(cmul(sdak[k], u), cmul(al, du)));
+                p.du[o] = cadd(cmul(sdbk[k], u), cmul(sbk[k], du));
             }
-            p.t[o] = cadd(p.t[o], cmul(sak[k], u));
-            p.u[o] = cadd(cmul(d[m], ip), cmul(sbk[k], u));
+            p.t[o] = cadd(p.t[o], cmul(al, u));
+            p.u[o] = cmk(d[m] * inv_nu + un.x, un.y);
         }
     }
     // block reductions: number of unconverged shifts, worst residual (ties -> lowest k)
@@ -1760,71 +1805,26 @@ __global__ void __launch_bounds__(THREADS) k_shift_step(DevSystem s, PanelDev p)
         }
         __syncthreads();
     }
-    if (tid == 0) {
-        ColState out = cs;
-        out.iters = it + 1;
-        out.n_unconv = s_cnt[0];
-        if (out.n_unconv == 0) out.active = 0;
-        int sw = 0;
-        const int s2 = s_bestk[0];
-        if (out.active && p.switching) {
-            const bool seed_conv = p.conv_iter[(size_t)c * K + cs.seed] >= 0;
-            const bool forced = p.force_switch_every > 0 && ((it + 1) % p.force_switch_every == 0);
-            if ((seed_conv || forced) && s2 < K && s2 != cs.seed) sw = 1;
-        }
-        if (sw) {
-            const double2 c1 = p.pi[(size_t)c * K + s2], c0 = p.pi_prev[(size_t)c * K + s2];
-            out.rho = cdiv(cs.rho_new, cmul(c1, c1));
-            out.alpha_prev = sak[s2];
-            out.beta_prev = sbk[s2];
-            out.sc_cur = cdiv(one, c1);
-            out.sc_prev = cdiv(one, c0);
-            out.zs = p.z[s2];
-            out.seed = s2;
-            out.switches += 1;
-            s_c1 = c1;
-            s_c0 = c0;
-        } else {
-            out.rho = cs.rho_new;
-            out.alpha_prev = alpha;
-            out.beta_prev = beta;
-            out.sc_cur = one;
-            out.sc_prev = one;
-        }
-        s_sw = sw;
-        p.col[c] = out;
-        if (out.active) atomicAdd(&p.flags[2], 1);
-    }
-    __syncthreads();
-    if (s_sw) {
-        const double2 c1 = s_c1, c0 = s_c0;
-        for (int k = tid; k < K; k += THREADS) {
-            const size_t o = (size_t)c * K + k;
-            p.pi[o] = cdiv(p.pi[o], c1);
-            p.pi_prev[o] = cdiv(p.pi_prev[o], c0);
-            if (p.deriv) {
-                p.dpi[o] = cdiv(p.dpi[o], c1);
-                p.dpi_prev[o] = cdiv(p.dpi_prev[o], c0);
-            }
-        }
-    }
+    if (tid == 0) shift_step_finish(p, c, cs, s_cnt[0], s_bestk[0], nu, inv_nu, Bn);
 }
 
-// Full mode: x^k += alpha^k p^k, p^k = r'_{n+1}/pi^k_{n+1} + beta^k p^k.
+// Full mode: x^k += alpha^k q^k, q^k = u'_{n+1} / nu_{n+1} + l^k q^k.
 __global__ void k_full_update(PanelDev p) {
     const int P = p.P;
     const long long per = (long long)p.npad * P;
     const long long items = per * p.K;
+    const double* Rp = reinterpret_cast<const double*>(p.Rp);
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
         const int c = (int)(idx % P);
         const int k = (int)(idx / per);
         const size_t o = (size_t)c * p.K + k;
-        const double2 ip = p.ipi[o];
-        if (ip.x == 0.0 && ip.y == 0.0) continue;
-        const double2 pk = p.Pk[idx];
-        p.X[idx] = cadd(p.X[idx], cmul(p.ak[o], pk));
-        p.Pk[idx] = cadd(cmul(p.Rp[idx % per], ip), cmul(p.bk[o], pk));
+        const double2 al = p.ak[o];
+        if (al.x == 0.0 && al.y == 0.0) continue;
+        const double2 q = p.Pk[idx];
+        const double2 qn = cmul(p.bk[o], q);
+        p.X[idx] = cadd(p.X[idx], cmul(al, q));
+        p.Pk[idx] = cmk(Rp[idx % per] * p.col[c].inv_nu + qn.x, qn.y);
     }
 }
 
@@ -2013,44 +2013,53 @@ __global__ void k_mulliken_output(PanelDev p, int ncols, const double2* __restri
 // Generalized Lanczos helpers (Section 3.2), one real vector stored in the
 // real part of a P = 1 panel column.
 // ---------------------------------------------------------------------------
-// Generalized Lanczos on a panel of P columns (Section 3.2), one
-// independent process per column; vectors [npad][P], real parts only.
+// Generalized Lanczos on a panel of P columns (Section 3.2), one independent
+// process per column; vectors [npad][C] pairs of columns.
 // y = M x for M = H or S
 __global__ void k_lz_spmv(DevSystem s, const double* __restrict__ M, const double2* __restrict__ x,
-                          double2* __restrict__ y, int P) {
-    const long long items = (long long)s.n_atoms * P;
+                          double2* __restrict__ y, int C) {
+    const long long items = (long long)s.n_atoms * C;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * blockDim.x) {
-        const int I = (int)(idx / P), c = (int)(idx % P);
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        const int I = (int)(idx / C), c = (int)(idx % C);
+        double2 acc[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) acc[a] = make_double2(0.0, 0.0);
         for (int b = s.brow[I]; b < s.brow[I + 1]; ++b) {
             const int J = s.bcol[b];
-            double xv[4];
+            double2 xv[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xv[e] = x[(size_t)(4 * J + e) * P + c].x;
+            for (int e = 0; e < 4; ++e) xv[e] = x[(size_t)(4 * J + e) * C + c];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) acc[a] += M[16 * (size_t)b + 4 * a + e] * xv[e];
+                for (int e = 0; e < 4; ++e) {
+                    const double m = M[16 * (size_t)b + 4 * a + e];
+                    acc[a].x += m * xv[e].x;
+                    acc[a].y += m * xv[e].y;
+                }
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) y[(size_t)(4 * I + a) * P + c] = cmk(acc[a], 0.0);
+        for (int a = 0; a < 4; ++a) y[(size_t)(4 * I + a) * C + c] = acc[a];
     }
 }
 
-// out[c * stride] = x_c^T y_c (mode 0) or sqrt(x_c^T y_c) (mode 1)
+// out[c * stride] = x_c^T y_c (mode 0) or sqrt(x_c^T y_c) (mode 1) for column c < P
 __global__ void __launch_bounds__(THREADS) k_lz_dot(PanelDev p, const double2* __restrict__ x,
                                                     const double2* __restrict__ y, double* out, int stride, int mode) {
-    __shared__ double smem[THREADS];
-    const int P = p.P;
-    double v[1] = {0.0};
-    const long long items = (long long)p.npad * P;
-    for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS)
-        v[0] += x[i].x * y[i].x;
-    if (grid_reduce_cols<1>(v, P, p, smem)) {
-        if (threadIdx.x < P) {
-            const double t = smem[threadIdx.x];
-            out[(size_t)threadIdx.x * stride] = (mode == 0) ? t : sqrt(fmax(t, 0.0));
+    __shared__ double smem[2 * THREADS];
+    const int C = p.C;
+    double v[2] = {0.0, 0.0};
+    const long long items = (long long)p.npad * C;
+    for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
+        const double2 a = x[i], b = y[i];
+        v[0] += a.x * b.x;
+        v[1] += a.y * b.y;
+    }
+    if (grid_reduce_cols<2>(v, C, p, smem)) {
+        for (int c = threadIdx.x; c < p.P; c += THREADS) {
+            const double t = smem[(c & 1) * THREADS + (c >> 1)];
+            out[(size_t)c * stride] = (mode == 0) ? t : sqrt(fmax(t, 0.0));
         }
     }
 }
@@ -2058,16 +2067,18 @@ __global__ void __launch_bounds__(THREADS) k_lz_dot(PanelDev p, const double2* _
 // u_c = v_c / sqrt(n2_c), n2_c = v[row_c][c] = e_j^T S^-1 e_j (inactive columns: u = 0)
 __global__ void k_lz_start(PanelDev p, const double2* __restrict__ v, double2* __restrict__ u, double* nrm2) {
     const int P = p.P;
+    const double* vv = reinterpret_cast<const double*>(v);
+    double* uu = reinterpret_cast<double*>(u);
     const long long items = (long long)p.npad * P;
     for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
         const int c = (int)(i % P);
         const ColState& cs = p.col[c];
         if (!cs.active) {
-            u[i] = cmk(0.0, 0.0);
+            uu[i] = 0.0;
             continue;
         }
-        const double n2 = v[(size_t)cs.row * P + c].x;
-        u[i] = cmk(v[i].x / sqrt(n2), 0.0);
+        const double n2 = vv[(size_t)cs.row * P + c];
+        uu[i] = vv[i] / sqrt(n2);
         if (i / P == 0) nrm2[c] = n2;
     }
 }
@@ -2076,23 +2087,27 @@ __global__ void k_lz_start(PanelDev p, const double2* __restrict__ v, double2* _
 __global__ void k_lz_combine(PanelDev p, const double2* __restrict__ y, const double2* __restrict__ u,
                              const double2* __restrict__ up, double2* __restrict__ w, const double* a,
                              const double* b, int sa, int sb) {
-    const int P = p.P;
-    const long long items = (long long)p.npad * P;
+    const int C = p.C;
+    const long long items = (long long)p.npad * C;
     for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
-        const int c = (int)(i % P);
-        w[i] = cmk(y[i].x - a[(size_t)c * sa] * u[i].x - b[(size_t)c * sb] * up[i].x, 0.0);
+        const int c = 2 * (int)(i % C);
+        const double2 yv = y[i], uv = u[i], pv = up[i];
+        w[i] = make_double2(yv.x - a[(size_t)c * sa] * uv.x - b[(size_t)c * sb] * pv.x,
+                            yv.y - a[(size_t)(c + 1) * sa] * uv.y - b[(size_t)(c + 1) * sb] * pv.y);
     }
 }
 
 // u_prev = u, u = w / b_c (0 when b_c = 0: invariant subspace found)
 __global__ void k_lz_scale(PanelDev p, const double2* __restrict__ w, double2* __restrict__ u,
                            double2* __restrict__ up, const double* bnext, int sb) {
-    const int P = p.P;
-    const long long items = (long long)p.npad * P;
+    const int C = p.C;
+    const long long items = (long long)p.npad * C;
     for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
-        const double bv = bnext[(size_t)(i % P) * sb];
+        const int c = 2 * (int)(i % C);
+        const double b0 = bnext[(size_t)c * sb], b1 = bnext[(size_t)(c + 1) * sb];
+        const double2 wv = w[i];
         up[i] = u[i];
-        u[i] = cmk(bv > 0.0 ? w[i].x / bv : 0.0, 0.0);
+        u[i] = make_double2(b0 > 0.0 ? wv.x / b0 : 0.0, b1 > 0.0 ? wv.y / b1 : 0.0);
     }
 }
 
@@ -2322,9 +2337,8 @@ __global__ void k_panel_rhs(PanelDev p, const double* __restrict__ rhs, const in
     for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
         const int c = (int)(i / n_orb), o = (int)(i % n_orb);
         const size_t e = (size_t)orb2pad[o] * p.P + c;
-        const double2 v = cmk(rhs[i], 0.0);
-        p.Rcur[e] = v;
-        p.Rin[e] = v;
+        reinterpret_cast<double*>(p.Rcur)[e] = rhs[i];
+        reinterpret_cast<double*>(p.Rin)[e] = rhs[i];
     }
 }
 
@@ -2680,73 +2694,64 @@ void launch_ased_build(const DevSystem& s, const double* eps_pad, double K, cuda
 void launch_panel_init(const DevSystem&, const PanelDev& p, cudaStream_t st) {
     {
         LaunchScope ls_(K_OTHER, st);
-        k_panel_init<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p);
+        k_panel_init<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p);
     }
 }
-void launch_outer_spmm(const DevSystem& s, const PanelDev& p, bool sx_from_residual, cudaStream_t st) {
-    {
-        LaunchScope ls_(K_OUTER_SPMM, st);
-        const bool rag = s.rag && g_df_rag;
-        if (p.mixed && sx_from_residual && rag)
-            k_outer_spmm<true, true, true><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p);
-        else if (p.mixed && sx_from_residual)
-            k_outer_spmm<true, true><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p);
-        else if (p.mixed && rag)
-            k_outer_spmm<true, false, true><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p);
-        else if (p.mixed)
-            k_outer_spmm<true><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p);
-        else
-            k_outer_spmm<false><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p);
-    }
+void launch_outer_spmm(const DevSystem& s, const PanelDev& p, cudaStream_t st) {
+    LaunchScope ls_(K_OUTER_SPMM, st);
+    const int g = grid_for((long long)s.n_atoms * p.C);
+    if (p.mixed && s.rag && g_df_rag) k_outer_spmm<true, true><<<g, THREADS, 0, st>>>(s, p);
+    else if (p.mixed) k_outer_spmm<true><<<g, THREADS, 0, st>>>(s, p);
+    else k_outer_spmm<false><<<g, THREADS, 0, st>>>(s, p);
 }
 void launch_outer_update(const DevSystem&, const PanelDev& p, cudaStream_t st) {
     {
         LaunchScope ls_(K_OUTER_UPDATE, st);
-        k_outer_update<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p);
+        k_outer_update<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p);
     }
 }
 void launch_inner_spmv(const DevSystem& s, const PanelDev& p, int it, cudaStream_t st) {
     {
         LaunchScope ls_(K_INNER_SPMV, st);
-        k_inner_spmv<<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p, it);
+        k_inner_spmv<<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, it);
     }
 }
 void launch_inner_update(const DevSystem&, const PanelDev& p, int it, cudaStream_t st) {
     {
         LaunchScope ls_(K_INNER_UPDATE, st);
-        k_inner_update<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, it);
+        k_inner_update<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, it);
     }
 }
 void launch_finish(const DevSystem&, const PanelDev& p, cudaStream_t st) {
     {
         LaunchScope ls_(K_FINISH, st);
-        k_finish<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p);
+        k_finish<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p);
     }
 }
 void launch_refine_start(const DevSystem&, const PanelDev& p, const double2* b, cudaStream_t st) {
     LaunchScope ls_(K_REFINE_AUX, st);
-    k_refine_start<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, b);
+    k_refine_start<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, b);
 }
 void launch_refine_residual(const DevSystem& s, const PanelDev& p, const double2* b, cudaStream_t st, bool fp64) {
     LaunchScope ls_(K_REFINE_RESIDUAL, st);
     if (fp64)   // FP64 products; columns already within inner_tol exit at once
-        k_refine_residual<false><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p, b);
+        k_refine_residual<false><<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, b);
     else if (s.rag && g_df_rag)
-        k_refine_residual<true, true><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p, b);
+        k_refine_residual<true, true><<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, b);
     else
-        k_refine_residual<true><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p, b);
+        k_refine_residual<true><<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, b);
 }
 void launch_refine_scale(const DevSystem&, const PanelDev& p, const double2* src, float cheb_gamma, cudaStream_t st) {
     LaunchScope ls_(K_REFINE_AUX, st);
-    k_refine_scale<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, src, cheb_gamma);
+    k_refine_scale<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, src, cheb_gamma);
 }
 void launch_split_panel(const PanelDev& p, cudaStream_t st) {
     LaunchScope ls_(K_REFINE_AUX, st);
-    k_split_panel<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p);
+    k_split_panel<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p);
 }
 void launch_refine_add(const DevSystem&, const PanelDev& p, cudaStream_t st) {
     LaunchScope ls_(K_REFINE_AUX, st);
-    k_refine_add<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p);
+    k_refine_add<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p);
 }
 size_t inner32_grp_smem(const DevSystem& s) {
     const size_t xregion = (size_t)s.max_union * 4 * PC * sizeof(float2);
@@ -2759,7 +2764,7 @@ void launch_inner32_spmv(const DevSystem& s, const PanelDev& p, int it, cudaStre
     // the grouped form wins on narrow panels (measured on the Si 4096-atom
     // system: 28 vs 35 us at 64 columns); from 128 columns on, the
     // register-gather form with its higher occupancy is faster
-    if (s.grpG > 0 && p.P >= PC && p.P <= 64) {
+    if (s.grpG > 0 && p.C >= PC && p.C <= 64) {
         const size_t sm = inner32_grp_smem(s);
         static const bool attr = [] {
             // the dynamic limit leaves room for the kernel's static shared memory
@@ -2771,11 +2776,10 @@ void launch_inner32_spmv(const DevSystem& s, const PanelDev& p, int it, cudaStre
                        cudaSuccess;
         }();
         (void)attr;
-        k_inner32_spmv_grp<<<s.n_groups * (p.P / PC), s.grpG * (PC / 2), sm, st>>>(s, p, it);
-    } else if (p.P >= 2) {
-        const int g = grid_for((long long)s.n_atoms * (p.P / 2));
-        switch (p.P) {
-            case 256: k_inner32_spmv<2, 256><<<g, THREADS, 0, st>>>(s, p, it); break;
+        k_inner32_spmv_grp<<<s.n_groups * (p.C / PC), s.grpG * (PC / 2), sm, st>>>(s, p, it);
+    } else if (p.C >= 2) {
+        const int g = grid_for((long long)s.n_atoms * (p.C / 2));
+        switch (p.C) {
             case 128: k_inner32_spmv<2, 128><<<g, THREADS, 0, st>>>(s, p, it); break;
             case 64: k_inner32_spmv<2, 64><<<g, THREADS, 0, st>>>(s, p, it); break;
             case 32: k_inner32_spmv<2, 32><<<g, THREADS, 0, st>>>(s, p, it); break;
@@ -2786,10 +2790,10 @@ void launch_inner32_spmv(const DevSystem& s, const PanelDev& p, int it, cudaStre
         }
     }
     else
-        k_inner32_spmv<1><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p, it);
+        k_inner32_spmv<1><<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, it);
 }
-// TB_CHEB_CPT=2 / 4 forces the two- or four-columns-per-thread form of the
-// Chebyshev step (panels narrower than 4 columns always take the two-column
+// TB_CHEB_CPT=2 / 4 forces the two- or four-pairs-per-thread form of the
+// Chebyshev step (panels narrower than 8 columns always take the two-pair
 // form); tb_autotune's choice for the call's size class comes first
 static const int g_cheb_cpt_env = [] {
     const char* e = std::getenv("TB_CHEB_CPT");
@@ -2805,19 +2809,17 @@ static const bool g_cheb_rag = [] {
 template <bool LAST>
 static void cheb4_launch(const DevSystem& s, const PanelDev& p, const float2* cur, float2* io, float omega,
                          float gamma, int mode, cudaStream_t st) {
-    const int g = std::min(grid_for((long long)s.n_atoms * (p.P / 4)), 3 * (gmax() / 4));
+    const int g = std::min(grid_for((long long)s.n_atoms * (p.C / 4)), 3 * (gmax() / 4));
     if (s.rag && g_cheb_rag) {
-        switch (p.P) {
-            case 256: k_inner32_cheb4r<256, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
-            case 128: k_inner32_cheb4r<128, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+        switch (p.C) {
+                case 128: k_inner32_cheb4r<128, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 64: k_inner32_cheb4r<64, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             default: k_inner32_cheb4r<0, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
         }
         return;
     }
-    switch (p.P) {
-        case 256: k_inner32_cheb4<256, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
-        case 128: k_inner32_cheb4<128, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+    switch (p.C) {
+            case 128: k_inner32_cheb4<128, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
         case 64: k_inner32_cheb4<64, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
         default: k_inner32_cheb4<0, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
     }
@@ -2826,23 +2828,22 @@ static void cheb4_launch(const DevSystem& s, const PanelDev& p, const float2* cu
 template <bool LAST>
 static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur, float2* io, float omega,
                         float gamma, int mode, cudaStream_t st) {
-    // default form: four columns per thread (measured best on the silicon
+    // default form: four pairs per thread (measured best on the silicon
     // benchmark and on ragged water batches, whose concurrent systems fill
     // the GPU; a small system solved alone runs faster with two, which
     // tb_autotune finds for its size class), two for narrow panels
-    // (measured on the 100 000-atom crystal: at 4 and 8 columns per panel the
-    // two-column form's twice as many threads win, 61 / 69 against 93 /
-    // 100 us per step; from 16 columns on, four columns per thread)
-    const int cpt = p.cheb_cpt ? p.cheb_cpt : g_cheb_cpt_env ? g_cheb_cpt_env : (p.P >= 16 ? 4 : 2);
-    if (cpt == 4 && p.P >= 4) {
+    // (measured on the 100 000-atom crystal: at 4 and 8 pairs per panel the
+    // two-pair form's twice as many threads win, 61 / 69 against 93 /
+    // 100 us per step; from 16 pairs on, four per thread)
+    const int cpt = p.cheb_cpt ? p.cheb_cpt : g_cheb_cpt_env ? g_cheb_cpt_env : (p.C >= 16 ? 4 : 2);
+    if (cpt == 4 && p.C >= 4) {
         cheb4_launch<LAST>(s, p, cur, io, omega, gamma, mode, st);
         return;
     }
 
-    if (p.P >= 2) {
-        const int g = grid_for((long long)s.n_atoms * (p.P / 2));
-        switch (p.P) {
-            case 256: k_inner32_cheb<2, 256, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+    if (p.C >= 2) {
+        const int g = grid_for((long long)s.n_atoms * (p.C / 2));
+        switch (p.C) {
             case 128: k_inner32_cheb<2, 128, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 64: k_inner32_cheb<2, 64, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 32: k_inner32_cheb<2, 32, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
@@ -2852,7 +2853,7 @@ static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur
             default: k_inner32_cheb<2, 0, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
         }
     } else {
-        k_inner32_cheb<1, 0, LAST><<<grid_for((long long)s.n_atoms * p.P), THREADS, 0, st>>>(s, p, cur, io, omega,
+        k_inner32_cheb<1, 0, LAST><<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, cur, io, omega,
                                                                                           gamma, mode);
     }
 }
@@ -2907,13 +2908,13 @@ void cheb_graph_destroy(cudaGraphExec_t g) {
 }
 void launch_inner32_update(const DevSystem&, const PanelDev& p, int it, cudaStream_t st) {
     LaunchScope ls_(K_INNER32_UPDATE, st);
-    if (p.P >= 2)
-        k_inner32_update<2><<<grid_for((long long)p.npad * p.P / 2), THREADS, 0, st>>>(p, it);
+    if (p.C >= 2)
+        k_inner32_update<2><<<grid_for((long long)p.npad * p.C / 2), THREADS, 0, st>>>(p, it);
     else
-        k_inner32_update<1><<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, it);
+        k_inner32_update<1><<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, it);
 }
 static size_t shift_smem(const PanelDev& p) {
-    return sizeof(double2) * ((size_t)(p.M > 0 ? p.M : 1) + (p.deriv ? 6 : 3) * (size_t)p.K);
+    return sizeof(double) * (size_t)(p.M > 0 ? p.M : 1) + sizeof(double2) * (p.deriv ? 4 : 2) * (size_t)p.K;
 }
 void launch_shift_init(const DevSystem& s, const PanelDev& p, cudaStream_t st) {
     const size_t sm = shift_smem(p);
@@ -2991,28 +2992,28 @@ void launch_mulliken_output(const PanelDev& p, int ncols, const double2* w, doub
         k_mulliken_output<<<p.P, THREADS, 0, st>>>(p, ncols, w, g_s, out);
     }
 }
-void launch_lz_spmv(const DevSystem& s, const double* M, const double2* x, double2* y, int P, cudaStream_t st) {
+void launch_lz_spmv(const DevSystem& s, const double* M, const double2* x, double2* y, int C, cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_spmv<<<grid_for((long long)s.n_atoms * P), THREADS, 0, st>>>(s, M, x, y, P);
+    k_lz_spmv<<<grid_for((long long)s.n_atoms * C), THREADS, 0, st>>>(s, M, x, y, C);
 }
 void launch_lz_dot(const PanelDev& p, const double2* x, const double2* y, double* out, int stride, int mode,
                    cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_dot<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, x, y, out, stride, mode);
+    k_lz_dot<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, x, y, out, stride, mode);
 }
 void launch_lz_combine(const PanelDev& p, const double2* y, double2* u, double2* u_prev, double2* w,
                        const double* a, const double* b, int sa, int sb, cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_combine<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, y, u, u_prev, w, a, b, sa, sb);
+    k_lz_combine<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, y, u, u_prev, w, a, b, sa, sb);
 }
 void launch_lz_scale(const PanelDev& p, double2* w, double2* u, double2* u_prev, const double* bnext, int sb,
                      cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_scale<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, w, u, u_prev, bnext, sb);
+    k_lz_scale<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, w, u, u_prev, bnext, sb);
 }
 void launch_lz_start(const PanelDev& p, const double2* v, double2* u, double* nrm2, cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_start<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, v, u, nrm2);
+    k_lz_start<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, v, u, nrm2);
 }
 
 
