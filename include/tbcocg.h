@@ -573,7 +573,9 @@ enum {
                               update, atom sums, mixing                        */
     TB_K_INNER32_CHEB = 13, /* TB_MIXED: one Chebyshev correction step (FP32
                               S d and the update of d in one kernel)          */
-    TB_K_COUNT = 14
+    TB_K_SLICE = 14,       /* whole outer steps of a slice of columns of a small
+                              system (one launch runs several steps)          */
+    TB_K_COUNT = 15
 };
 /*
  * FMA throughput of the current device, measured (no counterpart in the

@@ -28,6 +28,9 @@ namespace tb {
 int max_grid();
 }
 
+// orbitals of the largest system that the column slices take
+constexpr int64_t SLICE_MAX_ROWS = 2304;
+
 struct tb_handle {
     DevSystem ds;
     int device = 0;
@@ -60,6 +63,9 @@ struct tb_handle {
     int32_t* orb2pad_local = nullptr;      // device copy
     int32_t* bcol_local = nullptr;         // device [nb]: block column local to its system
     int* row_order_local = nullptr;        // device [n_atoms]: per system, its block-row order (local indices)
+    // small systems: their rows as the column slices take them, one per system
+    // of the handle (tb_create: one; a batch: one per system)
+    std::vector<SliceDev> slices;
     int* flags_pool = nullptr;             // pinned [NPOOL][NFLAGS]: status words of the worker threads
     // tb_autotune's choices, per size class (precision, correction method,
     // shift count rounded up to a power of two)
@@ -175,7 +181,8 @@ struct Solve {
     double* q_out = nullptr;            // srow, per column
     // launch choices (0: the handle's tuned value, else the default)
     int streams = 0;                    // panels in flight
-    int cheb_cpt = 0;                   // columns per thread of the Chebyshev step
+    int cheb_cpt = 0;                   // pairs of columns per thread of the Chebyshev step
+    int inflight = 1;                   // panels of the call solved at the same time
 };
 
 // What one solve sees of a system: the device arrays (a whole handle, or one
@@ -189,6 +196,7 @@ struct View {
     int64_t n_orb = 0;
     int* flags_host = nullptr;        // pinned [NFLAGS]
     tb_handle* owner = nullptr;       // the handle the view belongs to
+    const SliceDev* slice = nullptr;  // its rows for the column slices (nullptr: none)
 };
 
 tb_status check_opts(const tb_solve_opts* o) {
@@ -794,6 +802,24 @@ bool step_graph_build(View& v, PanelDev& p, InnerCtx& ic, int proj, int inner_ma
     return true;
 }
 
+// TB_SLICE=0 in the environment keeps small systems on the panel kernels
+static bool slices_on() {
+    const char* e = std::getenv("TB_SLICE");
+    return !(e && std::atoi(e) == 0);
+}
+// outer steps per slice launch: the host looks at the columns after each
+constexpr int SLICE_STEPS = 32;
+
+int sm_count() {
+    static const int n = [] {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        return sms > 0 ? sms : 1;
+    }();
+    return n;
+}
+
 tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* stats, cudaStream_t st) {
     const auto t0 = std::chrono::steady_clock::now();
     const int K = q.K, R = q.R;
@@ -877,6 +903,37 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     StepGraph sg;
     tb_status final_status = TB_OK;
 
+    // small systems: whole outer steps of a few columns per cluster
+    // (tb_slice.cu), on the mixed path with Chebyshev corrections and in FP64
+    SliceArgs sa;
+    bool slices = false;
+    if (slices_on() && !g_trace && v.slice && v.slice->noct > 0 && M <= 256 &&
+        (!p.mixed || (ic.cheb.n > 0 && ic.cheb.n <= 512))) {
+        slices = slice_choose(*v.slice, p, ic.cheb.n, std::min(P, R), std::max(1, sm_count() / std::max(1, q.inflight)), sa);
+        if (slices) {
+            sa.inner_max = o->inner_max_iter;
+            sa.inner_tol = o->inner_tol;
+            if (p.mixed) {
+                float* om = nullptr;
+                if ((s = dalloc(cl, &om, (size_t)ic.cheb.n)) != TB_OK) return s;
+                TB_CK(cudaMemcpyAsync(om, ic.cheb.omega.data(), sizeof(float) * ic.cheb.n, cudaMemcpyHostToDevice, st));
+                sa.omega = om;
+                sa.n = ic.cheb.n;
+                sa.n_last = ic.cheb.n_last;
+                sa.R = ic.cheb.R;
+                sa.gamma = ic.cheb.gamma;
+            }
+            if (q.proj != PROJ_NONE) {
+                if ((s = dalloc(cl, &p.ak, (size_t)P * K)) != TB_OK) return s;
+                if ((s = dalloc(cl, &p.bk, (size_t)P * K)) != TB_OK) return s;
+            }
+            if (p.deriv) {
+                if ((s = dalloc(cl, &sa.dak, (size_t)P * K)) != TB_OK) return s;
+                if ((s = dalloc(cl, &sa.dbk, (size_t)P * K)) != TB_OK) return s;
+            }
+        }
+    }
+
     for (int c0 = 0; c0 < R; c0 += P) {
         const int ncols = std::min(P, R - c0);
         for (int c = 0; c < P; ++c) {
@@ -907,63 +964,102 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
         if (q.proj == PROJ_ROWS)
             TB_CK(cudaMemcpyAsync(p.frow, frowh.data(), sizeof(int32_t) * P * M, cudaMemcpyHostToDevice, st));
 
-        // r_0 = e_j, r'_0 = S^-1 r_0, rho_0, pi = 1, x^k = 0, p^k = r'_0
+        // u_0 = e_j (or the given right-hand side)
         launch_panel_init(v.ds, p, st);
         if (q.rhs) launch_panel_rhs(p, q.rhs + (size_t)c0 * v.n_orb, v.o2p_d, (int)v.n_orb, ncols, st);
-        if ((s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st)) != TB_OK) return s;
-        if (v.flags_host[0] & ERR_NOT_SPD) return TB_ERR_S_NOT_SPD;
-        launch_finish(v.ds, p, st);
-        launch_shift_init(v.ds, p, st);
-        TB_CK(cudaGetLastError());
-
-        // step n: the end of step n-1 (rho, the shift step, full-mode
-        // update: the "tail"), the seed SpMM and r_{n+1}, the inner solve;
-        // then the host reads how many columns are still active.  On the
-        // mixed path with Chebyshev corrections a step after the first is
-        // one replay of the panel's step graph.
-        int active = ncols;
-        bool tail_pending = false;
-        for (int n = 0; n < o->max_iter; ++n) {
-            const bool use_graph = tail_pending && g_graphs && g_step_graphs && !g_trace && p.mixed &&
-                                   ic.cheb.n > 0 && ic.cheb.chebyshev(ic.rounds - 1) && !sg.failed;
-            if (use_graph && (!sg.exec || sg.rounds != ic.rounds))
-                step_graph_build(v, p, ic, q.proj, o->inner_max_iter, sg);
-            if (use_graph && sg.exec) {
-                graph_prof_launched(sg.prof);
-                TB_CK(cudaGraphLaunch(sg.exec, st));
+        bool sliced = false;
+        if (slices) {
+            int64_t inner_steps = 0;
+            int active = ncols;
+            sliced = true;
+            for (int n = 0; n < o->max_iter && active > 0; n += SLICE_STEPS) {
+                sa.start = n == 0 ? 1 : 0;
+                sa.nsteps = std::min(SLICE_STEPS, o->max_iter - n);
+                TB_CK(cudaMemsetAsync(p.flags + 2, 0, 2 * sizeof(int), st));   // active columns, inner steps
+                if (!launch_slice(*v.slice, v.ds, p, sa, ncols, st)) {
+                    sliced = false;
+                    break;
+                }
+                TB_CK(cudaMemcpyAsync(v.flags_host, p.flags, NFLAGS * sizeof(int), cudaMemcpyDeviceToHost, st));
                 TB_CK(cudaStreamSynchronize(st));
                 prof_harvest();
-                ic.total += sg.inner_steps;
-                // the planned rounds ran: what the inner solve does after its
-                // host check (redo in FP64 after a non-finite residual, more
-                // rounds while some real column is above inner_tol)
-                if (v.flags_host[0] & ERR_INNER) s = inner_redo(v, p, p.Rcur, o->inner_max_iter, ic, st);
-                else if (v.flags_host[4] > 0) s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st, ic.rounds);
-                else s = TB_OK;
-                if (s != TB_OK) return s;
-            } else {
-                if (tail_pending) {
-                    launch_finish(v.ds, p, st);
-                    launch_shift_step(v.ds, p, st);
-                    if (q.proj == PROJ_NONE) launch_full_update(v.ds, p, st);
+                inner_steps += v.flags_host[3];
+                active = v.flags_host[2];
+                if (v.flags_host[0] & ERR_INNER) {   // an inner solve that needs more than its planned rounds
+                    sliced = false;
+                    break;
                 }
-                launch_outer_spmm(v.ds, p, st);
-                launch_outer_update(v.ds, p, st);
-                s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st);
-                if (s != TB_OK) return s;
             }
-            tail_pending = false;
-            active = v.flags_host[2];     // columns still active after step n-1
-            errbits |= v.flags_host[0];
-            if (errbits & ERR_NOT_SPD) return TB_ERR_S_NOT_SPD;
-            if (active == 0) break;
-            tail_pending = true;
+            if (sliced) {
+                ic.total += inner_steps;
+                errbits |= v.flags_host[0];
+            } else {
+                // the panel again from its start by the panel kernels, whose
+                // inner solve has further rounds, FP32 CG and the FP64 CG; the
+                // rest of the call stays with them
+                slices = false;
+                TB_CK(cudaMemcpyAsync(p.col, colh.data(), sizeof(ColState) * P, cudaMemcpyHostToDevice, st));
+                TB_CK(cudaMemsetAsync(p.flags, 0, sizeof(int) * NFLAGS, st));
+                launch_panel_init(v.ds, p, st);
+                if (q.rhs) launch_panel_rhs(p, q.rhs + (size_t)c0 * v.n_orb, v.o2p_d, (int)v.n_orb, ncols, st);
+            }
         }
-        if (tail_pending) {   // max_iter ran out: the last step's tail
+        if (!sliced) {
+            if ((s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st)) != TB_OK) return s;
+            if (v.flags_host[0] & ERR_NOT_SPD) return TB_ERR_S_NOT_SPD;
             launch_finish(v.ds, p, st);
-            launch_shift_step(v.ds, p, st);
-            if (q.proj == PROJ_NONE) launch_full_update(v.ds, p, st);
+            launch_shift_init(v.ds, p, st);
             TB_CK(cudaGetLastError());
+
+            // step n: the end of step n-1 (rho, the shift step, full-mode
+            // update: the "tail"), the seed SpMM and r_{n+1}, the inner solve;
+            // then the host reads how many columns are still active.  On the
+            // mixed path with Chebyshev corrections a step after the first is
+            // one replay of the panel's step graph.
+            int active = ncols;
+            bool tail_pending = false;
+            for (int n = 0; n < o->max_iter; ++n) {
+                const bool use_graph = tail_pending && g_graphs && g_step_graphs && !g_trace && p.mixed &&
+                                       ic.cheb.n > 0 && ic.cheb.chebyshev(ic.rounds - 1) && !sg.failed;
+                if (use_graph && (!sg.exec || sg.rounds != ic.rounds))
+                    step_graph_build(v, p, ic, q.proj, o->inner_max_iter, sg);
+                if (use_graph && sg.exec) {
+                    graph_prof_launched(sg.prof);
+                    TB_CK(cudaGraphLaunch(sg.exec, st));
+                    TB_CK(cudaStreamSynchronize(st));
+                    prof_harvest();
+                    ic.total += sg.inner_steps;
+                    // the planned rounds ran: what the inner solve does after its
+                    // host check (redo in FP64 after a non-finite residual, more
+                    // rounds while some real column is above inner_tol)
+                    if (v.flags_host[0] & ERR_INNER) s = inner_redo(v, p, p.Rcur, o->inner_max_iter, ic, st);
+                    else if (v.flags_host[4] > 0) s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st, ic.rounds);
+                    else s = TB_OK;
+                    if (s != TB_OK) return s;
+                } else {
+                    if (tail_pending) {
+                        launch_finish(v.ds, p, st);
+                        launch_shift_step(v.ds, p, st);
+                        if (q.proj == PROJ_NONE) launch_full_update(v.ds, p, st);
+                    }
+                    launch_outer_spmm(v.ds, p, st);
+                    launch_outer_update(v.ds, p, st);
+                    s = inner_solve(v, p, p.Rcur, o->inner_max_iter, ic, st);
+                    if (s != TB_OK) return s;
+                }
+                tail_pending = false;
+                active = v.flags_host[2];     // columns still active after step n-1
+                errbits |= v.flags_host[0];
+                if (errbits & ERR_NOT_SPD) return TB_ERR_S_NOT_SPD;
+                if (active == 0) break;
+                tail_pending = true;
+            }
+            if (tail_pending) {   // max_iter ran out: the last step's tail
+                launch_finish(v.ds, p, st);
+                launch_shift_step(v.ds, p, st);
+                if (q.proj == PROJ_NONE) launch_full_update(v.ds, p, st);
+                TB_CK(cudaGetLastError());
+            }
         }
         // outputs of this panel
         if (q.proj == PROJ_NONE)
@@ -1016,6 +1112,7 @@ View whole_view(tb_handle* h) {
     v.n_orb = h->n_orb;
     v.flags_host = h->flags_host;
     v.owner = h;
+    if (h->sys_ds.empty() && h->slices.size() == 1) v.slice = &h->slices[0];
     return v;
 }
 
@@ -1095,6 +1192,7 @@ tb_status run_jobs(tb_handle* h, const Solve& q, const tb_solve_opts* o, tb_stat
                     v.o2p_h = h->orb2pad_local_h.data() + orb0;
                     v.o2p_d = h->orb2pad_local + orb0;
                     v.n_orb = Nq;
+                    v.slice = sys < (int)h->slices.size() ? &h->slices[sys] : nullptr;
                 }
                 v.flags_host = h->flags_pool + (size_t)NFLAGS * wid;
                 std::vector<int32_t> cols(Rq), pos(Rq);
@@ -1104,6 +1202,7 @@ tb_status run_jobs(tb_handle* h, const Solve& q, const tb_solve_opts* o, tb_stat
                 }
                 Solve q2 = q;
                 q2.R = Rq;
+                q2.inflight = nw;
                 q2.cols = cols.data();
                 std::vector<int64_t> rp2, gidx;
                 std::vector<int32_t> rows2;
@@ -1336,6 +1435,14 @@ SpmvGroups build_spmv_groups(const std::vector<int>& brow, const std::vector<int
 
 namespace {
 
+// The slices' copies of H after ds.H changed.
+void refill_slices_H(tb_handle* h, cudaStream_t st) {
+    for (SliceDev& d : h->slices)
+        if (d.noct > 0)
+            launch_slice_fill(h->ds.H, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64),
+                              reinterpret_cast<float*>(d.Hhi), reinterpret_cast<float*>(d.Hlo), st);
+}
+
 // Keep the Hamiltonian of tb_create before the first charge-dependent one
 // replaces it.
 tb_status ensure_H0(tb_handle* h, cudaStream_t st) {
@@ -1505,13 +1612,73 @@ tb_status tb_destroy(tb_handle* h) {
     cudaFree(h->H0);
     cudaFree(h->orb2pad_local);
     cudaFree(h->bcol_local);
+    for (SliceDev& d : h->slices) {
+        cudaFree(d.oct_ptr);
+        cudaFree(d.idx_ptr);
+        cudaFree(d.row_slot);
+        cudaFree(d.idx);
+        cudaFree(d.src);
+        cudaFree(d.Shi);
+        cudaFree(d.Slo);
+        cudaFree(d.Hhi);
+        cudaFree(d.Hlo);
+        cudaFree(d.S64);
+        cudaFree(d.H64);
+    }
     if (h->flags_pool) cudaFreeHost(h->flags_pool);
     if (h->flags_host) cudaFreeHost(h->flags_host);
     delete h;
     return TB_OK;
 }
 
+// Rows of one system (atoms [a0, a0 + n) of the handle) for the column slices;
+// systems too large for them get an empty entry.
+static cudaError_t add_slice(tb_handle* h, int a0, int n, cudaStream_t st) {
+    h->slices.emplace_back();
+    int64_t rows = 0;
+    for (int i = 0; i < n; ++i) rows += h->orb_per_atom[a0 + i];
+    if (rows > SLICE_MAX_ROWS) return cudaSuccess;
+    SliceHost hs;
+    slice_layout(n, h->orb_per_atom.data() + a0, h->brow_h.data() + a0, h->bcol_h.data(), a0, hs);
+    if (hs.nrows > 65535) return cudaSuccess;
+    SliceDev& d = h->slices.back();
+    const size_t ni = (size_t)hs.oct_ptr.back() * 8;
+    cudaError_t e;
+    auto up = [&](auto** dst, const void* srcp, size_t bytes) {
+        if ((e = cudaMalloc(reinterpret_cast<void**>(dst), std::max<size_t>(bytes, 16))) != cudaSuccess) return e;
+        return srcp && bytes ? cudaMemcpyAsync(*dst, srcp, bytes, cudaMemcpyHostToDevice, st) : cudaSuccess;
+    };
+    if ((e = up(&d.oct_ptr, hs.oct_ptr.data(), sizeof(int) * hs.oct_ptr.size())) != cudaSuccess) return e;
+    if ((e = up(&d.idx_ptr, hs.idx_ptr.data(), sizeof(int) * hs.idx_ptr.size())) != cudaSuccess) return e;
+    if ((e = up(&d.row_slot, hs.row_slot.data(), sizeof(int) * hs.row_slot.size())) != cudaSuccess) return e;
+    if ((e = up(&d.idx, hs.idx.data(), sizeof(unsigned short) * hs.idx.size())) != cudaSuccess) return e;
+    if ((e = up(&d.src, hs.src.data(), sizeof(int) * hs.src.size())) != cudaSuccess) return e;
+    if ((e = up(&d.Shi, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
+    if ((e = up(&d.Slo, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
+    if ((e = up(&d.Hhi, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
+    if ((e = up(&d.Hlo, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
+    if ((e = up(&d.S64, nullptr, 2 * sizeof(double2) * ni)) != cudaSuccess) return e;
+    if ((e = up(&d.H64, nullptr, 2 * sizeof(double2) * ni)) != cudaSuccess) return e;
+    d.n_items = (long long)ni;
+    launch_slice_fill(h->ds.S, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.S64), reinterpret_cast<float*>(d.Shi),
+                      reinterpret_cast<float*>(d.Slo), st);
+    launch_slice_fill(h->ds.H, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64), reinterpret_cast<float*>(d.Hhi),
+                      reinterpret_cast<float*>(d.Hlo), st);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;   // the host arrays are released here
+    d.nrows = hs.nrows;
+    d.noct = hs.noct;
+    d.unit_diag = h->ds.unit_diag;
+    return cudaSuccess;
+}
+
+static tb_status create_system(tb_handle** out, const tb_system_desc* d, void* stream, bool with_slices);
+
 tb_status tb_create(tb_handle** out, const tb_system_desc* d, void* stream) {
+    return create_system(out, d, stream, true);
+}
+
+static tb_status create_system(tb_handle** out, const tb_system_desc* d, void* stream, bool with_slices) {
     if (!out) return TB_ERR_INVALID_ARG;
     *out = nullptr;
     if (!d || d->n_atoms < 1 || !d->orb_per_atom || !d->brow_ptr || !d->bcol || !d->S_vals) return TB_ERR_INVALID_ARG;
@@ -1745,6 +1912,7 @@ tb_status tb_create(tb_handle** out, const tb_system_desc* d, void* stream) {
     if (noalloc_scratch(h->device, &h->noalloc_base) != TB_OK) return fail(cudaErrorUnknown);
     h->sys_atom_off = {0, (int64_t)n};
     h->sys_orb_off = {0, N};
+    if (with_slices && (e = add_slice(h, 0, n, st)) != cudaSuccess) return fail(e);
     *out = h;
     return TB_OK;
 }
@@ -1802,7 +1970,7 @@ tb_status tb_create_batch(tb_handle** out, const tb_system_desc* descs, int32_t 
     m.eps = h_given ? nullptr : eps.data();
     m.K = descs[0].K;
     m.precision = TB_FP64;
-    const tb_status s = tb_create(out, &m, stream);
+    const tb_status s = create_system(out, &m, stream, n_systems == 1);
     if (s != TB_OK) return s;
     tb_handle* h = *out;
     h->sys_atom_off = aoff;
@@ -1866,6 +2034,8 @@ tb_status tb_create_batch(tb_handle** out, const tb_system_desc* descs, int32_t 
         v.grpG = 0;                 // the grouped SpMV's atom groups are built for the whole handle
         h->sys_ds.push_back(v);
     }
+    for (int q = 0; q < n_systems; ++q)
+        if ((e = add_slice(h, (int)aoff[q], (int)(aoff[q + 1] - aoff[q]), st)) != cudaSuccess) return fail(e);
     h->ds.rag = 0;
     return TB_OK;
 }
@@ -2446,6 +2616,7 @@ tb_status tb_csc_hamiltonian(tb_handle* h, const double* gamma, const double* dq
         if (h->H0) {
             TB_CK(cudaMemcpyAsync(h->ds.H, h->H0, sizeof(double) * 16 * (size_t)h->ds.nb, cudaMemcpyDeviceToDevice, st));
             launch_split_f64(h->ds.H, h->ds.H32hi, h->ds.H32lo, 16 * (long long)h->ds.nb, st);
+            refill_slices_H(h, st);
             TB_CK(cudaGetLastError());
         }
         TB_CK(cudaStreamSynchronize(st));
@@ -2464,6 +2635,7 @@ tb_status tb_csc_hamiltonian(tb_handle* h, const double* gamma, const double* dq
     if ((s = dalloc(cl, &V, (size_t)n)) != TB_OK) return s;
     launch_csc_potential(gd, dqd, n, V, st);
     launch_csc_hamiltonian(h->ds, h->H0, V, st);
+    refill_slices_H(h, st);
     TB_CK(cudaGetLastError());
     TB_CK(cudaStreamSynchronize(st));
     return TB_OK;
@@ -2577,6 +2749,7 @@ tb_status tb_csc_loop(tb_handle* h, int32_t K, const double* z, const double* w,
     for (m = 1; m <= copts->max_scf; ++m) {
         launch_csc_potential(gd, dq_in, n, V, st);
         launch_csc_hamiltonian(h->ds, h->H0, V, st);
+        refill_slices_H(h, st);
         TB_CK(cudaGetLastError());
         tb_stats ts{};
         const tb_status run = mulliken_atoms_device(h, K, z, w, g_s, opts, q, &ts, st);

@@ -75,6 +75,37 @@ struct DevSystem {
     int* grp_cols = nullptr;   // distinct block-column atoms of each group, ascending
     int* blk_loc = nullptr;    // [nb] position of bcol[b] in the list of its group
 };
+// A small system's rows as the column slices consume them (tb_slice.cu):
+// eight streams per octet, the items of an octet interleaved step by step.
+struct SliceDev {
+    int nrows = 0, noct = 0;        // rows (8 per octet), octets; 0: the system takes no slices
+    int unit_diag = 0;              // as DevSystem::unit_diag
+    int* oct_ptr = nullptr;         // [noct + 1] first step of every octet (item = step * 8 + stream)
+    int* idx_ptr = nullptr;         // [noct + 1] first batch of four indices of every octet
+    int* row_slot = nullptr;        // [nrows] padded orbital slot of a row, -1: filling
+    ushort4* idx = nullptr;         // [batches][8] gathered rows of the items of steps 1, 2, ...
+    int* src = nullptr;             // [items][4] offsets of the coefficients in S and H, -1: zero
+    float4 *Shi = nullptr, *Slo = nullptr, *Hhi = nullptr, *Hlo = nullptr;   // [items]
+    double2 *S64 = nullptr, *H64 = nullptr;                                  // [items][2]
+    long long n_items = 0;
+};
+struct SliceHost {
+    int nrows = 0, noct = 0;
+    std::vector<int> oct_ptr, idx_ptr, row_slot, src;
+    std::vector<unsigned short> idx;
+};
+// Arguments of one slice launch: up to nsteps outer steps of every column
+struct SliceArgs {
+    int nc = 0, cl = 1;             // columns per slice, CTAs per cluster
+    int nsteps = 0, start = 0;      // start: the inner solve of u_0 and the shifts' first state come first
+    int n = 0, n_last = 0, R = 0;   // mixed: Chebyshev plan
+    float gamma = 0.f;
+    const float* omega = nullptr;   // device [n]
+    int inner_max = 0;              // FP64: CG iterations of an inner solve, at most
+    double inner_tol = 0.0;
+    double2 *dak = nullptr, *dbk = nullptr;   // [P][K] d/dz_k of alpha^k and l^k of a step (derivative mode)
+};
+
 size_t inner32_grp_smem(const DevSystem& s);   // dynamic shared memory of the grouped SpMV
 
 // Per right-hand side (column) state of a panel.  The Krylov vectors are real
@@ -163,7 +194,10 @@ struct PanelDev {
 // of the public header)
 enum { K_INNER_SPMV = 0, K_INNER_UPDATE, K_OUTER_SPMM, K_OUTER_UPDATE, K_FINISH, K_SHIFT_STEP,
        K_FULL_UPDATE, K_OTHER, K_INNER32_SPMV, K_INNER32_UPDATE, K_REFINE_RESIDUAL, K_REFINE_AUX, K_CSC, K_INNER32_CHEB,
-       K_COUNT };
+       K_SLICE, K_COUNT };
+// one counted (and, with timing on, timed) launch made outside tb_kernels.cu: begin, launch, end
+void* launch_mark_begin(int id, cudaStream_t st);
+void launch_mark_end(void* mark);
 void profile_enable(bool on);
 void prof_harvest();
 // launch accounting of a captured graph: the event pairs recorded by its
@@ -181,6 +215,13 @@ void graph_prof_release(GraphProf& gp);
 void profile_read(int id, int64_t* launches, double* ms);
 double profile_busy(int id);
 int64_t launch_count();
+
+// ---- column slices (tb_slice.cu) -------------------------------------------
+void slice_layout(int n, const int32_t* orb, const int64_t* brow, const int32_t* bcol, int32_t col0, SliceHost& out);
+bool slice_choose(const SliceDev& ss, const PanelDev& p, int n_omega, int ncols, int sms, SliceArgs& a);
+bool launch_slice(const SliceDev& ss, const DevSystem& s, const PanelDev& p, const SliceArgs& a, int ncols,
+                  cudaStream_t st);
+void launch_slice_fill(const double* M, const int* src, long long n, double* m64, float* hi, float* lo, cudaStream_t st);
 
 // ---- launchers (tb_kernels.cu) -------------------------------------------
 bool preload_noalloc_kernels();   // loads the allocation-free call's kernels onto the current device

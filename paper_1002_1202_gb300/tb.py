@@ -169,7 +169,8 @@ SIGNATURES = [
 
 KERNELS = {"inner_spmv": 0, "inner_update": 1, "outer_spmm": 2, "outer_update": 3, "finish": 4,
            "shift_step": 5, "full_update": 6, "other": 7, "inner32_spmv": 8, "inner32_update": 9,
-           "refine_residual": 10, "refine_aux": 11, "csc": 12, "inner32_cheb": 13}
+           "refine_residual": 10, "refine_aux": 11, "csc": 12, "inner32_cheb": 13,
+           "slice": 14}
 
 _lib = None
 
