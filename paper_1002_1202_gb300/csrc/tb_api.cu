@@ -2818,7 +2818,9 @@ tb_status tb_generalized_lanczos_batch(tb_handle* h, int32_t R, const int32_t* c
     if ((s = check_cols(h, R, cols)) != TB_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int npad = h->ds.npad;
-    const int P = std::max(2, std::min(opts->panel ? opts->panel : 64, next_pow2(R)));
+    // one panel at a time: as wide as a panel can be unless the caller says
+    // otherwise (128 columns x 24 steps of 1728 atoms: 24.9 ms as one panel, 40.0 as two)
+    const int P = std::max(2, std::min(opts->panel ? opts->panel : MAX_P, next_pow2(R)));
     Cleanup cl_out;
     cl_out.st = st;
     OutBuf oa, ob, on;

@@ -2731,14 +2731,18 @@ static void cheb4_launch(const DevSystem& s, const PanelDev& p, const float2* cu
 template <bool LAST>
 static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur, float2* io, float omega,
                         float gamma, int mode, cudaStream_t st) {
-    // default form: four pairs per thread (measured best on the silicon
-    // benchmark and on ragged water batches, whose concurrent systems fill
-    // the GPU; a small system solved alone runs faster with two, which
-    // tb_autotune finds for its size class), two for narrow panels
-    // (measured on the 100 000-atom crystal: at 4 and 8 pairs per panel the
-    // two-pair form's twice as many threads win, 61 / 69 against 93 /
-    // 100 us per step; from 16 pairs on, four per thread)
-    const int cpt = p.cheb_cpt ? p.cheb_cpt : g_cheb_cpt_env ? g_cheb_cpt_env : (p.C >= 16 ? 4 : 2);
+    // default form: two pairs per thread.  The step is bound by the latency of
+    // its gathers, so the form with twice the threads wins while the panel has
+    // fewer threads than the SMs can hold many times over (panels in pairs,
+    // 64 / 128 / 256 columns: 4096 atoms 159 / 158 / 193 ms per call against
+    // 170 / 169 / 202 with four; 1728 atoms 177 / 174 / 184 against 229 / 215 /
+    // 209; 24 Lanczos steps of 128 columns 40.0 / 24.9 ms against 56.2 / 32.1;
+    // prefetching the next block's rows into registers was slower in every
+    // form: 165-560 ms).  Four pairs for systems with s-only atoms, whose
+    // ragged form has them, and from eight waves of the four-pair form on
+    // (the 100 000-atom crystal from 64 columns on)
+    const bool wide = (s.rag && g_cheb_rag && p.C >= 16) || (long long)s.n_atoms * (p.C / 4) >= 8LL * 3 * (gmax() / 4) * THREADS;
+    const int cpt = p.cheb_cpt ? p.cheb_cpt : g_cheb_cpt_env ? g_cheb_cpt_env : (wide ? 4 : 2);
     if (cpt == 4 && p.C >= 4) {
         cheb4_launch<LAST>(s, p, cur, io, omega, gamma, mode, st);
         return;
