@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <thread>
 #include <vector>
@@ -28,7 +29,9 @@ namespace tb {
 int max_grid();
 }
 
-// orbitals of the largest system that the column slices take
+// orbitals of the largest system that the column slices take: beyond it S no
+// longer stays in the shared memory of a cluster, and the panel kernels are
+// faster (6912 orbitals, 256 columns: 184 ms against 380-610)
 constexpr int64_t SLICE_MAX_ROWS = 2304;
 
 struct tb_handle {
@@ -63,9 +66,10 @@ struct tb_handle {
     int32_t* orb2pad_local = nullptr;      // device copy
     int32_t* bcol_local = nullptr;         // device [nb]: block column local to its system
     int* row_order_local = nullptr;        // device [n_atoms]: per system, its block-row order (local indices)
-    // small systems: their rows as the column slices take them, one per system
-    // of the handle (tb_create: one; a batch: one per system)
-    std::vector<SliceDev> slices;
+    // the rows of every system of the handle as the column slices take them,
+    // one layout per cluster size, built on first use
+    std::mutex slice_mu;
+    std::vector<std::vector<std::unique_ptr<SliceDev>>> slices;
     int* flags_pool = nullptr;             // pinned [NPOOL][NFLAGS]: status words of the worker threads
     // tb_autotune's choices, per size class (precision, correction method,
     // shift count rounded up to a power of two)
@@ -182,7 +186,7 @@ struct Solve {
     // launch choices (0: the handle's tuned value, else the default)
     int streams = 0;                    // panels in flight
     int cheb_cpt = 0;                   // pairs of columns per thread of the Chebyshev step
-    int inflight = 1;                   // panels of the call solved at the same time
+    int columns = 0;                    // columns of the call solved at the same time (0: this solve's)
 };
 
 // What one solve sees of a system: the device arrays (a whole handle, or one
@@ -196,7 +200,7 @@ struct View {
     int64_t n_orb = 0;
     int* flags_host = nullptr;        // pinned [NFLAGS]
     tb_handle* owner = nullptr;       // the handle the view belongs to
-    const SliceDev* slice = nullptr;  // its rows for the column slices (nullptr: none)
+    int sys = -1;                     // system of the handle (-1: a batch seen as one system)
 };
 
 tb_status check_opts(const tb_solve_opts* o) {
@@ -802,6 +806,160 @@ bool step_graph_build(View& v, PanelDev& p, InnerCtx& ic, int proj, int inner_ma
     return true;
 }
 
+void free_slice(SliceDev& d) {
+    void* ptrs[] = {d.rank_oct, d.oct_ptr, d.idx_ptr, d.dest_ptr, d.dest, d.row_slot, d.idx, d.src,
+                    d.Shi, d.Slo, d.Hhi, d.Hlo, d.S64, d.H64};
+    for (void* q : ptrs) cudaFree(q);
+    d = SliceDev();
+}
+
+// The layout of system `sys` of the handle for clusters of cl CTAs, built on
+// first use on stream st (nullptr: not available, e.g. out of memory).
+const SliceDev* get_slice(tb_handle* h, int sys, int cl, cudaStream_t st) {
+    std::lock_guard<std::mutex> lk(h->slice_mu);
+    if ((int)h->slices.size() <= sys) h->slices.resize(sys + 1);
+    for (auto& d : h->slices[sys])
+        if (d->cl == cl) return d->noct > 0 ? d.get() : nullptr;
+    const int a0 = (int)h->sys_atom_off[sys], n = (int)(h->sys_atom_off[sys + 1] - a0);
+    auto dev = std::make_unique<SliceDev>();
+    SliceDev& d = *dev;
+    d.cl = cl;
+    SliceHost hs;
+    slice_layout(n, h->orb_per_atom.data() + a0, h->brow_h.data() + a0, h->bcol_h.data(), a0, cl, hs);
+    const size_t ni = (size_t)hs.oct_ptr.back() * 8;
+    bool ok = hs.nloc <= 65535 && ni * 4 < ((size_t)1 << 31);
+    auto up = [&](auto** dst, const void* srcp, size_t bytes) {
+        if (!ok) return;
+        ok = cudaMalloc(reinterpret_cast<void**>(dst), std::max<size_t>(bytes, 16)) == cudaSuccess &&
+             (!srcp || !bytes || cudaMemcpyAsync(*dst, srcp, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess);
+    };
+    up(&d.rank_oct, hs.rank_oct.data(), sizeof(int) * hs.rank_oct.size());
+    up(&d.oct_ptr, hs.oct_ptr.data(), sizeof(int) * hs.oct_ptr.size());
+    up(&d.idx_ptr, hs.idx_ptr.data(), sizeof(int) * hs.idx_ptr.size());
+    up(&d.dest_ptr, hs.dest_ptr.data(), sizeof(int) * hs.dest_ptr.size());
+    up(&d.dest, hs.dest.data(), sizeof(int) * hs.dest.size());
+    up(&d.row_slot, hs.row_slot.data(), sizeof(int) * hs.row_slot.size());
+    up(&d.idx, hs.idx.data(), sizeof(unsigned short) * hs.idx.size());
+    up(&d.src, hs.src.data(), sizeof(int) * hs.src.size());
+    up(&d.Shi, nullptr, sizeof(float4) * ni);
+    up(&d.Slo, nullptr, sizeof(float4) * ni);
+    up(&d.Hhi, nullptr, sizeof(float4) * ni);
+    up(&d.Hlo, nullptr, sizeof(float4) * ni);
+    up(&d.S64, nullptr, 2 * sizeof(double2) * ni);
+    up(&d.H64, nullptr, 2 * sizeof(double2) * ni);
+    if (ok) {
+        d.n_items = (long long)ni;
+        launch_slice_fill(h->ds.S, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.S64),
+                          reinterpret_cast<float*>(d.Shi), reinterpret_cast<float*>(d.Slo), st);
+        launch_slice_fill(h->ds.H, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64),
+                          reinterpret_cast<float*>(d.Hhi), reinterpret_cast<float*>(d.Hlo), st);
+        ok = cudaGetLastError() == cudaSuccess;
+    }
+    // the host arrays are released here, and other streams use the layout
+    if (cudaStreamSynchronize(st) != cudaSuccess) ok = false;
+    if (!ok) {
+        cudaGetLastError();
+        free_slice(d);
+        d.cl = cl;   // remembered: not tried again
+        h->slices[sys].push_back(std::move(dev));
+        return nullptr;
+    }
+    d.nrows = hs.nrows;
+    d.noct = hs.noct;
+    d.nloc = hs.nloc;
+    d.max_len = hs.max_len;
+    d.max_oct = hs.max_oct;
+    d.max_steps = hs.max_steps;
+    d.max_bat = hs.max_bat;
+    d.max_dest = hs.max_dest;
+    d.unit_diag = h->ds.unit_diag;
+    h->slices[sys].push_back(std::move(dev));
+    return h->slices[sys].back().get();
+}
+
+int sm_count();
+
+// Columns per slice, CTAs per cluster and whether S is kept in registers, for
+// ncols columns solved at the same time, by a model of a slice's outer step in
+// cycles; nullptr: nothing fits.  The
+// constants are measured (64-512 atoms): a warp's item costs 9 cycles of the
+// shared memory with S in registers, 14 / 9 / 5.5 with S there for 2 / 4 / 8
+// columns; the copies of the ring arrive at ~13 bytes per cycle; an item's
+// latency is ~35 cycles; a cluster barrier with the stores into the copies
+// costs 500 + 180 per CTA, __syncthreads ~100; an FP64 CG iteration has ~7500
+// cycles of reductions and scalars; FP64 arithmetic runs at 1.7 FMA per cycle
+// and SM; ~25 000 cycles of an outer step are latencies of its passes.
+const SliceDev* slice_choose(const View& v, const PanelDev& p, int ncols, SliceArgs& a, cudaStream_t st) {
+    tb_handle* h = v.owner;
+    const bool mixed = p.mixed != 0;
+    const double N = (double)v.n_orb;
+    if (N > (double)SLICE_MAX_ROWS) return nullptr;
+    // TB_SLICE_NC, TB_SLICE_CL, TB_SLICE_REG (0 / 1): the choice by hand
+    const char* nc_env = std::getenv("TB_SLICE_NC");
+    const char* cl_env = std::getenv("TB_SLICE_CL");
+    const char* rg_env = std::getenv("TB_SLICE_REG");
+    const int env_nc = nc_env ? std::atoi(nc_env) : 0, env_cl = cl_env ? std::atoi(cl_env) : 0;
+    const int env_reg = rg_env ? std::atoi(rg_env) : -1;
+    const double sms = sm_count();
+    const int64_t a0 = h->sys_atom_off[v.sys], a1 = h->sys_atom_off[v.sys + 1];
+    const double nnz = (double)(h->boff_h[h->brow_h[a1]] - h->boff_h[h->brow_h[a0]]);
+    const double L = nnz / 4 / N * 1.1 + 1;       // items of a stream
+    const double items = N * L;
+    const double inner = mixed ? std::max(1, 2 * a.n) : 45.0;
+    struct Cand {
+        int nc, cl;
+        bool reg;
+        double cost;
+    };
+    std::vector<Cand> cand;
+    std::vector<int> cls = {1, 2, 3, 4, 6, 8};
+    if (env_cl > 0) cls = {std::min(env_cl, 16)};
+    for (int nc : {1, 2, 4, 8}) {
+        if (mixed ? nc < 2 : nc > 4) continue;
+        if (nc > p.P || (env_nc > 0 && nc != std::min(std::max(env_nc, mixed ? 2 : 1), mixed ? 8 : 4))) continue;
+        for (int cl : cls)
+            for (int reg = 0; reg <= (mixed ? 1 : 0); ++reg) {
+                if (mixed && (env_reg == 0 || env_reg == 1) && reg != env_reg) continue;
+                if (env_cl <= 0 && cl > 1 && N < 16.0 * cl) continue;   // at least two octets per CTA
+                const int lps = !mixed ? nc : reg && nc >= 4 ? nc / 4 : nc / 2;
+                const double rows = N / cl, wi = items / cl * lps / 32, threads = std::min(512.0, rows * lps + 31);
+                if (reg && (rows * lps > 540 || L > 24)) continue;
+                const double passes = std::ceil(rows * lps / 512);
+                // shared memory, and so the clusters that run at once
+                const double vec = std::min(N, rows * (1 + 6.0 / std::sqrt(N / 64))) * nc * 8;
+                const double smem = vec + rows * nc * (mixed ? 4 : 32) + 8e3 + threads * (mixed ? 16 : 8) +
+                                    (reg ? 0 : items / cl * (mixed ? 18 : 34));
+                const bool fits = smem < 220e3;
+                const int thr = ((int)threads + 31) / 32 * 32;
+                const double room = slice_clusters(mixed, nc, reg != 0, cl, std::min(thr, 512), (size_t)std::min(smem, 220e3));
+                if (room < 1) continue;
+                const double slices = std::ceil((double)ncols / nc), fill = slices / room;
+                const double waves = fill <= 1.0 ? 1.0 : fill + 0.3 * (std::ceil(fill) - fill);
+                const double load = std::max(1.0, std::min(slices, room) * cl / sms);   // CTAs that share an SM
+                const double bar = cl > 1 ? 500 + 180 * cl : 100;
+                double step, outer;
+                if (mixed) {
+                    const double wf = reg ? 9.0 : nc >= 8 ? 5.5 : nc == 4 ? 9.0 : 14.0;
+                    const double stream = fits ? 0.0 : items / cl * 18 / 13;
+                    step = std::max({load * wi * wf, passes * L * 35 + 250, stream}) + bar;
+                    outer = 15 * bar + load * rows * nc * 60 / 1.7 + 4 * (load * wi * 30 + passes * L * 60) + 25e3;
+                } else {
+                    step = load * items / cl * 4 * nc / 1.7 + passes * L * 160 + 7500 + 2 * bar;
+                    outer = 10 * bar + load * rows * nc * 20 / 1.7 + 25e3;
+                }
+                outer += load * (double)p.K * nc * 60 / cl / 1.7;
+                cand.push_back({nc, cl, reg != 0, waves * (inner * step + outer)});
+            }
+    }
+    std::sort(cand.begin(), cand.end(), [](const Cand& x, const Cand& y) { return x.cost < y.cost; });
+    for (const Cand& c : cand) {
+        const SliceDev* d = get_slice(h, v.sys, c.cl, st);
+        if (!d || d->max_oct == 0) continue;
+        if (slice_fit(*d, p, c.nc, c.reg, a)) return d;
+    }
+    return nullptr;
+}
+
 // TB_SLICE=0 in the environment keeps small systems on the panel kernels
 static bool slices_on() {
     const char* e = std::getenv("TB_SLICE");
@@ -907,9 +1065,12 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     // (tb_slice.cu), on the mixed path with Chebyshev corrections and in FP64
     SliceArgs sa;
     bool slices = false;
-    if (slices_on() && !g_trace && v.slice && v.slice->noct > 0 && M <= 256 &&
+    const SliceDev* sl = nullptr;
+    if (slices_on() && !g_trace && v.owner && v.sys >= 0 && M <= 256 &&
         (!p.mixed || (ic.cheb.n > 0 && ic.cheb.n <= 512))) {
-        slices = slice_choose(*v.slice, p, ic.cheb.n, std::min(P, R), std::max(1, sm_count() / std::max(1, q.inflight)), sa);
+        sa.n = ic.cheb.n;
+        sl = slice_choose(v, p, std::max(std::min(P, R), q.columns), sa, st);
+        slices = sl != nullptr;
         if (slices) {
             sa.inner_max = o->inner_max_iter;
             sa.inner_tol = o->inner_tol;
@@ -918,18 +1079,31 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
                 if ((s = dalloc(cl, &om, (size_t)ic.cheb.n)) != TB_OK) return s;
                 TB_CK(cudaMemcpyAsync(om, ic.cheb.omega.data(), sizeof(float) * ic.cheb.n, cudaMemcpyHostToDevice, st));
                 sa.omega = om;
-                sa.n = ic.cheb.n;
                 sa.n_last = ic.cheb.n_last;
                 sa.R = ic.cheb.R;
                 sa.gamma = ic.cheb.gamma;
             }
-            if (q.proj != PROJ_NONE) {
-                if ((s = dalloc(cl, &p.ak, (size_t)P * K)) != TB_OK) return s;
-                if ((s = dalloc(cl, &p.bk, (size_t)P * K)) != TB_OK) return s;
-            }
-            if (p.deriv) {
-                if ((s = dalloc(cl, &sa.dak, (size_t)P * K)) != TB_OK) return s;
-                if ((s = dalloc(cl, &sa.dbk, (size_t)P * K)) != TB_OK) return s;
+            if (q.proj == PROJ_NONE || M > 1 || p.deriv) {
+                // block mode: up to 512 steps per block (most solves end within
+                // one) as far as 128 MB hold them, at least one launch's
+                SliceBlock& b = sa.blk;
+                b.rows = q.proj == PROJ_NONE ? npad : M;
+                const size_t PK = (size_t)P * K;
+                const double per_step = (double)PK * (p.deriv ? 64 : 32) + (double)P * b.rows * 8;
+                const char* be = std::getenv("TB_SLICE_BLOCK");   // steps per block by hand
+                double len = be && std::atoi(be) > 0 ? std::atoi(be) : std::min(512.0, 134217728.0 / per_step);
+                len = std::min(len, (double)(o->max_iter + SLICE_STEPS - 1));
+                b.len = (int)len / SLICE_STEPS * SLICE_STEPS;
+                if (b.len < SLICE_STEPS) {
+                    slices = false;
+                } else {
+                    if ((s = dalloc(cl, &b.A, PK * b.len)) != TB_OK) return s;
+                    if ((s = dalloc(cl, &b.L, PK * b.len)) != TB_OK) return s;
+                    if (p.deriv && (s = dalloc(cl, &b.dA, PK * b.len)) != TB_OK) return s;
+                    if (p.deriv && (s = dalloc(cl, &b.dL, PK * b.len)) != TB_OK) return s;
+                    if ((s = dalloc(cl, &b.D, (size_t)P * b.rows * (b.len + 1))) != TB_OK) return s;
+                    if ((s = dalloc(cl, &b.count, PK)) != TB_OK) return s;
+                }
             }
         }
     }
@@ -972,11 +1146,18 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
             int64_t inner_steps = 0;
             int active = ncols;
             sliced = true;
+            int blk0 = 0;         // outer step at which the present block began
+            sa.blk.step = 0;
             for (int n = 0; n < o->max_iter && active > 0; n += SLICE_STEPS) {
                 sa.start = n == 0 ? 1 : 0;
                 sa.nsteps = std::min(SLICE_STEPS, o->max_iter - n);
+                if (sa.blk.D && n - blk0 >= sa.blk.len) {
+                    launch_block_flush(p, sa.blk, n - blk0, blk0, true, st);
+                    blk0 = n;
+                }
+                sa.blk.step = n - blk0;
                 TB_CK(cudaMemsetAsync(p.flags + 2, 0, 2 * sizeof(int), st));   // active columns, inner steps
-                if (!launch_slice(*v.slice, v.ds, p, sa, ncols, st)) {
+                if (!launch_slice(*sl, v.ds, p, sa, ncols, st)) {
                     sliced = false;
                     break;
                 }
@@ -991,6 +1172,8 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
                 }
             }
             if (sliced) {
+                if (sa.blk.D) launch_block_flush(p, sa.blk, sa.blk.len, blk0, false, st);
+                TB_CK(cudaGetLastError());
                 ic.total += inner_steps;
                 errbits |= v.flags_host[0];
             } else {
@@ -1112,7 +1295,7 @@ View whole_view(tb_handle* h) {
     v.n_orb = h->n_orb;
     v.flags_host = h->flags_host;
     v.owner = h;
-    if (h->sys_ds.empty() && h->slices.size() == 1) v.slice = &h->slices[0];
+    if (h->sys_ds.empty()) v.sys = 0;
     return v;
 }
 
@@ -1192,7 +1375,7 @@ tb_status run_jobs(tb_handle* h, const Solve& q, const tb_solve_opts* o, tb_stat
                     v.o2p_h = h->orb2pad_local_h.data() + orb0;
                     v.o2p_d = h->orb2pad_local + orb0;
                     v.n_orb = Nq;
-                    v.slice = sys < (int)h->slices.size() ? &h->slices[sys] : nullptr;
+                    v.sys = sys;
                 }
                 v.flags_host = h->flags_pool + (size_t)NFLAGS * wid;
                 std::vector<int32_t> cols(Rq), pos(Rq);
@@ -1202,7 +1385,7 @@ tb_status run_jobs(tb_handle* h, const Solve& q, const tb_solve_opts* o, tb_stat
                 }
                 Solve q2 = q;
                 q2.R = Rq;
-                q2.inflight = nw;
+                q2.columns = std::min(R, nw * (int)jobs[0].cols.size());
                 q2.cols = cols.data();
                 std::vector<int64_t> rp2, gidx;
                 std::vector<int32_t> rows2;
@@ -1312,6 +1495,13 @@ int workers_for(const tb_handle* h) {
     return h->sys_ds.empty() ? 4 : 8;
 }
 
+// Whether every system of the handle is small enough for the column slices.
+bool slice_system(const tb_handle* h) {
+    for (size_t s = 0; s + 1 < h->sys_orb_off.size(); ++s)
+        if (h->sys_orb_off[s + 1] - h->sys_orb_off[s] > SLICE_MAX_ROWS) return false;
+    return true;
+}
+
 // The tuned choices of this handle for a call (nullptr: none).
 const tb_handle::Tuned* tuned_for(tb_handle* h, const tb_solve_opts* o, int K) {
     std::lock_guard<std::mutex> lk(h->tune_mu);
@@ -1328,6 +1518,10 @@ tb_status run_solve(tb_handle* h, const Solve& q0, const tb_solve_opts* o, tb_st
     tb_solve_opts oe = *o;
     const tb_handle::Tuned* t = o->panel == 0 ? tuned_for(h, o, q.K) : nullptr;
     if (t) oe.panel = t->panel;
+    // systems that the column slices take: panels as wide as they can be, so
+    // that all slices run at once (288 columns of a 144-atom water box: five
+    // panels of 64 on four streams took two rounds)
+    else if (o->panel == 0 && slices_on() && slice_system(h)) oe.panel = MAX_P;
     if (q.cheb_cpt == 0 && t) q.cheb_cpt = t->cpt;
     const int nw = q.streams ? q.streams : (t ? t->streams : workers_for(h));
     const int Pw = std::min(oe.panel ? oe.panel : 64, next_pow2(q.R));
@@ -1437,10 +1631,12 @@ namespace {
 
 // The slices' copies of H after ds.H changed.
 void refill_slices_H(tb_handle* h, cudaStream_t st) {
-    for (SliceDev& d : h->slices)
-        if (d.noct > 0)
-            launch_slice_fill(h->ds.H, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64),
-                              reinterpret_cast<float*>(d.Hhi), reinterpret_cast<float*>(d.Hlo), st);
+    std::lock_guard<std::mutex> lk(h->slice_mu);
+    for (auto& list : h->slices)
+        for (auto& d : list)
+            if (d->noct > 0)
+                launch_slice_fill(h->ds.H, d->src, 4 * d->n_items, reinterpret_cast<double*>(d->H64),
+                                  reinterpret_cast<float*>(d->Hhi), reinterpret_cast<float*>(d->Hlo), st);
 }
 
 // Keep the Hamiltonian of tb_create before the first charge-dependent one
@@ -1612,73 +1808,15 @@ tb_status tb_destroy(tb_handle* h) {
     cudaFree(h->H0);
     cudaFree(h->orb2pad_local);
     cudaFree(h->bcol_local);
-    for (SliceDev& d : h->slices) {
-        cudaFree(d.oct_ptr);
-        cudaFree(d.idx_ptr);
-        cudaFree(d.row_slot);
-        cudaFree(d.idx);
-        cudaFree(d.src);
-        cudaFree(d.Shi);
-        cudaFree(d.Slo);
-        cudaFree(d.Hhi);
-        cudaFree(d.Hlo);
-        cudaFree(d.S64);
-        cudaFree(d.H64);
-    }
+    for (auto& list : h->slices)
+        for (auto& d : list) free_slice(*d);
     if (h->flags_pool) cudaFreeHost(h->flags_pool);
     if (h->flags_host) cudaFreeHost(h->flags_host);
     delete h;
     return TB_OK;
 }
 
-// Rows of one system (atoms [a0, a0 + n) of the handle) for the column slices;
-// systems too large for them get an empty entry.
-static cudaError_t add_slice(tb_handle* h, int a0, int n, cudaStream_t st) {
-    h->slices.emplace_back();
-    int64_t rows = 0;
-    for (int i = 0; i < n; ++i) rows += h->orb_per_atom[a0 + i];
-    if (rows > SLICE_MAX_ROWS) return cudaSuccess;
-    SliceHost hs;
-    slice_layout(n, h->orb_per_atom.data() + a0, h->brow_h.data() + a0, h->bcol_h.data(), a0, hs);
-    if (hs.nrows > 65535) return cudaSuccess;
-    SliceDev& d = h->slices.back();
-    const size_t ni = (size_t)hs.oct_ptr.back() * 8;
-    cudaError_t e;
-    auto up = [&](auto** dst, const void* srcp, size_t bytes) {
-        if ((e = cudaMalloc(reinterpret_cast<void**>(dst), std::max<size_t>(bytes, 16))) != cudaSuccess) return e;
-        return srcp && bytes ? cudaMemcpyAsync(*dst, srcp, bytes, cudaMemcpyHostToDevice, st) : cudaSuccess;
-    };
-    if ((e = up(&d.oct_ptr, hs.oct_ptr.data(), sizeof(int) * hs.oct_ptr.size())) != cudaSuccess) return e;
-    if ((e = up(&d.idx_ptr, hs.idx_ptr.data(), sizeof(int) * hs.idx_ptr.size())) != cudaSuccess) return e;
-    if ((e = up(&d.row_slot, hs.row_slot.data(), sizeof(int) * hs.row_slot.size())) != cudaSuccess) return e;
-    if ((e = up(&d.idx, hs.idx.data(), sizeof(unsigned short) * hs.idx.size())) != cudaSuccess) return e;
-    if ((e = up(&d.src, hs.src.data(), sizeof(int) * hs.src.size())) != cudaSuccess) return e;
-    if ((e = up(&d.Shi, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
-    if ((e = up(&d.Slo, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
-    if ((e = up(&d.Hhi, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
-    if ((e = up(&d.Hlo, nullptr, sizeof(float4) * ni)) != cudaSuccess) return e;
-    if ((e = up(&d.S64, nullptr, 2 * sizeof(double2) * ni)) != cudaSuccess) return e;
-    if ((e = up(&d.H64, nullptr, 2 * sizeof(double2) * ni)) != cudaSuccess) return e;
-    d.n_items = (long long)ni;
-    launch_slice_fill(h->ds.S, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.S64), reinterpret_cast<float*>(d.Shi),
-                      reinterpret_cast<float*>(d.Slo), st);
-    launch_slice_fill(h->ds.H, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64), reinterpret_cast<float*>(d.Hhi),
-                      reinterpret_cast<float*>(d.Hlo), st);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;   // the host arrays are released here
-    d.nrows = hs.nrows;
-    d.noct = hs.noct;
-    d.unit_diag = h->ds.unit_diag;
-    return cudaSuccess;
-}
-
-static tb_status create_system(tb_handle** out, const tb_system_desc* d, void* stream, bool with_slices);
-
 tb_status tb_create(tb_handle** out, const tb_system_desc* d, void* stream) {
-    return create_system(out, d, stream, true);
-}
-
-static tb_status create_system(tb_handle** out, const tb_system_desc* d, void* stream, bool with_slices) {
     if (!out) return TB_ERR_INVALID_ARG;
     *out = nullptr;
     if (!d || d->n_atoms < 1 || !d->orb_per_atom || !d->brow_ptr || !d->bcol || !d->S_vals) return TB_ERR_INVALID_ARG;
@@ -1912,7 +2050,6 @@ static tb_status create_system(tb_handle** out, const tb_system_desc* d, void* s
     if (noalloc_scratch(h->device, &h->noalloc_base) != TB_OK) return fail(cudaErrorUnknown);
     h->sys_atom_off = {0, (int64_t)n};
     h->sys_orb_off = {0, N};
-    if (with_slices && (e = add_slice(h, 0, n, st)) != cudaSuccess) return fail(e);
     *out = h;
     return TB_OK;
 }
@@ -1970,7 +2107,7 @@ tb_status tb_create_batch(tb_handle** out, const tb_system_desc* descs, int32_t 
     m.eps = h_given ? nullptr : eps.data();
     m.K = descs[0].K;
     m.precision = TB_FP64;
-    const tb_status s = create_system(out, &m, stream, n_systems == 1);
+    const tb_status s = tb_create(out, &m, stream);
     if (s != TB_OK) return s;
     tb_handle* h = *out;
     h->sys_atom_off = aoff;
@@ -2034,8 +2171,6 @@ tb_status tb_create_batch(tb_handle** out, const tb_system_desc* descs, int32_t 
         v.grpG = 0;                 // the grouped SpMV's atom groups are built for the whole handle
         h->sys_ds.push_back(v);
     }
-    for (int q = 0; q < n_systems; ++q)
-        if ((e = add_slice(h, (int)aoff[q], (int)(aoff[q + 1] - aoff[q]), st)) != cudaSuccess) return fail(e);
     h->ds.rag = 0;
     return TB_OK;
 }

@@ -75,35 +75,56 @@ struct DevSystem {
     int* grp_cols = nullptr;   // distinct block-column atoms of each group, ascending
     int* blk_loc = nullptr;    // [nb] position of bcol[b] in the list of its group
 };
-// A small system's rows as the column slices consume them (tb_slice.cu):
-// eight streams per octet, the items of an octet interleaved step by step.
+// A system's rows as the column slices consume them, for clusters of cl CTAs
+// (tb_slice.cu): octets of eight rows, consecutive octets per CTA, eight
+// streams of items per octet, interleaved step by step.
 struct SliceDev {
-    int nrows = 0, noct = 0;        // rows (8 per octet), octets; 0: the system takes no slices
+    int nrows = 0, noct = 0;        // rows (8 per octet), octets; 0: no layout
+    int cl = 0;                     // CTAs per cluster
     int unit_diag = 0;              // as DevSystem::unit_diag
+    int nloc = 0;                   // rows of the gathered vector in a CTA (own and halo), at most
+    int max_len = 0;                // steps of an octet, at most
+    int max_oct = 0, max_steps = 0, max_bat = 0, max_dest = 0;   // octets, steps, index batches, destinations of a CTA
+    int* rank_oct = nullptr;        // [cl + 1] first octet of every CTA
     int* oct_ptr = nullptr;         // [noct + 1] first step of every octet (item = step * 8 + stream)
     int* idx_ptr = nullptr;         // [noct + 1] first batch of four indices of every octet
+    int* dest_ptr = nullptr;        // [2 noct + 1] copies of a group's rows: rank << 16 | group there
+    int* dest = nullptr;
     int* row_slot = nullptr;        // [nrows] padded orbital slot of a row, -1: filling
-    ushort4* idx = nullptr;         // [batches][8] gathered rows of the items of steps 1, 2, ...
+    ushort4* idx = nullptr;         // [batches][8] places (in the CTA's vector) of the items of steps 1, 2, ...
     int* src = nullptr;             // [items][4] offsets of the coefficients in S and H, -1: zero
     float4 *Shi = nullptr, *Slo = nullptr, *Hhi = nullptr, *Hlo = nullptr;   // [items]
     double2 *S64 = nullptr, *H64 = nullptr;                                  // [items][2]
     long long n_items = 0;
 };
 struct SliceHost {
-    int nrows = 0, noct = 0;
-    std::vector<int> oct_ptr, idx_ptr, row_slot, src;
+    int nrows = 0, noct = 0, cl = 0, nloc = 0, max_len = 0, max_oct = 0, max_steps = 0, max_bat = 0, max_dest = 0;
+    std::vector<int> rank_oct, oct_ptr, idx_ptr, dest_ptr, dest, row_slot, src;
     std::vector<unsigned short> idx;
+};
+// A block of outer steps whose updates of x^k (full solutions; several
+// projected functionals; z-derivatives) are made at its end: the shifts'
+// coefficients of every step and the real vectors (tb_slice.cu)
+struct SliceBlock {
+    int len = 0, rows = 0;          // steps it holds; values of a stored vector (M or npad)
+    int step = 0;                   // steps stored so far
+    double2 *A = nullptr, *L = nullptr, *dA = nullptr, *dL = nullptr;   // [len][P][K]
+    double* D = nullptr;            // [len + 1][P][rows]; nullptr: no block mode
+    int* count = nullptr;           // [P][K] steps of the block that a shift takes part in
 };
 // Arguments of one slice launch: up to nsteps outer steps of every column
 struct SliceArgs {
     int nc = 0, cl = 1;             // columns per slice, CTAs per cluster
+    int threads = 0;                // per CTA
+    int resident = 0;               // S of the inner solve: 0 copied ahead (FP64: global), 1 in shared memory, 2 in registers
+    int obytes = 0, ibase = 0;      // ring: bytes per octet, offset of its indices
     int nsteps = 0, start = 0;      // start: the inner solve of u_0 and the shifts' first state come first
     int n = 0, n_last = 0, R = 0;   // mixed: Chebyshev plan
     float gamma = 0.f;
     const float* omega = nullptr;   // device [n]
     int inner_max = 0;              // FP64: CG iterations of an inner solve, at most
     double inner_tol = 0.0;
-    double2 *dak = nullptr, *dbk = nullptr;   // [P][K] d/dz_k of alpha^k and l^k of a step (derivative mode)
+    SliceBlock blk;
 };
 
 size_t inner32_grp_smem(const DevSystem& s);   // dynamic shared memory of the grouped SpMV
@@ -217,10 +238,13 @@ double profile_busy(int id);
 int64_t launch_count();
 
 // ---- column slices (tb_slice.cu) -------------------------------------------
-void slice_layout(int n, const int32_t* orb, const int64_t* brow, const int32_t* bcol, int32_t col0, SliceHost& out);
-bool slice_choose(const SliceDev& ss, const PanelDev& p, int n_omega, int ncols, int sms, SliceArgs& a);
+void slice_layout(int n, const int32_t* orb, const int64_t* brow, const int32_t* bcol, int32_t col0, int cl,
+                  SliceHost& out);
+bool slice_fit(const SliceDev& ss, const PanelDev& p, int nc, bool reg, SliceArgs& a);
+int slice_clusters(bool mixed, int nc, bool reg, int cl, int threads, size_t smem);
 bool launch_slice(const SliceDev& ss, const DevSystem& s, const PanelDev& p, const SliceArgs& a, int ncols,
                   cudaStream_t st);
+void launch_block_flush(const PanelDev& p, const SliceBlock& b, int nsteps, int n0, bool goes_on, cudaStream_t st);
 void launch_slice_fill(const double* M, const int* src, long long n, double* m64, float* hi, float* lo, cudaStream_t st);
 
 // ---- launchers (tb_kernels.cu) -------------------------------------------

@@ -46,11 +46,13 @@ def _grid(s, K=12, eta=1.0):
     return gauss_legendre_grid(K, lo, hi, eta)
 
 
-# (slice width, cluster size): 0 = the library's choice; widths above the
-# FP64 path's largest are clipped to it
-@pytest.mark.parametrize("nc,cl", [(0, 0), (1, 1), (2, 3), (4, 8), (8, 2)])
+# (slice width, cluster size, S in registers): 0 = the library's choice; widths
+# above the FP64 path's largest are clipped to it, and a shape that does not
+# fit a system leaves it to the panel kernels
+@pytest.mark.parametrize("nc,cl,reg", [(0, 0, -1), (1, 1, 0), (2, 3, 0), (4, 8, 0), (8, 2, 0), (2, 1, 1), (2, 4, 1),
+                                       (4, 3, 1), (8, 8, 1)])
 @pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
-def test_fixed_steps_equal_the_panel_path(P, case, monkeypatch, prec, nc, cl):
+def test_fixed_steps_equal_the_panel_path(P, case, monkeypatch, prec, nc, cl, reg):
     """Twenty outer steps with forced seed switches: the same recurrences in
     another summation order, so the full solutions agree as the panel path
     agrees with the oracle's method after a fixed number of steps (1e-9; the
@@ -64,6 +66,7 @@ def test_fixed_steps_equal_the_panel_path(P, case, monkeypatch, prec, nc, cl):
     monkeypatch.setenv("TB_SLICE", "1")
     monkeypatch.setenv("TB_SLICE_NC", str(nc))
     monkeypatch.setenv("TB_SLICE_CL", str(cl))
+    monkeypatch.setenv("TB_SLICE_REG", str(reg))
     x, st = P.tb_shifted_cocg(h, z, cols, opts=opts, allow_unconverged=True)
     ref, x = ref.cpu().numpy(), x.cpu().numpy()
     assert np.abs(x - ref).max() <= 1e-9 * np.abs(ref).max()
@@ -71,11 +74,13 @@ def test_fixed_steps_equal_the_panel_path(P, case, monkeypatch, prec, nc, cl):
 
 
 @pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
-@pytest.mark.parametrize("R", [1, 3, 16])
-def test_outputs_against_dense(P, small, prec, R):
+@pytest.mark.parametrize("R,block", [(1, 0), (3, 32), (16, 64)])
+def test_outputs_against_dense(P, small, monkeypatch, prec, R, block):
     """Converged solutions, Green's-function elements with their z-derivatives
     and populations against the dense definitions (broadening 1 eV, tol 1e-10:
-    the forward error is at most |A^-1| tol ~ 1e-9 |x|)."""
+    the forward error is at most |A^-1| tol ~ 1e-9 |x|); the sums of solutions
+    and derivatives over one block of steps and over several."""
+    monkeypatch.setenv("TB_SLICE_BLOCK", str(block))
     s, H, S, h = small
     z, w = _grid(s, K=6)
     cols = np.linspace(0, s.n_orb - 1, R).astype(np.int32)
