@@ -1954,6 +1954,7 @@ tb_status tb_create(tb_handle** out, const tb_system_desc* d, void* stream) {
     h->ds.n_atoms = n;
     h->ds.nb = nb;
     h->ds.npad = 4 * n;
+    for (int i = 0; i < n; ++i) h->ds.max_row = std::max(h->ds.max_row, browh[i + 1] - browh[i]);
     // systems with s-only atoms keep the diagonal block in the product: on
     // water the changed FP32 rounding of the corrections made more of them
     // fall short of inner_lo_tol (7 % more Chebyshev steps, measured)

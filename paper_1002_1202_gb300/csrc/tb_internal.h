@@ -37,6 +37,7 @@ struct DevSystem {
     int n_atoms = 0;
     int64_t nb = 0;
     int npad = 0;              // 4 * n_atoms
+    int max_row = 0;           // blocks of a block row, at most
     int* brow = nullptr;       // [n_atoms + 1]
     int* bcol = nullptr;       // [nb]
     double* S = nullptr;       // [nb][16] row-major 4x4 blocks

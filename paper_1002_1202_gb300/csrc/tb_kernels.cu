@@ -1251,6 +1251,100 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelD
     }
 }
 
+// The step of k_inner32_cheb<2, ...> with S staged: a CTA takes RPC = 256 / (C / 2)
+// consecutive block rows, whose blocks of S and block columns are one
+// contiguous stretch that it copies to shared memory first, and the gathers of
+// a block's rows are issued one block ahead (60 registers, four CTAs per SM).
+// What is left is the gathers' way from L2 (~7 TB/s for the rows that L1 does
+// not hold): 256 columns of 4096 atoms 160.6 -> 152.5 ms per call, of 1728
+// atoms 184.4 -> 180.5, 24 Lanczos steps of 128 columns 24.9 -> 23.7 ms.  Three
+// CTAs per SM (77 registers): 164.9 / 188.1 / 24.3; starting the copy while the
+// step before ends (programmatic dependent launch): 153.6 / 195.7 / 28.5, the
+// waiting CTAs take the places of running ones.
+template <int PW, bool LAST>
+__global__ void __launch_bounds__(THREADS, 4) k_inner32_chebs(DevSystem s, PanelDev p, const float2* __restrict__ cur,
+                                                               float2* io, float omega, float gamma, int mode) {
+    extern __shared__ __align__(16) float4 s_dyn[];
+    const int C = PW > 0 ? PW : p.C;
+    const int TPR = C / 2, RPC = THREADS / TPR;
+    const int I0 = blockIdx.x * RPC, I1 = min(s.n_atoms, I0 + RPC);
+    const int g0 = __ldg(s.brow + I0), ng = __ldg(s.brow + I1) - g0;
+    float4* Ss = s_dyn;
+    int* Js = reinterpret_cast<int*>(s_dyn + 4 * (size_t)s.max_row * RPC);
+    {
+        const float4* src = reinterpret_cast<const float4*>(s.S32) + 4 * (size_t)g0;
+        const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(Ss));
+        for (int i = threadIdx.x; i < 4 * ng; i += THREADS)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * (uint32_t)i), "l"(src + i));
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        for (int i = threadIdx.x; i < ng; i += THREADS) Js[i] = __ldg(s.bcol + g0 + i);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (*(volatile int*)&p.flags[4] == 0) return;
+    const int t0 = threadIdx.x % TPR, I = I0 + threadIdx.x / TPR;
+    const int c0 = 2 * t0;
+    if (I >= I1 || !(cheb_live(p, c0) || cheb_live(p, c0 + 1))) return;
+    int b = __ldg(s.brow + I) - g0;
+    const int e1 = __ldg(s.brow + I + 1) - g0;
+    float acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[a][q] = 0.f;
+    const float2* base = cur + c0;
+    float4 xn[4];
+    auto fetch = [&](int bb) {
+        const float2* xb = base + (size_t)(4 * Js[bb]) * C;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xn[e] = *reinterpret_cast<const float4*>(xb + (size_t)e * C);
+    };
+    // the identity diagonal block (unit_diag) is skipped as in k_inner32_cheb
+    auto next = [&](int bb) { return s.unit_diag && bb < e1 && Js[bb] == I ? bb + 1 : bb; };
+    b = next(b);
+    if (b < e1) fetch(b);
+    while (b < e1) {
+        float4 xv[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xv[e] = xn[e];
+        const int nb = next(b + 1);
+        if (nb < e1) fetch(nb);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const float4 sr = Ss[4 * b + a];
+            acc[a][0] += sr.x * xv[0].x + sr.y * xv[1].x + sr.z * xv[2].x + sr.w * xv[3].x;
+            acc[a][1] += sr.x * xv[0].y + sr.y * xv[1].y + sr.z * xv[2].y + sr.w * xv[3].y;
+            acc[a][2] += sr.x * xv[0].z + sr.y * xv[1].z + sr.z * xv[2].z + sr.w * xv[3].z;
+            acc[a][3] += sr.x * xv[0].w + sr.y * xv[1].w + sr.z * xv[2].w + sr.w * xv[3].w;
+        }
+        b = nb;
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const size_t e = (size_t)(4 * I + a) * C + c0;
+        const float4 f4 = *reinterpret_cast<const float4*>(p.r32 + e);
+        const float4 c4 = *reinterpret_cast<const float4*>(cur + e);
+        const float4 p4 = mode == 1 ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(io + e);
+        const float f[4] = {f4.x, f4.y, f4.z, f4.w}, dc[4] = {c4.x, c4.y, c4.z, c4.w}, dp[4] = {p4.x, p4.y, p4.z, p4.w};
+        float dn[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dn[q] = dp[q] + omega * (gamma * (f[q] - (s.unit_diag ? acc[a][q] + dc[q] : acc[a][q])) + dc[q] - dp[q]);
+        if (LAST) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const InnerState i0 = p.inner32[2 * (c0 + j)], i1 = p.inner32[2 * (c0 + j) + 1];
+                double2 x = p.Rp[e + j];
+                if (!i0.skip && isfinite(dn[2 * j])) x.x += (double)dn[2 * j] * i0.unscale;
+                if (!i1.skip && isfinite(dn[2 * j + 1])) x.y += (double)dn[2 * j + 1] * i1.unscale;
+                p.Rp[e + j] = x;
+                p.RpS[e + j] = df_split(x);
+            }
+        } else {
+            *reinterpret_cast<float4*>(io + e) = make_float4(dn[0], dn[1], dn[2], dn[3]);
+        }
+    }
+}
+
 // The same Chebyshev step with four column pairs per thread and packed
 // FP32 FMAs: thread t0 of a block row (C / 4 threads per row) takes the
 // pairs (2 t0, 2 t0 + 1) and (C/2 + 2 t0, C/2 + 2 t0 + 1), so each of
@@ -2728,6 +2822,19 @@ static void cheb4_launch(const DevSystem& s, const PanelDev& p, const float2* cu
     }
 }
 
+template <int PW, bool LAST>
+static bool chebs_launch(const DevSystem& s, const PanelDev& p, const float2* cur, float2* io, float omega,
+                         float gamma, int mode, cudaStream_t st) {
+    const int rpc = THREADS / (p.C / 2);
+    const size_t sm = (size_t)s.max_row * rpc * (4 * sizeof(float4) + sizeof(int));
+    if (sm > 48 * 1024) return false;   // four CTAs per SM; long block rows take the unstaged form
+    static size_t lim = 0;
+    const auto k = k_inner32_chebs<PW, LAST>;
+    if (!ensure_dyn_smem((const void*)k, sm, lim)) return false;
+    k<<<(s.n_atoms + rpc - 1) / rpc, THREADS, sm, st>>>(s, p, cur, io, omega, gamma, mode);
+    return true;
+}
+
 template <bool LAST>
 static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur, float2* io, float omega,
                         float gamma, int mode, cudaStream_t st) {
@@ -2748,6 +2855,15 @@ static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur
         return;
     }
 
+    // two pairs per thread, S staged where a CTA's block rows fit
+    {
+        bool done = false;
+        if (p.C == 128) done = chebs_launch<128, LAST>(s, p, cur, io, omega, gamma, mode, st);
+        else if (p.C == 64) done = chebs_launch<64, LAST>(s, p, cur, io, omega, gamma, mode, st);
+        else if (p.C == 32) done = chebs_launch<32, LAST>(s, p, cur, io, omega, gamma, mode, st);
+        else if (p.C == 16) done = chebs_launch<16, LAST>(s, p, cur, io, omega, gamma, mode, st);
+        if (done) return;
+    }
     if (p.C >= 2) {
         const int g = grid_for((long long)s.n_atoms * (p.C / 2));
         switch (p.C) {
