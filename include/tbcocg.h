@@ -12,7 +12,8 @@
  * populations.  H is the tight-binding Hamiltonian matrix and S the overlap
  * matrix of Section 2.2; both are real symmetric, S positive definite.
  * The solver is the generalized shifted COCG method of Section 3.3 with
- * r' = S^-1 r from an inner solve (CG in FP64; with TB_MIXED, FP64
+ * r' = S^-1 r from an inner solve (in FP64: CG, or, on small systems at
+ * complex shifts, Chebyshev steps for the spectrum of S; with TB_MIXED, FP64
  * iterative refinement with FP32 corrections).  With real H, S and e_j the
  * collinear residuals of Eq. (collinear) are complex multiples of one real
  * vector, so the iteration carries that real vector (the Lanczos vector of
@@ -197,7 +198,7 @@ typedef struct {
                                  (and for an S whose bounds are unusable) FP32 CG.
                                  TB_INNER_CG: FP32 CG in every round.  Either way the
                                  FP64 residual of each round decides convergence, so both
-                                 reach the same inner_tol.  Ignored for TB_FP64 (CG).   */
+                                 reach the same inner_tol.  Ignored for TB_FP64.        */
     int64_t state_bytes;      /* energy-point checkpointing: device bytes allowed for the
                                  full-vector state of the shifts (x^k and p^k of every
                                  shift for the columns in flight, plus the device copy of

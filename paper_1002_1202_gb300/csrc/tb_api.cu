@@ -85,6 +85,13 @@ struct tb_handle {
     std::once_flag s_once;
     double s_lo = 0.0, s_hi = 0.0;
     tb_status s_status = TB_OK;
+    struct SysBounds {
+        bool done = false;
+        double lo = 0.0, hi = 0.0;
+        tb_status status = TB_OK;
+    };
+    std::mutex sys_mu;
+    std::vector<SysBounds> sys_bounds;   // batch: of the systems one by one
     // device address of the allocation-free call's fixed scratch on this
     // handle's device (looked up by tb_create)
     unsigned char* noalloc_base = nullptr;
@@ -393,6 +400,30 @@ tb_status s_bounds(tb_handle* h, double& lo, double& hi) {
     return h->s_status;
 }
 
+// The same bounds for one system of the handle alone: a batch's system then
+// takes the steps that it takes in a handle of its own.
+tb_status system_bounds(tb_handle* h, int sys, double& lo, double& hi) {
+    if (h->sys_ds.empty()) return s_bounds(h, lo, hi);
+    std::lock_guard<std::mutex> lk(h->sys_mu);
+    if (h->sys_bounds.empty()) h->sys_bounds.resize(h->sys_atom_off.size() - 1);
+    tb_handle::SysBounds& b = h->sys_bounds[sys];
+    if (!b.done) {
+        const int64_t a0 = h->sys_atom_off[sys], n = h->sys_atom_off[sys + 1] - a0;
+        const int64_t b0 = h->brow_h[a0], b1 = h->brow_h[a0 + n], v0 = h->boff_h[b0];
+        std::vector<int64_t> brow(n + 1), boff(b1 - b0 + 1);
+        std::vector<int32_t> bcol(b1 - b0);
+        for (int64_t i = 0; i <= n; ++i) brow[i] = h->brow_h[a0 + i] - b0;
+        for (int64_t k = b0; k <= b1; ++k) boff[k - b0] = h->boff_h[k] - v0;
+        for (int64_t k = b0; k < b1; ++k) bcol[k - b0] = h->bcol_h[k] - (int32_t)a0;
+        b.status = lanczos_bounds((int)n, h->orb_per_atom.data() + a0, brow.data(), bcol.data(), boff.data(),
+                                  h->S_h.data() + v0, b.lo, b.hi);
+        b.done = true;
+    }
+    lo = b.lo;
+    hi = b.hi;
+    return b.status;
+}
+
 // Coefficients of the Chebyshev corrections: n steps (odd, so that d_n ends
 // in x32) reduce the error by at least 1 / T_n(1 / sigma) <= lo_tol per
 // round.  R rounds are planned so that lo_tol^(R-1) times the last round's
@@ -413,6 +444,8 @@ struct ChebPlan {
     int R = 1;                 // rounds planned
     float gamma = 0.f;
     std::vector<float> omega;  // omega[k] multiplies step k (1 <= k < n)
+    double gamma64 = 0.0;      // the same unrounded, for steps in FP64
+    std::vector<double> omega64;
     int steps(int round) const { return round >= R - 1 ? n_last : n; }
     bool chebyshev(int round) const { return n > 0 && round < R + SPARE; }
     // the residual after this round in FP64 (spare rounds; with FP32 CG
@@ -436,12 +469,15 @@ ChebPlan cheb_plan(double lo, double hi, double lo_tol, double inner_tol, int ca
     cp.R = std::max(1, (int)std::ceil(std::log(inner_tol) / std::log(lo_tol) - 1e-9));
     const double rest = 0.5 * inner_tol / std::pow(lo_tol, cp.R - 1);
     cp.n_last = std::min(n, cheb_steps(sigma, rest));
-    cp.gamma = (float)(2.0 / (lo + hi));
+    cp.gamma64 = 2.0 / (lo + hi);
+    cp.gamma = (float)cp.gamma64;
     cp.omega.assign(n, 0.f);
+    cp.omega64.assign(n, 0.0);
     double om = 1.0;
     for (int k = 1; k < n; ++k) {
         om = (k == 1) ? 1.0 / (1.0 - 0.5 * sigma * sigma) : 1.0 / (1.0 - 0.25 * om * sigma * sigma);
         cp.omega[k] = (float)om;
+        cp.omega64[k] = om;
     }
     return cp;
 }
@@ -905,7 +941,7 @@ const SliceDev* slice_choose(const View& v, const PanelDev& p, int ncols, SliceA
     const double nnz = (double)(h->boff_h[h->brow_h[a1]] - h->boff_h[h->brow_h[a0]]);
     const double L = nnz / 4 / N * 1.1 + 1;       // items of a stream
     const double items = N * L;
-    const double inner = mixed ? std::max(1, 2 * a.n) : 45.0;
+    const double inner = mixed ? std::max(1, 2 * a.n) : a.n > 0 ? a.n : 45.0;
     struct Cand {
         int nc, cl;
         bool reg;
@@ -927,7 +963,7 @@ const SliceDev* slice_choose(const View& v, const PanelDev& p, int ncols, SliceA
                 const double passes = std::ceil(rows * lps / 512);
                 // shared memory, and so the clusters that run at once
                 const double vec = std::min(N, rows * (1 + 6.0 / std::sqrt(N / 64))) * nc * 8;
-                const double smem = vec + rows * nc * (mixed ? 4 : 32) + 8e3 + threads * (mixed ? 16 : 8) +
+                const double smem = vec * (mixed ? 1 : 2) + rows * nc * (mixed ? 4 : 32) + 8e3 + threads * (mixed ? 16 : 8) +
                                     (reg ? 0 : items / cl * (mixed ? 18 : 34));
                 const bool fits = smem < 220e3;
                 const int thr = ((int)threads + 31) / 32 * 32;
@@ -944,7 +980,7 @@ const SliceDev* slice_choose(const View& v, const PanelDev& p, int ncols, SliceA
                     step = std::max({load * wi * wf, passes * L * 35 + 250, stream}) + bar;
                     outer = 15 * bar + load * rows * nc * 60 / 1.7 + 4 * (load * wi * 30 + passes * L * 60) + 25e3;
                 } else {
-                    step = load * items / cl * 4 * nc / 1.7 + passes * L * 160 + 7500 + 2 * bar;
+                    step = load * items / cl * 4 * nc / 1.7 + passes * L * 160 + (a.n > 0 ? 500 + bar : 7500 + 2 * bar);
                     outer = 10 * bar + load * rows * nc * 20 / 1.7 + 25e3;
                 }
                 outer += load * (double)p.K * nc * 60 / cl / 1.7;
@@ -1066,9 +1102,20 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     SliceArgs sa;
     bool slices = false;
     const SliceDev* sl = nullptr;
-    if (slices_on() && !g_trace && v.owner && v.sys >= 0 && M <= 256 &&
+    if (slices_on() && !g_trace && v.owner && v.sys >= 0 && v.n_orb <= SLICE_MAX_ROWS && M <= 256 &&
         (!p.mixed || (ic.cheb.n > 0 && ic.cheb.n <= 512))) {
-        sa.n = ic.cheb.n;
+        // FP64 inner solves of the slices: Chebyshev steps in FP64 to inner_tol
+        // when S has usable bounds, else the CG; also the CG when some shift is
+        // real, where a pivot can vanish and S = 1 has to be solved exactly to
+        // see it
+        ChebPlan c64;
+        bool real_shift = false;
+        for (int k = 0; k < K; ++k) real_shift = real_shift || q.z[2 * k + 1] == 0.0;
+        if (!p.mixed && !real_shift) {
+            double lo = 0.0, hi = 0.0;
+            if (system_bounds(v.owner, v.sys, lo, hi) == TB_OK) c64 = cheb_plan(lo, hi, o->inner_tol, o->inner_tol, std::min(o->inner_max_iter, 512));
+        }
+        sa.n = p.mixed ? ic.cheb.n : c64.n;
         sl = slice_choose(v, p, std::max(std::min(P, R), q.columns), sa, st);
         slices = sl != nullptr;
         if (slices) {
@@ -1082,6 +1129,14 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
                 sa.n_last = ic.cheb.n_last;
                 sa.R = ic.cheb.R;
                 sa.gamma = ic.cheb.gamma;
+            }
+            if (!p.mixed && c64.n > 0) {
+                double* om = nullptr;
+                if ((s = dalloc(cl, &om, (size_t)c64.n)) != TB_OK) return s;
+                TB_CK(cudaMemcpyAsync(om, c64.omega64.data(), sizeof(double) * c64.n, cudaMemcpyHostToDevice, st));
+                sa.omega64 = om;
+                sa.n_last = std::min(c64.n, 9);
+                sa.gamma64 = c64.gamma64;
             }
             if (q.proj == PROJ_NONE || M > 1 || p.deriv) {
                 // block mode: up to 512 steps per block (most solves end within

@@ -120,10 +120,15 @@ struct SliceArgs {
     int resident = 0;               // S of the inner solve: 0 copied ahead (FP64: global), 1 in shared memory, 2 in registers
     int obytes = 0, ibase = 0;      // ring: bytes per octet, offset of its indices
     int nsteps = 0, start = 0;      // start: the inner solve of u_0 and the shifts' first state come first
-    int n = 0, n_last = 0, R = 0;   // mixed: Chebyshev plan
+    // Chebyshev plan of the inner solve: steps of a full and of a last round,
+    // planned rounds (mixed), coefficients on the device [n]; FP64: n = 0 takes
+    // the CG, of at most inner_max iterations
+    int n = 0, n_last = 0, R = 0;
     float gamma = 0.f;
-    const float* omega = nullptr;   // device [n]
-    int inner_max = 0;              // FP64: CG iterations of an inner solve, at most
+    const float* omega = nullptr;
+    double gamma64 = 0.0;
+    const double* omega64 = nullptr;
+    int inner_max = 0;
     double inner_tol = 0.0;
     SliceBlock blk;
 };

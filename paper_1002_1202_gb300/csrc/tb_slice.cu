@@ -139,9 +139,9 @@ __host__ __device__ __forceinline__ SliceMem slice_mem(const SliceDev& ss, int M
     m.part = up16(sizeof(SliceShared<NC>));
     m.dfun = m.part + up16(sizeof(double) * CPL * T);
     m.omega = m.dfun + up16(sizeof(double) * NC * (size_t)(M > 0 ? M : 1));
-    m.tab = m.omega + up16(sizeof(float) * (size_t)(MIXED ? n_omega : 0));
+    m.tab = m.omega + up16((MIXED ? sizeof(float) : sizeof(double)) * (size_t)n_omega);
     m.vec = m.tab + up16(sizeof(int) * (size_t)(4 * ss.max_oct + 3 + ss.max_dest));
-    m.own = m.vec + sizeof(double) * NC * (size_t)ss.nloc;      // mixed: two FP32 vectors; FP64: one
+    m.own = m.vec + (MIXED ? 1 : 2) * sizeof(double) * NC * (size_t)ss.nloc;   // two vectors, FP32 or FP64
     m.sbuf = m.own + (MIXED ? sizeof(float) * CPL * nel_pad : sizeof(double) * 4 * nel_pad);
     m.total = m.sbuf;
     if (resident == 2) return m;                                // S in registers
@@ -783,19 +783,13 @@ struct Slice {   // CPL: columns per lane
             for (int e0 = 0; e0 < nel_pad; e0 += T) {
                 if (e0 + (tid & ~31) >= nel_pad) break;
                 const Elem e = elem(e0);
-                const double2* mc = nullptr;
-                const ushort4* ix = nullptr;
-                if (a.resident && e.on) {
-                    mc = reinterpret_cast<const double2*>(sbuf + (size_t)optr[e.oct] * LINE) + e.s8;
-                    ix = reinterpret_cast<const ushort4*>(sbuf + (size_t)nsteps_all * LINE) + (size_t)iptr[e.oct] * 8 + e.s8;
-                }
-                const Cols<CPL> w = spmv64(e, ss.S64, rv, mc, ix);
+                const double w = product_S(e, rv);
                 if (!e.on) continue;
                 const double r = rv[(size_t)e.row * NC + e.q];
-                wv[e0 + tid] = w.v[0];
+                wv[e0 + tid] = w;
                 if (e.slot >= 0) {
                     v[0][0] += r * r;
-                    v[1][0] += w.v[0] * r;
+                    v[1][0] += w * r;
                 }
             }
             double out[2];
@@ -875,9 +869,95 @@ struct Slice {   // CPL: columns per lane
         __syncthreads();
         return true;
     }
+    // ---- inner solve in FP64 by Chebyshev steps for the spectrum of S (the
+    // recurrence of the mixed path's corrections, all of it in FP64): no inner
+    // products, so a step is a product and a barrier where a CG iteration has two
+    // reductions, ~2000 cycles of scalars and a second barrier.  The residual
+    // u - S u' at its end decides; a column above inner_tol takes further rounds
+    // on its residual (a.n_last steps each).
+    __device__ bool inner_cheb64(int& steps) {
+        double* xa = reinterpret_cast<double*>(vec);
+        double* xb = xa + (size_t)nloc * NC;
+        double* fb = reinterpret_cast<double*>(own);
+        double* xs = fb + nel_pad;
+        const double* om = reinterpret_cast<const double*>(omega);
+        for (int round = 0;; ++round) {
+            const int n = round == 0 ? a.n : a.n_last;
+            steps += n;
+            for (int e0 = 0; e0 < nel_pad; e0 += T) {
+                const Elem e = elem(e0);
+                if (!e.on) continue;
+                const double f = e.slot >= 0 && !sh.skip[e.q] ? *at(round == 0 ? p.Rcur : p.Rin, e) : 0.0;
+                fb[e0 + tid] = f;
+                if (round == 0) xs[e0 + tid] = 0.0;
+                bcast(xa, e.row, NC, e.q, a.gamma64 * f);
+                if (n == 1) xs[e0 + tid] += a.gamma64 * f;
+            }
+            barrier();
+            for (int k = 1; k < n; ++k) {
+                const double* cur = (k & 1) ? xa : xb;
+                double* io = (k & 1) ? xb : xa;
+                const double w = om[k];
+                for (int e0 = 0; e0 < nel_pad; e0 += T) {
+                    if (e0 + (tid & ~31) >= nel_pad) break;
+                    const Elem e = elem(e0);
+                    const double y = product_S(e, cur);
+                    if (!e.on) continue;
+                    const size_t i = (size_t)e.row * NC + e.q;
+                    const double dc = cur[i], dp = k == 1 ? 0.0 : io[i];
+                    const double dn = e.slot < 0 ? 0.0 : dp + w * (a.gamma64 * (fb[e0 + tid] - y) + dc - dp);
+                    if (k == n - 1) xs[e0 + tid] += dn;
+                    else bcast(io, e.row, NC, e.q, dn);
+                }
+                barrier();
+            }
+            // u' published, then its residual and t = u^T u'
+            for (int e0 = 0; e0 < nel_pad; e0 += T) {
+                const Elem e = elem(e0);
+                if (e.on) bcast(xa, e.row, NC, e.q, xs[e0 + tid]);
+            }
+            barrier();
+            double v[2][CPL] = {};
+            for (int e0 = 0; e0 < nel_pad; e0 += T) {
+                if (e0 + (tid & ~31) >= nel_pad) break;
+                const Elem e = elem(e0);
+                const double y = product_S(e, xa);
+                if (e.slot < 0) continue;
+                const double u = *at(p.Rcur, e), x = xs[e0 + tid], r = u - y;
+                *at(p.Rin, e) = r;
+                *at(p.Rp, e) = x;
+                v[0][0] += r * r;
+                v[1][0] += u * x;
+            }
+            double out[2];
+            sum<2>(v, out);
+            if (tid == 0) sh.open = sh.bad = 0;
+            __syncthreads();
+            if (tid < NC) {
+                sh.tsum[tid] = out[1];
+                if (!isfinite(out[0])) atomicExch(&sh.bad, 1);
+                if (out[0] <= a.inner_tol * a.inner_tol * sh.b2[tid]) sh.skip[tid] = 1;
+                if (!sh.skip[tid]) atomicAdd(&sh.open, 1);
+            }
+            __syncthreads();
+            if (sh.bad) return false;
+            if (sh.open == 0) return true;
+            if (round >= SL_SPARE + 1) return false;
+        }
+    }
+    // one row of S x with the coefficients where they are
+    __device__ __forceinline__ double product_S(const Elem& e, const double* x) const {
+        const double2* mc = nullptr;
+        const ushort4* ix = nullptr;
+        if (a.resident && e.on) {
+            mc = reinterpret_cast<const double2*>(sbuf + (size_t)optr[e.oct] * LINE) + e.s8;
+            ix = reinterpret_cast<const ushort4*>(sbuf + (size_t)nsteps_all * LINE) + (size_t)iptr[e.oct] * 8 + e.s8;
+        }
+        return spmv64(e, ss.S64, x, mc, ix).v[0];
+    }
     __device__ bool inner(int& steps) {
         if (MIXED) return inner_mixed(steps);
-        return inner_fp64(steps);
+        return a.n > 0 ? inner_cheb64(steps) : inner_fp64(steps);
     }
 
     // ---- functionals of u' (written by every CTA of the cluster: read at L2)
@@ -1207,8 +1287,10 @@ __global__ void __launch_bounds__(SL_T, 1) k_slice(SliceDev ss, DevSystem s, Pan
     sl.nsteps_all = __ldg(ss.oct_ptr + sl.oct0 + noct_l) - sl.step0;
     const int tid = threadIdx.x;
     for (int i = tid; i < NC; i += sl.T) sh.cs[i] = p.col[sl.c0 + i];
-    if (MIXED)
-        for (int i = tid; i < a.n; i += sl.T) sl.omega[i] = a.omega[i];
+    for (int i = tid; i < a.n; i += sl.T) {
+        if (MIXED) sl.omega[i] = a.omega[i];
+        else reinterpret_cast<double*>(sl.omega)[i] = a.omega64[i];
+    }
     if (tid == 0) {
         sh.open = sh.bad = sh.wanted = sh.active = 0;
         sh.bstep = a.blk.step;
