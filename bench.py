@@ -518,19 +518,20 @@ KERNEL_INFO = {
 }
 
 
-# columns per thread of the Chebyshev step that the autotuner chose (None:
-# the library default)
+# column pairs per thread of the Chebyshev step as the run took it (the
+# autotuner's choice or the library's default; None: no run yet)
 CHEB_CPT = None
 
 
 def cheb_kernel_name(panel, n_atoms):
-    """The Chebyshev step's kernel, as the library picks it: the autotuner's
-    choice, else TB_CHEB_CPT, else four columns per thread with packed FMAs
-    from 16 columns per panel on and two below that."""
+    """The Chebyshev step's kernel of a panel of ``panel`` column pairs: with
+    two pairs per thread the form with S staged in shared memory for 16 to
+    128 pairs, else the plain one; with four pairs the packed one (from 16
+    pairs on; taken when no run or TB_CHEB_CPT says otherwise)."""
     env = os.environ.get("TB_CHEB_CPT")
     cpt = CHEB_CPT if CHEB_CPT else (int(env) if env else (4 if panel >= 16 else 2))
     if cpt == 2 or panel < 4:
-        return "k_inner32_cheb"
+        return "k_inner32_chebs" if panel in (16, 32, 64, 128) else "k_inner32_cheb"
     return "k_inner32_cheb4"
 
 
@@ -539,7 +540,9 @@ DF_INSTR_PER_MAC = 12   # FP32 instructions of one double-float multiply-add (ex
 
 def roofline_for(kname, ms, launches, s, panel, peaks, mixed=False, busy_ms=None):
     """Roofline of one SpMM-type kernel: algorithmic flops and bytes per
-    launch over its CUDA-event time per launch.  With two panels in flight
+    launch over its CUDA-event time per launch; ``panel`` counts pairs of
+    real columns (the Krylov vectors are real, so a panel of P right-hand
+    sides has P / 2 pairs).  With two panels in flight
     the launches of a kernel class overlap (and share the GPU), so the time
     per launch is the class's busy time (union of its launch intervals,
     ``busy_ms``) over its launches; the mean of the individual durations is
@@ -553,14 +556,13 @@ def roofline_for(kname, ms, launches, s, panel, peaks, mixed=False, busy_ms=None
         kern = cheb_kernel_name(panel, s.n_atoms)
     double_float = mixed and kname in ("outer_spmm", "refine_residual")
     nnz = 16 * s.nb
-    mats = 2 if kname == "outer_spmm" else 1
-    flops = 2.0 * nnz * 2 * panel * mats
+    flops = 2.0 * nnz * 2 * panel
     if kname == "inner32_cheb":
         flops += 5.0 * s.n_orb * 2 * panel      # d_{k+1} = d_{k-1} + omega (gamma (f - S d_k) + d_k - d_{k-1})
     # panel vectors moved once: the SpMVs read x and write y; the Chebyshev
     # step reads d_k, f and d_{k-1} and writes d_{k+1}
     vec_io = {"inner_spmv": 2, "inner32_spmv": 2, "inner32_cheb": 4, "refine_residual": 3, "outer_spmm": 5}[kname]
-    nbytes = mats * nnz * mb + 4 * s.nb + 4 * (s.n_atoms + 1) + vec_io * s.n_orb * panel * vb
+    nbytes = nnz * mb + 4 * s.nb + 4 * (s.n_atoms + 1) + vec_io * s.n_orb * panel * vb
     mean_s = ms / max(launches, 1) / 1e3
     avg_s = busy_ms / max(launches, 1) / 1e3 if busy_ms else mean_s
     if avg_s <= 0:
@@ -621,6 +623,8 @@ def run_ours(args):
     s, z, w = workload()
     h = P.tb_create_system(s)
     alu_peaks = measure_alu_peaks(P)
+    global CHEB_CPT
+    CHEB_CPT = int(os.environ.get("TB_CHEB_CPT", "2"))
     prec = 1 if args.precision == "mixed" else 0
     inner_method = P.tb.TB_INNER_CG if args.inner_method == "cg" else P.tb.TB_INNER_CHEBYSHEV
     tune = None
@@ -632,8 +636,7 @@ def run_ours(args):
         o_t = P.tb_default_opts(tol=args.tol, precision=prec, inner_tol=args.inner_tol, inner_method=inner_method)
         tune = P.tb_autotune(h, z, w, 2.0, opts=o_t, iters=3)
         best = tune[0]["panel"]
-        global CHEB_CPT
-        CHEB_CPT = tune[0]["cheb_cpt"] or None
+        CHEB_CPT = tune[0]["cheb_cpt"] or CHEB_CPT
         if world > 1:
             t = torch.tensor([best], device="cuda", dtype=torch.int64)
             dist.broadcast(t, 0)
@@ -713,15 +716,16 @@ def run_ours(args):
     # roofline of the dominant kernel (largest device time in the timed region)
     peaks = measured_peaks()
     dom = max((k for k in KERNEL_INFO), key=lambda k: kernel_ms[k][1])
-    roofline = roofline_for(dom, kernel_ms[dom][1], kernel_ms[dom][0], s, args.panel, peaks, prec == 1,
+    pairs = max(args.panel // 2, 1)
+    roofline = roofline_for(dom, kernel_ms[dom][1], kernel_ms[dom][0], s, pairs, peaks, prec == 1,
                             kernel_busy[dom])
-    others = {k: roofline_for(k, kernel_ms[k][1], kernel_ms[k][0], s, args.panel, peaks, prec == 1, kernel_busy[k])
+    others = {k: roofline_for(k, kernel_ms[k][1], kernel_ms[k][0], s, pairs, peaks, prec == 1, kernel_busy[k])
               for k in KERNEL_INFO if k != dom and kernel_ms[k][0] > 0}
     share = {k: round(v[1], 3) for k, v in kernel_ms.items() if v[0] > 0}
     # second part of the metric: SpMM algorithmic HBM GB/s against the measured copy peak
     spmm_hbm = {}
     for k in ("inner32_cheb", "inner32_spmv", "outer_spmm", "inner_spmv"):
-        rec = roofline if roofline and roofline.get("kernel") == KERNEL_INFO[k][0] else others.get(k)
+        rec = roofline if k == dom else others.get(k)
         if not rec:
             continue
         gbs = rec["algorithmic_bytes_per_launch"] / (rec["avg_launch_us"] * 1e-6) / 1e9
@@ -729,7 +733,7 @@ def run_ours(args):
                        "frac": gbs / peaks["hbm_gbs"],
                        "note": "algorithmic bytes (matrix once, every panel vector the kernel touches read or "
                                "written once) per busy time per launch; at 128-256 columns per panel the SpMM "
-                               "does 8-16 flop per such byte, so it is limited by the gathers and the ALUs, not "
+                               "does 4-8 flop per such byte, so it is limited by the gathers and the ALUs, not "
                                "by HBM"}
 
     # the other precision on the same panel, for comparison

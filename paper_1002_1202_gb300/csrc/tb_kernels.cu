@@ -1255,9 +1255,10 @@ __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelD
 // consecutive block rows, whose blocks of S and block columns are one
 // contiguous stretch that it copies to shared memory first, and the gathers of
 // a block's rows are issued one block ahead (60 registers, four CTAs per SM).
-// What is left is the gathers' way from L2 (~7 TB/s for the rows that L1 does
-// not hold): 256 columns of 4096 atoms 160.6 -> 152.5 ms per call, of 1728
-// atoms 184.4 -> 180.5, 24 Lanczos steps of 128 columns 24.9 -> 23.7 ms.  Three
+// What is left is the gathers' way from L2 (ncu, 256 columns of 4096 atoms:
+// 257 MB in 31.4 us, 8.2 TB/s, L1 hit 31 %, 57 % issue; packed FMAs and fewer
+// moves change nothing): 256 columns of 4096 atoms 160.6 -> 152.5 ms per call,
+// of 1728 atoms 184.4 -> 180.5, 24 Lanczos steps of 128 columns 24.9 -> 23.7 ms.  Three
 // CTAs per SM (77 registers): 164.9 / 188.1 / 24.3; starting the copy while the
 // step before ends (programmatic dependent launch): 153.6 / 195.7 / 28.5, the
 // waiting CTAs take the places of running ones.

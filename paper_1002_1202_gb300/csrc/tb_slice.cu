@@ -1483,7 +1483,7 @@ __global__ void k_slice_fill(const double* __restrict__ M, const int* __restrict
 // z-derivatives), and x, q are read and written once per block, not per step.
 // FP64 arithmetic bounds both (1.7 FMA per cycle and SM on this part): 64 atoms,
 // all 256 columns, 68 rows, 64 shifts with z-derivatives: 31.6 ms per call with
-// updates every step.  In the first block q_0 = v_0.
+// updates every step, 20.4 with blocks.  In the first block q_0 = v_0.
 
 // (alpha, l) -> (C, E) in place, one thread per (column, shift); a shift's
 // steps end at its convergence
