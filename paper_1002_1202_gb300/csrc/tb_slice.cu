@@ -699,6 +699,30 @@ struct Slice {   // CPL: columns per lane
         for (int j = 0; j < CPL; ++j) dk.v[j] = a.gamma * f.v[j];
         const int st = e.s8 & 3;
         const bool up = st & 2, odd = st & 1;
+        // where the row's first REMOTE copies lie (shared::cluster addresses in xa;
+        // xb at the same distance in every CTA), worked out once a round: 13 columns
+        // of 144 atoms, four CTAs per slice, 36.9 -> 34.7 ms per call.  With four
+        // columns per lane the registers are full (512 atoms: 109.0 -> 110.0 ms), and
+        // every copy is looked up at its store.
+        constexpr int REMOTE = CPL == 2 ? 3 : 0;
+        const size_t own_at = (size_t)e.row * LPS + e.q;
+        unsigned ra[REMOTE + 1];
+        int nd = 0, dbeg = 0;
+        if (e.on) {
+            dbeg = dptr[e.row >> 2];
+            nd = dptr[(e.row >> 2) + 1] - dbeg;
+        }
+#pragma unroll
+        for (int i = 0; i < REMOTE; ++i) {
+            ra[i] = 0;
+            if (i < nd) {
+                const int d = dest[dbeg + i];
+                const uint32_t here = static_cast<uint32_t>(
+                    __cvta_generic_to_shared(xa + ((size_t)(d & 0xffff) * 4 + (e.row & 3)) * LPS + e.q));
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra[i]) : "r"(here), "r"(d >> 16));
+            }
+        }
+        const unsigned to_b = (unsigned)(reinterpret_cast<unsigned char*>(xb) - reinterpret_cast<unsigned char*>(xa));
         for (int k = 1; k < n; ++k) {
             const float* xq = reinterpret_cast<const float*>((k & 1) ? xa : xb) + e.q * CPL;
             float acc[4][CPL];
@@ -734,12 +758,32 @@ struct Slice {   // CPL: columns per lane
             }
             dp = dk;
             dk = dn;
-            if (k < n - 1 && e.on) bcast((k & 1) ? xb : xa, e.row, LPS, e.q, dn);
+            if (k < n - 1 && e.on) {
+                VF* to = (k & 1) ? xb : xa;
+                if constexpr (REMOTE == 0) {
+                    bcast(to, e.row, LPS, e.q, dn);
+                } else {
+                    to[own_at] = dn;
+                    const unsigned off = (k & 1) ? to_b : 0u;
+#pragma unroll
+                    for (int i = 0; i < REMOTE; ++i)
+                        if (i < nd) st_remote(ra[i] + off, dn);
+                    for (int i = REMOTE; i < nd; ++i) {
+                        const int d = dest[dbeg + i];
+                        *cg::this_cluster().map_shared_rank(
+                            to + ((size_t)(d & 0xffff) * 4 + (e.row & 3)) * LPS + e.q, d >> 16) = dn;
+                    }
+                }
+            }
             barrier();
         }
         if (n > 1 && e.slot >= 0) add_correction(e, dk, round);
     }
 
+    __device__ __forceinline__ static void st_remote(unsigned addr, const VF& v) {
+        static_assert(CPL == 2, "a pair of columns");
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.v[0]), "f"(v.v[1]) : "memory");
+    }
     // u' += d * ||res|| (a non-finite correction is dropped, as in k_refine_add)
     __device__ __forceinline__ void add_correction(const Elem& e, const VF& d, int round) {
         Cols<CPL> x{};
