@@ -350,6 +350,59 @@ struct Slice {   // CPL: columns per lane
         }
         cp_commit();
     }
+    // Where the first REMOTE copies of an element's row lie (shared::cluster
+    // addresses in xa; xb at the same distance in every CTA), worked out once a
+    // round: 13 columns of 144 atoms, four CTAs per slice, 36.9 -> 34.8 ms per
+    // call; with S in shared memory and one element per thread too, a
+    // charge-self-consistent call of 48 water molecules 42.6 -> 40.9 ms (the row
+    // itself kept across steps: 40.5, but a batch of boxes 26.0 -> 26.5).  With
+    // four columns per lane the registers are full (512 atoms: 109.0 -> 110.0
+    // ms), and every copy is looked up at its store.
+    static constexpr int REMOTE = CPL == 2 ? 3 : 0;
+    struct Copies {
+        unsigned at[REMOTE + 1];
+        unsigned to_b;
+        int n, first;
+    };
+    __device__ __forceinline__ Copies copies(const Elem& e, VF* xa, VF* xb) {
+        Copies c;
+        c.n = c.first = 0;
+        c.to_b = (unsigned)(reinterpret_cast<unsigned char*>(xb) - reinterpret_cast<unsigned char*>(xa));
+        if (e.on) {
+            c.first = dptr[e.row >> 2];
+            c.n = dptr[(e.row >> 2) + 1] - c.first;
+        }
+#pragma unroll
+        for (int i = 0; i < REMOTE; ++i) {
+            c.at[i] = 0;
+            if (i < c.n) {
+                const int d = dest[c.first + i];
+                const uint32_t here = static_cast<uint32_t>(
+                    __cvta_generic_to_shared(xa + ((size_t)(d & 0xffff) * 4 + (e.row & 3)) * LPS + e.q));
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(c.at[i]) : "r"(here), "r"(d >> 16));
+            }
+        }
+        return c;
+    }
+    // bcast(to, ...) of a row whose copies are known; to: xa, or xb (b)
+    __device__ __forceinline__ void publish(const Elem& e, const Copies& c, VF* to, bool b, const VF& v) {
+        if constexpr (REMOTE == 0) {
+            bcast(to, e.row, LPS, e.q, v);
+        } else {
+            to[(size_t)e.row * LPS + e.q] = v;
+            const unsigned off = b ? c.to_b : 0u;
+#pragma unroll
+            for (int i = 0; i < REMOTE; ++i)
+                if (i < c.n)
+                    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(c.at[i] + off), "f"(v.v[0]),
+                                 "f"(v.v[1])
+                                 : "memory");
+            for (int i = REMOTE; i < c.n; ++i) {
+                const int d = dest[c.first + i];
+                *cg::this_cluster().map_shared_rank(to + ((size_t)(d & 0xffff) * 4 + (e.row & 3)) * LPS + e.q, d >> 16) = v;
+            }
+        }
+    }
     // FP32 product with S; cf, ix: the stream's coefficients and indices in
     // shared memory.  Scalar FMAs: a packed one needs its coefficient twice in a
     // register pair, which costs as many moves as it saves.  The four streams'
@@ -542,6 +595,9 @@ struct Slice {   // CPL: columns per lane
             }
             barrier();
             if (REG) chebyshev_reg(n, round, xa, xb, fb);
+            // one element per thread: its row's copies are the same in every step
+            const bool single = !REG && nel_pad <= T;
+            const Copies cp = copies(elem(0), xa, xb);
             for (int k = 1; !REG && k < n; ++k) {
                 const VF* cur = (k & 1) ? xa : xb;
                 VF* io = (k & 1) ? xb : xa;
@@ -583,7 +639,8 @@ struct Slice {   // CPL: columns per lane
                     if (k == n - 1) {
                         if (e.slot >= 0) add_correction(e, dn, round);
                     } else {
-                        bcast(io, e.row, LPS, e.q, dn);
+                        if (single) publish(e, cp, io, (k & 1) != 0, dn);
+                        else bcast(io, e.row, LPS, e.q, dn);
                     }
                 }
                 barrier();
@@ -699,30 +756,7 @@ struct Slice {   // CPL: columns per lane
         for (int j = 0; j < CPL; ++j) dk.v[j] = a.gamma * f.v[j];
         const int st = e.s8 & 3;
         const bool up = st & 2, odd = st & 1;
-        // where the row's first REMOTE copies lie (shared::cluster addresses in xa;
-        // xb at the same distance in every CTA), worked out once a round: 13 columns
-        // of 144 atoms, four CTAs per slice, 36.9 -> 34.7 ms per call.  With four
-        // columns per lane the registers are full (512 atoms: 109.0 -> 110.0 ms), and
-        // every copy is looked up at its store.
-        constexpr int REMOTE = CPL == 2 ? 3 : 0;
-        const size_t own_at = (size_t)e.row * LPS + e.q;
-        unsigned ra[REMOTE + 1];
-        int nd = 0, dbeg = 0;
-        if (e.on) {
-            dbeg = dptr[e.row >> 2];
-            nd = dptr[(e.row >> 2) + 1] - dbeg;
-        }
-#pragma unroll
-        for (int i = 0; i < REMOTE; ++i) {
-            ra[i] = 0;
-            if (i < nd) {
-                const int d = dest[dbeg + i];
-                const uint32_t here = static_cast<uint32_t>(
-                    __cvta_generic_to_shared(xa + ((size_t)(d & 0xffff) * 4 + (e.row & 3)) * LPS + e.q));
-                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra[i]) : "r"(here), "r"(d >> 16));
-            }
-        }
-        const unsigned to_b = (unsigned)(reinterpret_cast<unsigned char*>(xb) - reinterpret_cast<unsigned char*>(xa));
+        const Copies cp = copies(e, xa, xb);
         for (int k = 1; k < n; ++k) {
             const float* xq = reinterpret_cast<const float*>((k & 1) ? xa : xb) + e.q * CPL;
             float acc[4][CPL];
@@ -758,32 +792,12 @@ struct Slice {   // CPL: columns per lane
             }
             dp = dk;
             dk = dn;
-            if (k < n - 1 && e.on) {
-                VF* to = (k & 1) ? xb : xa;
-                if constexpr (REMOTE == 0) {
-                    bcast(to, e.row, LPS, e.q, dn);
-                } else {
-                    to[own_at] = dn;
-                    const unsigned off = (k & 1) ? to_b : 0u;
-#pragma unroll
-                    for (int i = 0; i < REMOTE; ++i)
-                        if (i < nd) st_remote(ra[i] + off, dn);
-                    for (int i = REMOTE; i < nd; ++i) {
-                        const int d = dest[dbeg + i];
-                        *cg::this_cluster().map_shared_rank(
-                            to + ((size_t)(d & 0xffff) * 4 + (e.row & 3)) * LPS + e.q, d >> 16) = dn;
-                    }
-                }
-            }
+            if (k < n - 1 && e.on) publish(e, cp, (k & 1) ? xb : xa, (k & 1) != 0, dn);
             barrier();
         }
         if (n > 1 && e.slot >= 0) add_correction(e, dk, round);
     }
 
-    __device__ __forceinline__ static void st_remote(unsigned addr, const VF& v) {
-        static_assert(CPL == 2, "a pair of columns");
-        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.v[0]), "f"(v.v[1]) : "memory");
-    }
     // u' += d * ||res|| (a non-finite correction is dropped, as in k_refine_add)
     __device__ __forceinline__ void add_correction(const Elem& e, const VF& d, int round) {
         Cols<CPL> x{};
