@@ -355,16 +355,18 @@ struct Slice {   // CPL: columns per lane
     // round: 13 columns of 144 atoms, four CTAs per slice, 36.9 -> 34.8 ms per
     // call; with S in shared memory and one element per thread too, a
     // charge-self-consistent call of 48 water molecules 42.6 -> 40.9 ms (the row
-    // itself kept across steps: 40.5, but a batch of boxes 26.0 -> 26.5).  With
+    // itself kept across steps: 40.5, but a batch of boxes 26.0 -> 26.5); FP64,
+    // one column of 64 atoms 36.2 -> 34.6, 48 of 216 atoms 107.3 -> 105.9.  With
     // four columns per lane the registers are full (512 atoms: 109.0 -> 110.0
     // ms), and every copy is looked up at its store.
-    static constexpr int REMOTE = CPL == 2 ? 3 : 0;
+    static constexpr int REMOTE = CPL <= 2 ? 3 : 0;
     struct Copies {
         unsigned at[REMOTE + 1];
         unsigned to_b;
         int n, first;
     };
-    __device__ __forceinline__ Copies copies(const Elem& e, VF* xa, VF* xb) {
+    template <class V>
+    __device__ __forceinline__ Copies copies(const Elem& e, V* xa, V* xb) {
         Copies c;
         c.n = c.first = 0;
         c.to_b = (unsigned)(reinterpret_cast<unsigned char*>(xb) - reinterpret_cast<unsigned char*>(xa));
@@ -384,8 +386,15 @@ struct Slice {   // CPL: columns per lane
         }
         return c;
     }
+    __device__ __forceinline__ static void st_remote(unsigned at, double v) {
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory");
+    }
+    __device__ __forceinline__ static void st_remote(unsigned at, const VF& v) {
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(at), "f"(v.v[0]), "f"(v.v[CPL - 1]) : "memory");
+    }
     // bcast(to, ...) of a row whose copies are known; to: xa, or xb (b)
-    __device__ __forceinline__ void publish(const Elem& e, const Copies& c, VF* to, bool b, const VF& v) {
+    template <class V>
+    __device__ __forceinline__ void publish(const Elem& e, const Copies& c, V* to, bool b, const V& v) {
         if constexpr (REMOTE == 0) {
             bcast(to, e.row, LPS, e.q, v);
         } else {
@@ -393,10 +402,7 @@ struct Slice {   // CPL: columns per lane
             const unsigned off = b ? c.to_b : 0u;
 #pragma unroll
             for (int i = 0; i < REMOTE; ++i)
-                if (i < c.n)
-                    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(c.at[i] + off), "f"(v.v[0]),
-                                 "f"(v.v[1])
-                                 : "memory");
+                if (i < c.n) st_remote(c.at[i] + off, v);
             for (int i = REMOTE; i < c.n; ++i) {
                 const int d = dest[c.first + i];
                 *cg::this_cluster().map_shared_rank(to + ((size_t)(d & 0xffff) * 4 + (e.row & 3)) * LPS + e.q, d >> 16) = v;
@@ -952,6 +958,8 @@ struct Slice {   // CPL: columns per lane
                 if (n == 1) xs[e0 + tid] += a.gamma64 * f;
             }
             barrier();
+            const bool single = nel_pad <= T;
+            const Copies cp = copies(elem(0), xa, xb);
             for (int k = 1; k < n; ++k) {
                 const double* cur = (k & 1) ? xa : xb;
                 double* io = (k & 1) ? xb : xa;
@@ -965,6 +973,7 @@ struct Slice {   // CPL: columns per lane
                     const double dc = cur[i], dp = k == 1 ? 0.0 : io[i];
                     const double dn = e.slot < 0 ? 0.0 : dp + w * (a.gamma64 * (fb[e0 + tid] - y) + dc - dp);
                     if (k == n - 1) xs[e0 + tid] += dn;
+                    else if (single) publish(e, cp, io, (k & 1) != 0, dn);
                     else bcast(io, e.row, NC, e.q, dn);
                 }
                 barrier();

@@ -73,6 +73,28 @@ def test_fixed_steps_equal_the_panel_path(P, case, monkeypatch, prec, nc, cl, re
     assert st["outer_iterations"] == st0["outer_iterations"] and st["switches"] == st0["switches"]
 
 
+@pytest.mark.parametrize("prec,nc,cl,reg", [(1, 2, 8, 1), (1, 4, 16, 0), (1, 2, 6, 0), (0, 1, 16, 0), (0, 2, 5, 0)])
+def test_rows_with_more_copies_than_a_lane_keeps(P, monkeypatch, prec, nc, cl, reg):
+    """A lane keeps the remote addresses of its row's first three copies; in
+    larger clusters of a small system a row has up to cl - 1 of them.  Two
+    bitwise equal runs (a copy stored late or to the wrong place shows there
+    too) that agree with the panel path after fixed steps to 1e-9, as above."""
+    s = SYSTEMS["si64"]()
+    h = P.tb_create_system(s)
+    z, w = _grid(s)
+    cols = np.array([0, 101, 255], dtype=np.int32)
+    opts = P.tb_default_opts(precision=prec, max_iter=12, panel=4)
+    monkeypatch.setenv("TB_SLICE", "0")
+    ref = P.tb_shifted_cocg(h, z, cols, opts=opts, allow_unconverged=True)[0].cpu().numpy()
+    monkeypatch.setenv("TB_SLICE", "1")
+    monkeypatch.setenv("TB_SLICE_NC", str(nc))
+    monkeypatch.setenv("TB_SLICE_CL", str(cl))
+    monkeypatch.setenv("TB_SLICE_REG", str(reg))
+    x, y = (P.tb_shifted_cocg(h, z, cols, opts=opts, allow_unconverged=True)[0].cpu().numpy() for _ in range(2))
+    assert np.array_equal(x, y)
+    assert np.abs(x - ref).max() <= 1e-9 * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
 @pytest.mark.parametrize("R,block", [(1, 0), (3, 32), (16, 64)])
 def test_outputs_against_dense(P, small, monkeypatch, prec, R, block):
