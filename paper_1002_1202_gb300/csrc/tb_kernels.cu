@@ -809,18 +809,18 @@ __device__ void inner32_ticket_tail(const PanelDev& p, int it) {
 }
 
 // w = S r (FP32) and the sums gamma = r.r, delta = w.r of every real column.
-// CPT column pairs per thread (2: one float4 per orbital row), C / CPT
-// threads per block row; the block-column index of the next block is loaded
-// one block ahead so the panel-row gathers do not wait on it.
-// PW: the panel's pair count as a compile-time constant (4 ... 128: row strides
-// fold into the load offsets; measured 4 % faster at 256 pairs), 0 for
-// any width at run time.
-template <int CPT, int PW = 0>
+// CPT column pairs per thread (2: one float4 per orbital row; 1 in panels of
+// fewer than 32 columns, see launch_inner32_spmv), C / CPT threads per block
+// row; the block-column index of the next block is loaded one block ahead so
+// the panel-row gathers do not wait on it.
+// PW: the panel's pair count (a compile-time constant: row strides fold into
+// the load offsets; measured 4 % faster at 256 pairs).
+template <int CPT, int PW>
 __global__ void __launch_bounds__(THREADS, 4) k_inner32_spmv(DevSystem s, PanelDev p, int it) {
     __shared__ double smem[4 * CPT * THREADS];
     if (*(volatile int*)&p.flags[1] == 0) return;
-    const int C = PW > 0 ? PW : p.C;
-    const int TPR = C / CPT;                    // threads per block row
+    constexpr int C = PW;
+    constexpr int TPR = C / CPT;                // threads per block row
     const int t0 = threadIdx.x % TPR;
     const int c0 = t0 * CPT;
     const InnerState* base = p.inner32;
@@ -1155,21 +1155,20 @@ __device__ __forceinline__ bool cheb_live(const PanelDev& p, int c) {
 
 // One Chebyshev step: io <- io + omega (gamma (f - S cur) + cur - io) on the
 // own rows, with S cur gathered as in k_inner32_spmv (CPT column pairs
-// per thread, C / CPT threads per block row, PW the pair count when it is
-// a compile-time constant).  mode 1: the first step (d_0 = 0, io is not
-// read).  mode 2 (the LAST instance): the last step, which adds its result
-// to the FP64 solution of the refinement instead of storing it
-// (x += d_n / scale and the double-float split, as k_refine_add; a
-// non-finite value is dropped).  When every diagonal block of S is the
+// per thread, C / CPT threads per block row, PW the pair count).  mode 1: the
+// first step (d_0 = 0, io is not read).  mode 2 (the LAST instance): the last
+// step, which adds its result to the FP64 solution of the refinement instead
+// of storing it (x += d_n / scale and the double-float split, as
+// k_refine_add; a non-finite value is dropped).  When every diagonal block of S is the
 // identity (s.unit_diag: orthonormal orbitals on one atom), the gather skips
 // it and S cur = (S - 1) cur + cur takes the own rows of cur, which the
 // update reads anyway: one block of ~17 per block row fewer to gather.
-template <int CPT, int PW = 0, bool LAST = false>
+template <int CPT, int PW, bool LAST = false>
 __global__ void __launch_bounds__(THREADS, 4) k_inner32_cheb(DevSystem s, PanelDev p, const float2* __restrict__ cur,
                                                             float2* io, float omega, float gamma, int mode) {
     if (*(volatile int*)&p.flags[4] == 0) return;
-    const int C = PW > 0 ? PW : p.C;
-    const int TPR = C / CPT;
+    constexpr int C = PW;
+    constexpr int TPR = C / CPT;
     const int t0 = threadIdx.x % TPR;
     const int c0 = t0 * CPT;
     bool live = false;
@@ -2761,7 +2760,11 @@ void launch_inner32_spmv(const DevSystem& s, const PanelDev& p, int it, cudaStre
     LaunchScope ls_(K_INNER32_SPMV, st);
     // the grouped form wins on narrow panels (measured on the Si 4096-atom
     // system: 28 vs 35 us at 64 columns); from 128 columns on, the
-    // register-gather form with its higher occupancy is faster
+    // register-gather form with its higher occupancy is faster.  Panels of
+    // fewer than 32 columns take one pair per thread: with two a block row has
+    // so few threads that a step waits on its chain of gathers with half the
+    // warps in flight (8 outer steps, 4 / 16 columns of 1000 silicon atoms
+    // 14.7 / 15.6 -> 11.4 / 12.2 ms, 16 of 512 water molecules 29.1 -> 19.5)
     if (s.grpG > 0 && p.C >= PC && p.C <= 64) {
         const size_t sm = inner32_grp_smem(s);
         static const bool attr = [] {
@@ -2775,24 +2778,28 @@ void launch_inner32_spmv(const DevSystem& s, const PanelDev& p, int it, cudaStre
         }();
         (void)attr;
         k_inner32_spmv_grp<<<s.n_groups * (p.C / PC), s.grpG * (PC / 2), sm, st>>>(s, p, it);
-    } else if (p.C >= 2) {
+    } else if (p.C >= 16) {
         const int g = grid_for((long long)s.n_atoms * (p.C / 2));
         switch (p.C) {
             case 128: k_inner32_spmv<2, 128><<<g, THREADS, 0, st>>>(s, p, it); break;
             case 64: k_inner32_spmv<2, 64><<<g, THREADS, 0, st>>>(s, p, it); break;
             case 32: k_inner32_spmv<2, 32><<<g, THREADS, 0, st>>>(s, p, it); break;
-            case 16: k_inner32_spmv<2, 16><<<g, THREADS, 0, st>>>(s, p, it); break;
-            case 8: k_inner32_spmv<2, 8><<<g, THREADS, 0, st>>>(s, p, it); break;
-            case 4: k_inner32_spmv<2, 4><<<g, THREADS, 0, st>>>(s, p, it); break;
-            default: k_inner32_spmv<2><<<g, THREADS, 0, st>>>(s, p, it); break;
+            default: k_inner32_spmv<2, 16><<<g, THREADS, 0, st>>>(s, p, it); break;
+        }
+    } else {
+        const int g = grid_for((long long)s.n_atoms * p.C);
+        switch (p.C) {
+            case 8: k_inner32_spmv<1, 8><<<g, THREADS, 0, st>>>(s, p, it); break;
+            case 4: k_inner32_spmv<1, 4><<<g, THREADS, 0, st>>>(s, p, it); break;
+            case 2: k_inner32_spmv<1, 2><<<g, THREADS, 0, st>>>(s, p, it); break;
+            default: k_inner32_spmv<1, 1><<<g, THREADS, 0, st>>>(s, p, it); break;
         }
     }
-    else
-        k_inner32_spmv<1><<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, it);
 }
 // TB_CHEB_CPT=2 / 4 forces the two- or four-pairs-per-thread form of the
-// Chebyshev step (panels narrower than 8 columns always take the two-pair
-// form); tb_autotune's choice for the call's size class comes first
+// Chebyshev step (panels of fewer than 16 columns take one pair per thread
+// with 2, and of fewer than 8 with 4 too); tb_autotune's choice for the call's
+// size class comes first
 static const int g_cheb_cpt_env = [] {
     const char* e = std::getenv("TB_CHEB_CPT");
     return e ? std::atoi(e) : 0;
@@ -2865,20 +2872,26 @@ static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur
         else if (p.C == 16) done = chebs_launch<16, LAST>(s, p, cur, io, omega, gamma, mode, st);
         if (done) return;
     }
-    if (p.C >= 2) {
+    // fewer than 16 columns: one pair per thread, for the warps in flight (16
+    // outer steps, 4 / 8 columns of 1000 silicon atoms 16.0 / 14.0 -> 11.4 /
+    // 10.1 ms, 4 of 512 water molecules 39.7 -> 25.7, panels of 8 for 256 of
+    // them 240 -> 184; 8 columns of 100 000 atoms, 4 steps, 17.7)
+    if (p.C >= 8) {
         const int g = grid_for((long long)s.n_atoms * (p.C / 2));
         switch (p.C) {
             case 128: k_inner32_cheb<2, 128, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 64: k_inner32_cheb<2, 64, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 32: k_inner32_cheb<2, 32, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 16: k_inner32_cheb<2, 16, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
-            case 8: k_inner32_cheb<2, 8, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
-            case 4: k_inner32_cheb<2, 4, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
-            default: k_inner32_cheb<2, 0, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+            default: k_inner32_cheb<2, 8, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
         }
     } else {
-        k_inner32_cheb<1, 0, LAST><<<grid_for((long long)s.n_atoms * p.C), THREADS, 0, st>>>(s, p, cur, io, omega,
-                                                                                          gamma, mode);
+        const int g = grid_for((long long)s.n_atoms * p.C);
+        switch (p.C) {
+            case 4: k_inner32_cheb<1, 4, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+            case 2: k_inner32_cheb<1, 2, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+            default: k_inner32_cheb<1, 1, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+        }
     }
 }
 void launch_inner32_cheb(const DevSystem& s, const PanelDev& p, const float2* cur, float2* io, float omega,

@@ -1,0 +1,77 @@
+"""The panel kernels, which solve every system above the column slices' size,
+on small systems (TB_SLICE=0): every panel width, so every form of the
+Chebyshev step and of the FP32 CG product (one, two and four column pairs per
+thread, S staged in shared memory or not), full and partly filled CTAs,
+systems of s-only atoms.  Each test checks from the launch counters that the
+slices took no part."""
+import numpy as np
+import pytest
+
+from tbinputs import gauss_legendre_grid, si_system, water_system
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1002_1202_gb300 as pkg
+    pkg.build()
+    return pkg
+
+
+def launches(P):
+    return {k: P.tb_profile_read(k)[0] for k in P.tb.KERNELS}
+
+
+@pytest.fixture
+def ran(P, monkeypatch):
+    """Counts the launches of a test per kernel class, on the panel kernels only."""
+    monkeypatch.setenv("TB_SLICE", "0")
+    before = launches(P)
+
+    def delta():
+        return {k: n - before[k] for k, n in launches(P).items()}
+
+    yield delta
+    assert delta()["slice"] == 0
+
+
+# 64 atoms of silicon (identity diagonal blocks, 17 blocks a row: S staged) and
+# 99 of water (s and sp atoms, rows too long to stage in the narrower panels, a
+# last CTA with fewer rows in every form)
+SYSTEMS = {"si64": lambda: si_system((2, 2, 2), sigma=0.05, seed=1),
+           "water33": lambda: water_system(33, seed=6, excess_proton=False)}
+STEPS = 12
+
+
+@pytest.fixture(scope="module", params=list(SYSTEMS))
+def case(request, P):
+    s = SYSTEMS[request.param]()
+    h = P.tb_create_system(s)
+    lo, hi = (-20.0, 5.0) if s.eps.min() > -20 else (-40.0, 0.0)
+    z, _ = gauss_legendre_grid(6, lo, hi, 1.0)
+    cols = np.random.default_rng(3).permutation(s.n_orb)[:256].astype(np.int32)
+    mp = pytest.MonkeyPatch()
+    mp.setenv("TB_SLICE", "0")
+    ref = P.tb_shifted_cocg(h, z, cols, opts=P.tb_default_opts(max_iter=STEPS, panel=64),
+                            allow_unconverged=True)[0].cpu().numpy()
+    mp.undo()
+    return h, z, cols, ref
+
+
+@pytest.mark.parametrize("method", [0, 1], ids=["chebyshev", "cg"])
+@pytest.mark.parametrize("panel", [1, 2, 4, 8, 16, 32, 64, 128, 256])
+def test_panel_widths(P, case, ran, panel, method):
+    """A fixed number of outer steps of full solutions, mixed precision, for
+    every panel width against the FP64 panels of 64 columns: the same
+    recurrences with inner solves to 1e-13, so they agree to 1e-9 as the slices
+    and the panels do."""
+    h, z, cols, ref = case
+    n = min(panel, len(cols))
+    opts = P.tb_default_opts(precision=1, inner_method=method, max_iter=STEPS, panel=panel)
+    x = P.tb_shifted_cocg(h, z, cols[:n], opts=opts, allow_unconverged=True)[0].cpu().numpy()
+    assert np.abs(x - ref[:, :n]).max() <= 1e-9 * np.abs(ref).max()
+    assert ran()["inner32_cheb" if method == 0 else "inner32_spmv"] > 0
