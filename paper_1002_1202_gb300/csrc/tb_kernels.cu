@@ -2004,107 +2004,109 @@ __global__ void k_mulliken_output(PanelDev p, int ncols, const double2* __restri
 }
 
 // ---------------------------------------------------------------------------
-// Generalized Lanczos helpers (Section 3.2), one real vector stored in the
-// real part of a P = 1 panel column.
-// ---------------------------------------------------------------------------
 // Generalized Lanczos on a panel of P columns (Section 3.2), one independent
-// process per column; vectors [npad][C] pairs of columns.
-// y = M x for M = H or S
-__global__ void k_lz_spmv(DevSystem s, const double* __restrict__ M, const double2* __restrict__ x,
-                          double2* __restrict__ y, int C) {
-    const long long items = (long long)s.n_atoms * C;
+// process per column; vectors [npad][P].
+// ---------------------------------------------------------------------------
+// y = M x for M = H or S, W columns per thread (1, or the 2 of a pair)
+template <int W>
+__global__ void k_lz_spmv(DevSystem s, const double* __restrict__ M, const double* __restrict__ x,
+                          double* __restrict__ y, int P) {
+    const int TPR = P / W;
+    const long long items = (long long)s.n_atoms * TPR;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * blockDim.x) {
-        const int I = (int)(idx / C), c = (int)(idx % C);
-        double2 acc[4];
+        const int I = (int)(idx / TPR), c = W * (int)(idx % TPR);
+        double acc[4][W];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) acc[a] = make_double2(0.0, 0.0);
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int j = 0; j < W; ++j) acc[a][j] = 0.0;
         for (int b = s.brow[I]; b < s.brow[I + 1]; ++b) {
-            const int J = s.bcol[b];
-            double2 xv[4];
+            const double* xb = x + (size_t)(4 * s.bcol[b]) * P + c;
+            double xv[4][W];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xv[e] = x[(size_t)(4 * J + e) * C + c];
+            for (int e = 0; e < 4; ++e) {
+                if (W == 2) {
+                    const double2 q = *reinterpret_cast<const double2*>(xb + (size_t)e * P);
+                    xv[e][0] = q.x;
+                    xv[e][W - 1] = q.y;
+                } else {
+                    xv[e][0] = xb[(size_t)e * P];
+                }
+            }
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const double m = M[16 * (size_t)b + 4 * a + e];
-                    acc[a].x += m * xv[e].x;
-                    acc[a].y += m * xv[e].y;
+#pragma unroll
+                    for (int j = 0; j < W; ++j) acc[a][j] += m * xv[e][j];
                 }
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) y[(size_t)(4 * I + a) * C + c] = acc[a];
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int j = 0; j < W; ++j) y[(size_t)(4 * I + a) * P + c + j] = acc[a][j];
     }
 }
 
 // out[c * stride] = x_c^T y_c (mode 0) or sqrt(x_c^T y_c) (mode 1) for column c < P
-__global__ void __launch_bounds__(THREADS) k_lz_dot(PanelDev p, const double2* __restrict__ x,
-                                                    const double2* __restrict__ y, double* out, int stride, int mode) {
-    __shared__ double smem[2 * THREADS];
-    const int C = p.C;
-    double v[2] = {0.0, 0.0};
-    const long long items = (long long)p.npad * C;
-    for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
-        const double2 a = x[i], b = y[i];
-        v[0] += a.x * b.x;
-        v[1] += a.y * b.y;
-    }
-    if (grid_reduce_cols<2>(v, C, p, smem)) {
-        for (int c = threadIdx.x; c < p.P; c += THREADS) {
-            const double t = smem[(c & 1) * THREADS + (c >> 1)];
-            out[(size_t)c * stride] = (mode == 0) ? t : sqrt(fmax(t, 0.0));
+__global__ void __launch_bounds__(THREADS) k_lz_dot(PanelDev p, const double* __restrict__ x,
+                                                    const double* __restrict__ y, double* out, int stride, int mode) {
+    __shared__ double smem[THREADS];
+    const int P = p.P;
+    double v[1] = {0.0};
+    const long long items = (long long)p.npad * P;
+    for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS)
+        v[0] += x[i] * y[i];
+    if (grid_reduce_cols<1>(v, P, p, smem)) {
+        if (threadIdx.x < P) {
+            const double t = smem[threadIdx.x];
+            out[(size_t)threadIdx.x * stride] = (mode == 0) ? t : sqrt(fmax(t, 0.0));
         }
     }
 }
 
 // u_c = v_c / sqrt(n2_c), n2_c = v[row_c][c] = e_j^T S^-1 e_j (inactive columns: u = 0)
-__global__ void k_lz_start(PanelDev p, const double2* __restrict__ v, double2* __restrict__ u, double* nrm2) {
+__global__ void k_lz_start(PanelDev p, const double* __restrict__ v, double* __restrict__ u, double* nrm2) {
     const int P = p.P;
-    const double* vv = reinterpret_cast<const double*>(v);
-    double* uu = reinterpret_cast<double*>(u);
     const long long items = (long long)p.npad * P;
     for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
         const int c = (int)(i % P);
         const ColState& cs = p.col[c];
         if (!cs.active) {
-            uu[i] = 0.0;
+            u[i] = 0.0;
             continue;
         }
-        const double n2 = vv[(size_t)cs.row * P + c];
-        uu[i] = vv[i] / sqrt(n2);
+        const double n2 = v[(size_t)cs.row * P + c];
+        u[i] = v[i] / sqrt(n2);
         if (i / P == 0) nrm2[c] = n2;
     }
 }
 
 // w = y - a_c u - b_c u_prev
-__global__ void k_lz_combine(PanelDev p, const double2* __restrict__ y, const double2* __restrict__ u,
-                             const double2* __restrict__ up, double2* __restrict__ w, const double* a,
+__global__ void k_lz_combine(PanelDev p, const double* __restrict__ y, const double* __restrict__ u,
+                             const double* __restrict__ up, double* __restrict__ w, const double* a,
                              const double* b, int sa, int sb) {
-    const int C = p.C;
-    const long long items = (long long)p.npad * C;
+    const int P = p.P;
+    const long long items = (long long)p.npad * P;
     for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
-        const int c = 2 * (int)(i % C);
-        const double2 yv = y[i], uv = u[i], pv = up[i];
-        w[i] = make_double2(yv.x - a[(size_t)c * sa] * uv.x - b[(size_t)c * sb] * pv.x,
-                            yv.y - a[(size_t)(c + 1) * sa] * uv.y - b[(size_t)(c + 1) * sb] * pv.y);
+        const int c = (int)(i % P);
+        w[i] = y[i] - a[(size_t)c * sa] * u[i] - b[(size_t)c * sb] * up[i];
     }
 }
 
 // u_prev = u, u = w / b_c (0 when b_c = 0: invariant subspace found)
-__global__ void k_lz_scale(PanelDev p, const double2* __restrict__ w, double2* __restrict__ u,
-                           double2* __restrict__ up, const double* bnext, int sb) {
-    const int C = p.C;
-    const long long items = (long long)p.npad * C;
+__global__ void k_lz_scale(PanelDev p, const double* __restrict__ w, double* __restrict__ u,
+                           double* __restrict__ up, const double* bnext, int sb) {
+    const int P = p.P;
+    const long long items = (long long)p.npad * P;
     for (long long i = blockIdx.x * (long long)THREADS + threadIdx.x; i < items; i += (long long)gridDim.x * THREADS) {
-        const int c = 2 * (int)(i % C);
-        const double b0 = bnext[(size_t)c * sb], b1 = bnext[(size_t)(c + 1) * sb];
-        const double2 wv = w[i];
+        const double bv = bnext[(size_t)(i % P) * sb];
         up[i] = u[i];
-        u[i] = make_double2(b0 > 0.0 ? wv.x / b0 : 0.0, b1 > 0.0 ? wv.y / b1 : 0.0);
+        u[i] = bv > 0.0 ? w[i] / bv : 0.0;
     }
 }
-
 
 // ---------------------------------------------------------------------------
 // Charge self-consistency (Section 2.2, Eq. Hap-CSC)
@@ -2660,7 +2662,7 @@ static int grid_for(long long items) {
 // not placed yet), so that the call's first launches need no device memory.
 bool preload_noalloc_kernels() {
     const void* ks[] = {(const void*)k_panel_init, (const void*)k_inner_spmv, (const void*)k_inner_update,
-                        (const void*)k_lz_start,   (const void*)k_lz_spmv,    (const void*)k_lz_dot,
+                        (const void*)k_lz_start,   (const void*)k_lz_spmv<1>, (const void*)k_lz_dot,
                         (const void*)k_lz_combine, (const void*)k_lz_scale};
     for (const void* k : ks) {
         cudaFuncAttributes fa;
@@ -3029,28 +3031,39 @@ void launch_mulliken_output(const PanelDev& p, int ncols, const double2* w, doub
         k_mulliken_output<<<p.P, THREADS, 0, st>>>(p, ncols, w, g_s, out);
     }
 }
+static const double* cols_of(const double2* v) { return reinterpret_cast<const double*>(v); }
+static double* cols_of(double2* v) { return reinterpret_cast<double*>(v); }
 void launch_lz_spmv(const DevSystem& s, const double* M, const double2* x, double2* y, int C, cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_spmv<<<grid_for((long long)s.n_atoms * C), THREADS, 0, st>>>(s, M, x, y, C);
+    // One column per thread until pairs fill half of the resident threads: below
+    // that the threads, each a chain of FP64 sums, are too few (per call, pairs /
+    // columns: 20 steps of one column of 1000 atoms 66.9 / 65.9 ms, 24 of 16
+    // columns of 1728 atoms 17.9 / 17.1; of 128 columns 23.2 / 23.9)
+    const long long pairs = (long long)s.n_atoms * C;
+    if (2 * pairs >= (long long)gmax() * THREADS)
+        k_lz_spmv<2><<<grid_for(pairs), THREADS, 0, st>>>(s, M, cols_of(x), cols_of(y), 2 * C);
+    else
+        k_lz_spmv<1><<<grid_for(2 * pairs), THREADS, 0, st>>>(s, M, cols_of(x), cols_of(y), 2 * C);
 }
 void launch_lz_dot(const PanelDev& p, const double2* x, const double2* y, double* out, int stride, int mode,
                    cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_dot<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, x, y, out, stride, mode);
+    k_lz_dot<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, cols_of(x), cols_of(y), out, stride, mode);
 }
 void launch_lz_combine(const PanelDev& p, const double2* y, double2* u, double2* u_prev, double2* w,
                        const double* a, const double* b, int sa, int sb, cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_combine<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, y, u, u_prev, w, a, b, sa, sb);
+    k_lz_combine<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, cols_of(y), cols_of(u), cols_of(u_prev),
+                                                                         cols_of(w), a, b, sa, sb);
 }
 void launch_lz_scale(const PanelDev& p, double2* w, double2* u, double2* u_prev, const double* bnext, int sb,
                      cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_scale<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, w, u, u_prev, bnext, sb);
+    k_lz_scale<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, cols_of(w), cols_of(u), cols_of(u_prev), bnext, sb);
 }
 void launch_lz_start(const PanelDev& p, const double2* v, double2* u, double* nrm2, cudaStream_t st) {
     LaunchScope ls_(K_OTHER, st);
-    k_lz_start<<<grid_for((long long)p.npad * p.C), THREADS, 0, st>>>(p, v, u, nrm2);
+    k_lz_start<<<grid_for((long long)p.npad * p.P), THREADS, 0, st>>>(p, cols_of(v), cols_of(u), nrm2);
 }
 
 

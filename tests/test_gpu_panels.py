@@ -75,3 +75,21 @@ def test_panel_widths(P, case, ran, panel, method):
     x = P.tb_shifted_cocg(h, z, cols[:n], opts=opts, allow_unconverged=True)[0].cpu().numpy()
     assert np.abs(x - ref[:, :n]).max() <= 1e-9 * np.abs(ref).max()
     assert ran()["inner32_cheb" if method == 0 else "inner32_spmv"] > 0
+
+
+@pytest.mark.parametrize("R,prec", [(1, 0), (2, 0), (7, 1), (64, 1), (256, 1)])
+def test_lanczos_widths(P, R, prec):
+    """The Lanczos process of R columns at once (one column per thread of its
+    products, a pair from 256 columns of 640 atoms on) against the single-column
+    call: the coefficients of 10 steps to 1e-8, as the existing batch checks."""
+    s = si_system((4, 4, 5), sigma=0.05, seed=2)
+    h = P.tb_create_system(s)
+    cols = np.random.default_rng(R).permutation(s.n_orb)[:R].astype(np.int32)
+    a, b, nrm = (np.asarray(v.cpu() if hasattr(v, "cpu") else v)
+                 for v in P.tb_generalized_lanczos_batch(h, cols, 10, opts=P.tb_default_opts(precision=prec)))
+    for c in sorted({0, R // 2, R - 1}):
+        a0, b0, n0 = (np.asarray(v.cpu() if hasattr(v, "cpu") else v)
+                      for v in P.tb_generalized_lanczos(h, int(cols[c]), 10))
+        assert np.abs(a[c] - a0).max() <= 1e-8 * np.abs(a0).max()
+        assert np.abs(b[c] - b0).max() <= 1e-8 * np.abs(b0).max()
+        assert abs(nrm[c] - np.ravel(n0)[0]) <= 1e-10 * abs(np.ravel(n0)[0])
