@@ -396,38 +396,37 @@ __global__ void __launch_bounds__(THREADS) k_inner_spmv(DevSystem s, PanelDev p,
         }
     }
     if (grid_reduce_cols<4>(v, C, p, smem)) {
-        const int t = threadIdx.x;
+        // one thread per column: a column's divisions are a chain of ~2000 cycles
+        const int t = threadIdx.x, pair = t >> 1, part = t & 1;
         int nact = 0;
-        if (t < C) {
-            for (int part = 0; part < 2; ++part) {
-                const bool cact = p.col[2 * t + part].active != 0;
-                if (it == 0 && cact) p.col[2 * t + part].rnorm = sqrt(smem[part * THREADS + t]);
-                InnerState st = p.inner[2 * t + part];
-                const double gam = smem[part * THREADS + t];
-                const double del = smem[(2 + part) * THREADS + t];
-                if (it == 0) {
-                    st.bnorm2 = gam;
-                    st.conv = (!cact || gam == 0.0) ? 1 : 0;
-                }
-                if (!st.conv) {
-                    if (gam <= p.inner_tol * p.inner_tol * st.bnorm2) {
+        if (t < p.P) {
+            const bool cact = p.col[t].active != 0;
+            if (it == 0 && cact) p.col[t].rnorm = sqrt(smem[part * THREADS + pair]);
+            InnerState st = p.inner[t];
+            const double gam = smem[part * THREADS + pair];
+            const double del = smem[(2 + part) * THREADS + pair];
+            if (it == 0) {
+                st.bnorm2 = gam;
+                st.conv = (!cact || gam == 0.0) ? 1 : 0;
+            }
+            if (!st.conv) {
+                if (gam <= p.inner_tol * p.inner_tol * st.bnorm2) {
+                    st.conv = 1;
+                } else {
+                    const double beta = (it == 0) ? 0.0 : gam / st.gamma_prev;
+                    const double den = del - ((it == 0) ? 0.0 : beta * gam / st.alpha);
+                    if (!(den > 0.0)) {
+                        atomicOr(&p.flags[0], ERR_NOT_SPD);
                         st.conv = 1;
                     } else {
-                        const double beta = (it == 0) ? 0.0 : gam / st.gamma_prev;
-                        const double den = del - ((it == 0) ? 0.0 : beta * gam / st.alpha);
-                        if (!(den > 0.0)) {
-                            atomicOr(&p.flags[0], ERR_NOT_SPD);
-                            st.conv = 1;
-                        } else {
-                            st.alpha = gam / den;
-                            st.beta = beta;
-                            st.gamma_prev = gam;
-                        }
+                        st.alpha = gam / den;
+                        st.beta = beta;
+                        st.gamma_prev = gam;
                     }
                 }
-                nact += st.conv ? 0 : 1;
-                p.inner[2 * t + part] = st;
             }
+            nact += st.conv ? 0 : 1;
+            p.inner[t] = st;
         }
         // count unconverged real columns
         __shared__ int s_cnt;
@@ -517,21 +516,19 @@ __global__ void __launch_bounds__(THREADS) k_refine_start(PanelDev p, const doub
         }
     }
     if (grid_reduce_cols<2>(v, C, p, smem)) {
-        const int t = threadIdx.x;
+        const int t = threadIdx.x, pair = t >> 1, part = t & 1;
         int nact = 0;
-        if (t < C) {
-            for (int part = 0; part < 2; ++part) {
-                const bool cact = p.col[2 * t + part].active != 0;
-                if (cact) p.col[2 * t + part].rnorm = sqrt(smem[part * THREADS + t]);
-                const double b2 = smem[part * THREADS + t];
-                p.inner[2 * t + part].bnorm2 = b2;
-                InnerState st = p.inner32[2 * t + part];
-                st.skip = (!cact || b2 == 0.0) ? 1 : 0;
-                st.unscale = st.skip ? 0.0 : sqrt(b2);
-                st.scale = st.skip ? 0.0 : 1.0 / st.unscale;
-                p.inner32[2 * t + part] = st;
-                nact += st.skip ? 0 : 1;
-            }
+        if (t < p.P) {
+            const bool cact = p.col[t].active != 0;
+            if (cact) p.col[t].rnorm = sqrt(smem[part * THREADS + pair]);
+            const double b2 = smem[part * THREADS + pair];
+            p.inner[t].bnorm2 = b2;
+            InnerState st = p.inner32[t];
+            st.skip = (!cact || b2 == 0.0) ? 1 : 0;
+            st.unscale = st.skip ? 0.0 : sqrt(b2);
+            st.scale = st.skip ? 0.0 : 1.0 / st.unscale;
+            p.inner32[t] = st;
+            nact += st.skip ? 0 : 1;
         }
         refine_finish_counts(p, nact);
     }
@@ -603,31 +600,29 @@ __global__ void __launch_bounds__(THREADS) k_refine_residual(DevSystem s, PanelD
         }
     }
     if (grid_reduce_cols<2>(v, C, p, smem)) {
-        const int t = threadIdx.x;
+        const int t = threadIdx.x, pair = t >> 1, part = t & 1;
         int nact = 0;
-        if (t < C) {
-            for (int part = 0; part < 2; ++part) {
-                const bool cact = p.col[2 * t + part].active != 0;
-                InnerState st = p.inner32[2 * t + part];
-                if (!st.skip) {
-                    const double r2 = smem[part * THREADS + t];
-                    const double b2 = p.inner[2 * t + part].bnorm2;
-                    if (!isfinite(r2)) {
-                        atomicOr(&p.flags[0], ERR_INNER);
-                        if (p.dbg) {
-                            p.dbg[0] = -1.0; p.dbg[1] = 2 * t + part; p.dbg[2] = r2; p.dbg[3] = st.scale;
-                            p.dbg[4] = b2; p.dbg[5] = st.bnorm2; p.dbg[6] = st.gamma_prev; p.dbg[7] = st.alpha;
-                        }
-                        st.skip = 1;
-                    } else if (!cact || r2 <= p.inner_tol * p.inner_tol * b2 || r2 == 0.0) {
-                        st.skip = 1;
+        if (t < p.P) {
+            const bool cact = p.col[t].active != 0;
+            InnerState st = p.inner32[t];
+            if (!st.skip) {
+                const double r2 = smem[part * THREADS + pair];
+                const double b2 = p.inner[t].bnorm2;
+                if (!isfinite(r2)) {
+                    atomicOr(&p.flags[0], ERR_INNER);
+                    if (p.dbg) {
+                        p.dbg[0] = -1.0; p.dbg[1] = t; p.dbg[2] = r2; p.dbg[3] = st.scale;
+                        p.dbg[4] = b2; p.dbg[5] = st.bnorm2; p.dbg[6] = st.gamma_prev; p.dbg[7] = st.alpha;
                     }
-                    st.unscale = st.skip ? 0.0 : sqrt(r2);
-                    st.scale = st.skip ? 0.0 : 1.0 / st.unscale;
+                    st.skip = 1;
+                } else if (!cact || r2 <= p.inner_tol * p.inner_tol * b2 || r2 == 0.0) {
+                    st.skip = 1;
                 }
-                nact += st.skip ? 0 : 1;
-                p.inner32[2 * t + part] = st;
+                st.unscale = st.skip ? 0.0 : sqrt(r2);
+                st.scale = st.skip ? 0.0 : 1.0 / st.unscale;
             }
+            nact += st.skip ? 0 : 1;
+            p.inner32[t] = st;
         }
         refine_finish_counts(p, nact);
     }

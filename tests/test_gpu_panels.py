@@ -77,6 +77,17 @@ def test_panel_widths(P, case, ran, panel, method):
     assert ran()["inner32_cheb" if method == 0 else "inner32_spmv"] > 0
 
 
+@pytest.mark.parametrize("panel", [1, 8, 256])
+def test_fp64_panel_widths(P, case, ran, panel):
+    """The same in FP64: the scalars of the inner CG, one thread per column."""
+    h, z, cols, ref = case
+    n = min(panel, len(cols))
+    opts = P.tb_default_opts(max_iter=STEPS, panel=panel)
+    x = P.tb_shifted_cocg(h, z, cols[:n], opts=opts, allow_unconverged=True)[0].cpu().numpy()
+    assert np.abs(x - ref[:, :n]).max() <= 1e-9 * np.abs(ref).max()
+    assert ran()["inner_spmv"] > 0
+
+
 @pytest.mark.parametrize("R,prec", [(1, 0), (2, 0), (7, 1), (64, 1), (256, 1)])
 def test_lanczos_widths(P, R, prec):
     """The Lanczos process of R columns at once (one column per thread of its
