@@ -194,6 +194,7 @@ struct Solve {
     int streams = 0;                    // panels in flight
     int cheb_cpt = 0;                   // pairs of columns per thread of the Chebyshev step
     int columns = 0;                    // columns of the call solved at the same time (0: this solve's)
+    int inflight = 1;                   // panels of the call in flight
 };
 
 // What one solve sees of a system: the device arrays (a whole handle, or one
@@ -1050,6 +1051,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     p.mixed = o->precision == TB_MIXED ? 1 : 0;
     p.inner_lo_tol = o->inner_lo_tol;
     p.cheb_cpt = q.cheb_cpt;
+    p.inflight = q.inflight;
     const size_t nv = (size_t)npad * P;   // x^k, p^k: complex, one per column
     tb_status s;
     if ((s = alloc_inner_workspace(cl, p, st)) != TB_OK) return s;
@@ -1441,6 +1443,7 @@ tb_status run_jobs(tb_handle* h, const Solve& q, const tb_solve_opts* o, tb_stat
                 Solve q2 = q;
                 q2.R = Rq;
                 q2.columns = std::min(R, nw * (int)jobs[0].cols.size());
+                q2.inflight = nw;
                 q2.cols = cols.data();
                 std::vector<int64_t> rp2, gidx;
                 std::vector<int32_t> rows2;

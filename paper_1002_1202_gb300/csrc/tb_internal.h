@@ -179,6 +179,7 @@ struct PanelDev {
     int grid = 0;                 // CTAs of the grid-stride kernels
     int mixed = 0;                // 1: inner S^-1 by FP32 corrections inside FP64 refinement
     int cheb_cpt = 0;             // host side: pairs of columns per thread of the Chebyshev step (2 or 4; 0 = default)
+    int inflight = 1;             // host side: panels of the call in flight
     double tol = 1e-10, inner_tol = 1e-13, inner_lo_tol = 1e-6;
     int switching = 1, force_switch_every = 0;
     // panel vectors, [npad][C] pairs of columns: u_n, u_{n-1}, u'_n, W (and the

@@ -2844,16 +2844,24 @@ template <bool LAST>
 static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur, float2* io, float omega,
                         float gamma, int mode, cudaStream_t st) {
     // default form: two pairs per thread.  The step is bound by the latency of
-    // its gathers, so the form with twice the threads wins while the panel has
-    // fewer threads than the SMs can hold many times over (panels in pairs,
-    // 64 / 128 / 256 columns: 4096 atoms 159 / 158 / 193 ms per call against
-    // 170 / 169 / 202 with four; 1728 atoms 177 / 174 / 184 against 229 / 215 /
-    // 209; 24 Lanczos steps of 128 columns 40.0 / 24.9 ms against 56.2 / 32.1;
-    // prefetching the next block's rows into registers was slower in every
-    // form: 165-560 ms).  Four pairs for systems with s-only atoms, whose
-    // ragged form has them, and from eight waves of the four-pair form on
-    // (the 100 000-atom crystal from 64 columns on)
-    const bool wide = (s.rag && g_cheb_rag && p.C >= 16) || (long long)s.n_atoms * (p.C / 4) >= 8LL * 3 * (gmax() / 4) * THREADS;
+    // its gathers, so the form with twice the threads wins (64 / 128 / 256
+    // columns: 4096 atoms 159 / 158 / 193 ms per call against 170 / 169 / 202
+    // with four; 1728 atoms 177 / 174 / 184 against 229 / 215 / 209; 24 Lanczos
+    // steps of 128 columns 40.0 / 24.9 ms against 56.2 / 32.1; 100 000 atoms, 3
+    // outer steps of panels of 64 / 128 / 256 columns, one in flight 48.7 / 91.6 /
+    // 181 against 56.4 / 99.6 / 191, four 175 / 337 / 676 against 200 / 367 / 696;
+    // prefetching the next block's rows into registers was slower in every form:
+    // 165-560 ms).  Four pairs for systems with s-only atoms, whose ragged form
+    // has fewer gathers, once its panels in flight nearly fill the threads that the
+    // SMs hold (a wave), in wide panels earlier.  6 outer steps, ms, two / four
+    // pairs: 400 water molecules, panels of 64, 1 / 4 in flight 13.4 / 19.6 and
+    // 18.1 / 23.0 (0.08 and 0.3 waves); 800, panels of 64, 4 in flight 20.1 / 21.3
+    // (0.66); 1536, panels of 64, 1 / 2 / 4 in flight 13.8 / 18.1, 21.1 / 21.2 (0.6)
+    // and 34.7 / 29.0 (1.3), panels of 128, one in flight 19.9 / 18.2 (0.6); 512,
+    // panels of 256, one in flight 13.9 / 13.2 (0.4)
+    const double wave = 3.0 * (gmax() / 4) * THREADS;
+    const bool wide = s.rag && g_cheb_rag && p.C >= 16 &&
+                      (double)s.n_atoms * (p.C / 4) * p.inflight >= wave * std::min(0.9, 40.0 / p.C);
     const int cpt = p.cheb_cpt ? p.cheb_cpt : g_cheb_cpt_env ? g_cheb_cpt_env : (wide ? 4 : 2);
     if (cpt == 4 && p.C >= 4) {
         cheb4_launch<LAST>(s, p, cur, io, omega, gamma, mode, st);

@@ -104,3 +104,22 @@ def test_lanczos_widths(P, R, prec):
         assert np.abs(a[c] - a0).max() <= 1e-8 * np.abs(a0).max()
         assert np.abs(b[c] - b0).max() <= 1e-8 * np.abs(b0).max()
         assert abs(nrm[c] - np.ravel(n0)[0]) <= 1e-10 * abs(np.ravel(n0)[0])
+
+
+def test_ragged_and_padded_steps_of_a_large_box(P, ran):
+    """400 water molecules (2400 orbitals, above the slices' size): one panel of
+    256 columns takes the ragged four-pair step, four of 64 in flight and one of
+    64 the padded two-pair one; the same populations after fixed steps to 1e-9."""
+    s = water_system(400, seed=4, excess_proton=False)
+    h = P.tb_create_system(s)
+    z, w = gauss_legendre_grid(8, -60.0, -8.0, 1.0)
+    cols = np.random.default_rng(5).permutation(s.n_orb)[:256].astype(np.int32)
+
+    def q(n, panel):
+        o = P.tb_default_opts(precision=1, max_iter=8, panel=panel)
+        return P.tb_mulliken_orbital(h, z, w, cols[:n], 2.0, opts=o, allow_unconverged=True)[0].cpu().numpy()
+
+    wide, narrow, one = q(256, 256), q(256, 64), q(64, 64)
+    assert np.abs(wide - narrow).max() <= 1e-9 * np.abs(wide).max()
+    assert np.abs(wide[:64] - one).max() <= 1e-9 * np.abs(wide).max()
+    assert ran()["inner32_cheb"] > 0
