@@ -201,8 +201,11 @@ typedef struct {
                                  reach the same inner_tol.  Ignored for TB_FP64.        */
     int64_t state_bytes;      /* energy-point checkpointing: device bytes allowed for the
                                  full-vector state of the shifts (x^k and p^k of every
-                                 shift for the columns in flight, plus the device copy of
-                                 the full solutions; tb_shifted_cocg and tb_mulliken_vjp).
+                                 shift for the columns in flight, the column slices' sums
+                                 of steps, the device copy of the full solutions;
+                                 tb_shifted_cocg and tb_mulliken_vjp; calls of several
+                                 panels hold the solutions of the panels in flight once
+                                 more, half of their state).
                                  When all K shifts would exceed it, the shifts are taken
                                  in chunks, each a separate shifted solve of the same
                                  columns whose seed sequence is recomputed (its seed is

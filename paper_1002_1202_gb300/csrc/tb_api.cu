@@ -33,6 +33,9 @@ int max_grid();
 // longer stays in the shared memory of a cluster, and the panel kernels are
 // faster (6912 orbitals, 256 columns: 184 ms against 380-610)
 constexpr int64_t SLICE_MAX_ROWS = 2304;
+constexpr int SLICE_MAX_M = 256;        // projected rows per column that they take
+// outer steps per slice launch: the host looks at the columns after each
+constexpr int SLICE_STEPS = 32;
 
 struct tb_handle {
     DevSystem ds;
@@ -195,6 +198,10 @@ struct Solve {
     int cheb_cpt = 0;                   // pairs of columns per thread of the Chebyshev step
     int columns = 0;                    // columns of the call solved at the same time (0: this solve's)
     int inflight = 1;                   // panels of the call in flight
+    // device bytes of one panel for x^k and p^k (full solutions; 0: the state
+    // budget) and for the slices' block of steps, in units of its shortest block
+    // (below 0: the default)
+    double state_bytes = 0.0, block_scale = -1.0;
 };
 
 // What one solve sees of a system: the device arrays (a whole handle, or one
@@ -1002,9 +1009,6 @@ static bool slices_on() {
     const char* e = std::getenv("TB_SLICE");
     return !(e && std::atoi(e) == 0);
 }
-// outer steps per slice launch: the host looks at the columns after each
-constexpr int SLICE_STEPS = 32;
-
 int sm_count() {
     static const int n = [] {
         int dev = 0, sms = 0;
@@ -1015,19 +1019,35 @@ int sm_count() {
     return n;
 }
 
+// Device bytes of a block of `len` outer steps of a panel of P columns.
+double block_bytes(int P, int K, int rows, bool deriv, int len) {
+    const double PK = (double)P * K;
+    return len * PK * (deriv ? 64.0 : 32.0) + (len + 1.0) * P * rows * 8.0 + PK * 4.0;
+}
+
+// The arrays of a block; false (and no error) when the device has no room.
+bool block_alloc(Cleanup& cl, const PanelDev& p, SliceBlock& b) {
+    const size_t PK = (size_t)p.P * p.K;
+    bool ok = dalloc(cl, &b.A, PK * b.len) == TB_OK && dalloc(cl, &b.L, PK * b.len) == TB_OK;
+    if (ok && p.deriv) ok = dalloc(cl, &b.dA, PK * b.len) == TB_OK && dalloc(cl, &b.dL, PK * b.len) == TB_OK;
+    return ok && dalloc(cl, &b.D, (size_t)p.P * b.rows * (b.len + 1)) == TB_OK && dalloc(cl, &b.count, PK) == TB_OK;
+}
+
 tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* stats, cudaStream_t st) {
     const auto t0 = std::chrono::steady_clock::now();
     const int K = q.K, R = q.R;
     const int npad = v.ds.npad;
-    int P = o->panel ? o->panel : 64;
-    P = std::min(P, next_pow2(R));
+    int W = std::min(o->panel ? o->panel : 64, next_pow2(R));   // columns per panel
+    const double state = q.state_bytes > 0.0 ? q.state_bytes : (double)state_budget(o);
     if (q.proj == PROJ_NONE) {
         // keep the full-mode x^k, p^k within the state budget (the callers
         // chunk the shifts first; a single shift that still does not fit
         // takes narrower panels)
-        while (P > 1 && (double)K * npad * P * 32.0 > (double)state_budget(o)) P >>= 1;
+        while (W > 1 && (double)K * npad * W * 32.0 > state) W >>= 1;
     }
-    P = std::max(P, 2);   // the vector kernels take columns in pairs; a single column has an inactive partner
+    // the vector kernels take columns in pairs; a single column has an inactive
+    // partner, of which no solutions are kept
+    const int P = std::max(W, 2);
     int M = 0;
     if (q.proj == PROJ_ROWS) {
         for (int c = 0; c < R; ++c) M = std::max<int64_t>(M, q.row_ptr[c + 1] - q.row_ptr[c]);
@@ -1039,6 +1059,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     cl.st = st;
     PanelDev p;
     p.P = P;
+    p.XP = W;
     p.K = K;
     p.npad = npad;
     p.M = M;
@@ -1052,7 +1073,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     p.inner_lo_tol = o->inner_lo_tol;
     p.cheb_cpt = q.cheb_cpt;
     p.inflight = q.inflight;
-    const size_t nv = (size_t)npad * P;   // x^k, p^k: complex, one per column
+    const size_t nv = (size_t)npad * W;   // x^k, p^k: complex, one per column
     tb_status s;
     if ((s = alloc_inner_workspace(cl, p, st)) != TB_OK) return s;
     if ((s = dalloc(cl, &p.z, K)) != TB_OK) return s;
@@ -1104,7 +1125,7 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
     SliceArgs sa;
     bool slices = false;
     const SliceDev* sl = nullptr;
-    if (slices_on() && !g_trace && v.owner && v.sys >= 0 && v.n_orb <= SLICE_MAX_ROWS && M <= 256 &&
+    if (slices_on() && !g_trace && v.owner && v.sys >= 0 && v.n_orb <= SLICE_MAX_ROWS && M <= SLICE_MAX_M &&
         (!p.mixed || (ic.cheb.n > 0 && ic.cheb.n <= 512))) {
         // FP64 inner solves of the slices: Chebyshev steps in FP64 to inner_tol
         // when S has usable bounds, else the CG; also the CG when some shift is
@@ -1117,8 +1138,24 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
             double lo = 0.0, hi = 0.0;
             if (system_bounds(v.owner, v.sys, lo, hi) == TB_OK) c64 = cheb_plan(lo, hi, o->inner_tol, o->inner_tol, std::min(o->inner_max_iter, 512));
         }
+        // block mode: up to 512 steps per block (most solves end within one) as
+        // far as 128 MB hold them, at least one launch's; within what the call
+        // allows, else (full solutions under a small state budget) the panel kernels
+        SliceBlock& b = sa.blk;
+        bool room = true;
+        if (q.proj == PROJ_NONE || M > 1 || p.deriv) {
+            b.rows = q.proj == PROJ_NONE ? npad : M;
+            const char* be = std::getenv("TB_SLICE_BLOCK");   // steps per block by hand
+            const double least = block_bytes(P, K, b.rows, p.deriv != 0, SLICE_STEPS);
+            double limit = std::max(134217728.0, least);
+            if (q.block_scale >= 0.0) limit = std::min(limit, q.block_scale * least);
+            b.len = be && std::atoi(be) > 0 ? std::atoi(be) : 512;
+            b.len = std::min(b.len, (std::min(o->max_iter, 512) + SLICE_STEPS - 1)) / SLICE_STEPS * SLICE_STEPS;
+            while (b.len > 0 && block_bytes(P, K, b.rows, p.deriv != 0, b.len) > limit) b.len -= SLICE_STEPS;
+            room = b.len > 0 && block_alloc(cl, p, b);
+        }
         sa.n = p.mixed ? ic.cheb.n : c64.n;
-        sl = slice_choose(v, p, std::max(std::min(P, R), q.columns), sa, st);
+        if (room) sl = slice_choose(v, p, std::max(std::min(W, R), q.columns), sa, st);
         slices = sl != nullptr;
         if (slices) {
             sa.inner_max = o->inner_max_iter;
@@ -1140,33 +1177,11 @@ tb_status run_view(View& v, const Solve& q, const tb_solve_opts* o, tb_stats* st
                 sa.n_last = std::min(c64.n, 9);
                 sa.gamma64 = c64.gamma64;
             }
-            if (q.proj == PROJ_NONE || M > 1 || p.deriv) {
-                // block mode: up to 512 steps per block (most solves end within
-                // one) as far as 128 MB hold them, at least one launch's
-                SliceBlock& b = sa.blk;
-                b.rows = q.proj == PROJ_NONE ? npad : M;
-                const size_t PK = (size_t)P * K;
-                const double per_step = (double)PK * (p.deriv ? 64 : 32) + (double)P * b.rows * 8;
-                const char* be = std::getenv("TB_SLICE_BLOCK");   // steps per block by hand
-                double len = be && std::atoi(be) > 0 ? std::atoi(be) : std::min(512.0, 134217728.0 / per_step);
-                len = std::min(len, (double)(o->max_iter + SLICE_STEPS - 1));
-                b.len = (int)len / SLICE_STEPS * SLICE_STEPS;
-                if (b.len < SLICE_STEPS) {
-                    slices = false;
-                } else {
-                    if ((s = dalloc(cl, &b.A, PK * b.len)) != TB_OK) return s;
-                    if ((s = dalloc(cl, &b.L, PK * b.len)) != TB_OK) return s;
-                    if (p.deriv && (s = dalloc(cl, &b.dA, PK * b.len)) != TB_OK) return s;
-                    if (p.deriv && (s = dalloc(cl, &b.dL, PK * b.len)) != TB_OK) return s;
-                    if ((s = dalloc(cl, &b.D, (size_t)P * b.rows * (b.len + 1))) != TB_OK) return s;
-                    if ((s = dalloc(cl, &b.count, PK)) != TB_OK) return s;
-                }
-            }
         }
     }
 
-    for (int c0 = 0; c0 < R; c0 += P) {
-        const int ncols = std::min(P, R - c0);
+    for (int c0 = 0; c0 < R; c0 += W) {
+        const int ncols = std::min(W, R - c0);
         for (int c = 0; c < P; ++c) {
             ColState cs;
             std::memset(&cs, 0, sizeof(cs));
@@ -1569,25 +1584,101 @@ const tb_handle::Tuned* tuned_for(tb_handle* h, const tb_solve_opts* o, int K) {
     return nullptr;
 }
 
-tb_status run_solve(tb_handle* h, const Solve& q0, const tb_solve_opts* o, tb_stats* stats, cudaStream_t st) {
-    // automatic choices: the handle's tuned panel width, panels in flight and
-    // Chebyshev-step form for this size class, else the defaults
+// How a call's columns are laid out: columns per panel, panels in flight and
+// the step form, as run_solve takes them.
+struct Shape {
+    int panel = 64, streams = 1, cpt = 0;
+};
+
+// Columns per system of the handle.
+std::vector<int> system_columns(const tb_handle* h, int R, const int32_t* cols) {
+    if (h->sys_ds.empty()) return {R};
+    std::vector<int> n(h->sys_ds.size(), 0);
+    for (int c = 0; c < R; ++c)
+        ++n[std::upper_bound(h->sys_orb_off.begin(), h->sys_orb_off.end(), (int64_t)cols[c]) - h->sys_orb_off.begin() - 1];
+    return n;
+}
+
+// The most that f(columns of a panel, padded orbitals of its system) sums to
+// over the panels that can be in flight at once.
+template <class F>
+double in_flight(const tb_handle* h, const std::vector<int>& ncols, int panel, int streams, F&& f) {
+    std::vector<double> v;
+    for (size_t s = 0; s < ncols.size(); ++s) {
+        if (ncols[s] == 0) continue;
+        const int P = std::min(panel, next_pow2(ncols[s]));
+        const int npad = 4 * (int)(h->sys_atom_off[s + 1] - h->sys_atom_off[s]);
+        const int jobs = std::min((ncols[s] + P - 1) / P, streams);
+        v.insert(v.end(), jobs, f(P, npad));
+    }
+    std::sort(v.rbegin(), v.rend());
+    double sum = 0.0;
+    for (int i = 0; i < streams && i < (int)v.size(); ++i) sum += v[i];
+    return sum;
+}
+
+// The shape of a call: the caller's or the tuned panel width, else 64 columns;
+// up to MAX_P on systems that the column slices take, so that all slices run
+// at once (288 columns of a 144-atom water box: five panels of 64 on four
+// streams took two rounds; 300 rows per column, which the panel kernels take,
+// 512 columns of 216 atoms: 24.9 ms against 34.4 in panels of 64), as far as
+// bytes(panel, streams), the device memory of the panels in flight that grows
+// with their width, stays within `limit`.
+template <class F>
+Shape call_shape(tb_handle* h, const Solve& q, const tb_solve_opts* o, double limit, F&& bytes) {
+    Shape sh;
+    const tb_handle::Tuned* t = o->panel == 0 ? tuned_for(h, o, q.K) : nullptr;
+    sh.streams = q.streams ? q.streams : (t ? t->streams : workers_for(h));
+    sh.cpt = q.cheb_cpt ? q.cheb_cpt : (t ? t->cpt : 0);
+    if (o->panel || t) {
+        sh.panel = o->panel ? o->panel : t->panel;
+        return sh;
+    }
+    if (slices_on() && slice_system(h))
+        for (int P = MAX_P; P > 64; P >>= 1)
+            if (bytes(P, sh.streams) <= limit) {
+                sh.panel = P;
+                break;
+            }
+    return sh;
+}
+
+// Projected outputs: the wide default panels may hold this much of the shifts'
+// projections and of the slices' blocks of steps, together
+constexpr double WIDE_BYTES = 2147483648.0;
+
+tb_status run_shaped(tb_handle* h, const Solve& q0, const tb_solve_opts* o, const Shape& sh, tb_stats* stats,
+                     cudaStream_t st) {
     Solve q = q0;
     tb_solve_opts oe = *o;
-    const tb_handle::Tuned* t = o->panel == 0 ? tuned_for(h, o, q.K) : nullptr;
-    if (t) oe.panel = t->panel;
-    // systems that the column slices take: panels as wide as they can be, so
-    // that all slices run at once (288 columns of a 144-atom water box: five
-    // panels of 64 on four streams took two rounds)
-    else if (o->panel == 0 && slices_on() && slice_system(h)) oe.panel = MAX_P;
-    if (q.cheb_cpt == 0 && t) q.cheb_cpt = t->cpt;
-    const int nw = q.streams ? q.streams : (t ? t->streams : workers_for(h));
-    const int Pw = std::min(oe.panel ? oe.panel : 64, next_pow2(q.R));
-    if (h->sys_ds.empty() && (nw == 1 || q.R <= Pw)) {
+    oe.panel = sh.panel;
+    q.cheb_cpt = sh.cpt;
+    const int Pw = std::min(sh.panel, next_pow2(q.R));
+    if (h->sys_ds.empty() && (sh.streams == 1 || q.R <= Pw)) {
         View v = whole_view(h);
         return run_view(v, q, &oe, stats, st);
     }
-    return run_jobs(h, q, &oe, stats, st, nw);
+    return run_jobs(h, q, &oe, stats, st, sh.streams);
+}
+
+tb_status run_solve(tb_handle* h, const Solve& q, const tb_solve_opts* o, tb_stats* stats, cudaStream_t st) {
+    int M = 0;
+    if (q.proj == PROJ_ROWS)
+        for (int c = 0; c < q.R; ++c) M = std::max<int>(M, (int)(q.row_ptr[c + 1] - q.row_ptr[c]));
+    const bool deriv = q.dg_out != nullptr;
+    const std::vector<int> ncols = system_columns(h, q.R, q.cols);
+    Shape sh = call_shape(h, q, o, WIDE_BYTES, [&](int panel, int streams) {
+        return in_flight(h, ncols, panel, streams, [&](int P, int) {
+            const double block = M > 1 || deriv ? block_bytes(P, q.K, M, deriv, SLICE_STEPS) : 0.0;
+            return (double)P * q.K * std::max(M, 1) * (deriv ? 64.0 : 32.0) + block;
+        });
+    });
+    tb_status s = run_shaped(h, q, o, sh, stats, st);
+    if (s == TB_ERR_OOM && o->panel == 0 && sh.panel > 64) {   // the wide default does not fit beside what the caller holds
+        sh.panel = 64;
+        s = run_shaped(h, q, o, sh, stats, st);
+    }
+    return s;
 }
 
 tb_status check_cols(const tb_handle* h, int R, const int32_t* cols) {
@@ -2379,16 +2470,45 @@ tb_status tb_shifted_cocg(tb_handle* h, int32_t K, const double* z, int32_t R, c
     if ((s = check_shifts(K, z, opts)) != TB_OK) return s;
     if ((s = check_cols(h, R, cols)) != TB_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // energy-point checkpointing: shifts per chunk so that x^k, p^k of the
-    // panels in flight and the device copy of the chunk's solutions fit the
-    // state budget (x_out is [K][R][N]: a chunk of shifts is one contiguous
-    // slice of it)
+    // energy-point checkpointing: x^k, p^k of the panels in flight, the slices'
+    // blocks of steps and the device copy of the solutions fit the state budget
+    // (x_out is [K][R][N]: a chunk of shifts is one contiguous slice of it).
+    // Panels wider than 64 are taken while all shifts fit; else the shifts go in
+    // chunks; where not one shift fits, fewer panels are in flight, and run_view
+    // narrows the last.
     const int64_t N = h->n_orb;
     const bool host_out = !is_device_ptr(x_out);
-    const int Pw = std::min(opts->panel ? opts->panel : 64, next_pow2(R));
-    const int inflight = std::min<int64_t>(workers_for(h), (R + Pw - 1) / Pw);
-    const double per_shift = 32.0 * (double)h->ds.npad * Pw * inflight + (host_out ? 16.0 * (double)R * N : 0.0);
-    const int Kc = (int)std::max<double>(1.0, std::min<double>(K, std::floor((double)state_budget(opts) / per_shift)));
+    const double budget = (double)state_budget(opts), out_shift = host_out ? 16.0 * (double)R * N : 0.0;
+    const bool sliced = slices_on() && slice_system(h);
+    const std::vector<int> ncols = system_columns(h, R, cols);
+    auto state = [&](int panel, int streams) {   // of one shift
+        return in_flight(h, ncols, panel, streams, [](int P, int npad) { return 32.0 * npad * P; });
+    };
+    auto blocks = [&](int panel, int streams, int k) {
+        if (!sliced) return 0.0;
+        return in_flight(h, ncols, panel, streams,
+                         [&](int P, int npad) { return block_bytes(std::max(P, 2), k, npad, false, SLICE_STEPS); });
+    };
+    Solve qs;
+    qs.K = K;
+    Shape sh = call_shape(h, qs, opts, budget, [&](int panel, int streams) {
+        return K * (out_shift + state(panel, streams)) + blocks(panel, streams, K);
+    });
+    while (sh.streams > 1 && out_shift + state(sh.panel, sh.streams) > budget) --sh.streams;
+    // the slices run when their blocks have room: it is set aside where it is
+    // small beside the budget, with fewer panels in flight if need be
+    int few = sh.streams;
+    while (few > 1 && blocks(sh.panel, few, 0) > budget / 8) --few;
+    const bool room = sliced && blocks(sh.panel, few, 0) <= budget / 8;
+    if (room) sh.streams = few;
+    auto fitting = [&](double room, double per_shift) {
+        return (int)std::max<double>(1.0, std::min<double>(K, std::floor(room / per_shift)));
+    };
+    const double fixed = room ? blocks(sh.panel, sh.streams, 0) : 0.0;
+    const double per_k = room ? blocks(sh.panel, sh.streams, 1) - fixed : 0.0;
+    const int Kc = fitting(budget - fixed, out_shift + state(sh.panel, sh.streams) + per_k);
+    const double least = blocks(sh.panel, sh.streams, Kc);
+    const double spare = std::max(0.0, budget - Kc * (out_shift + state(sh.panel, sh.streams)));
     Cleanup cl;
     cl.st = st;
     OutBuf ob;
@@ -2408,7 +2528,13 @@ tb_status tb_shifted_cocg(tb_handle* h, int32_t K, const double* z, int32_t R, c
             conv.assign((size_t)R * kc, -1);
             ts.conv_iter = conv.data();
         }
-        const tb_status run = run_solve(h, q, &oc, stats ? &ts : nullptr, st);
+        q.state_bytes = std::max(1.0, budget - Kc * out_shift);
+        q.block_scale = least > 0.0 ? spare / least : 0.0;
+        tb_status run = run_shaped(h, q, &oc, sh, stats ? &ts : nullptr, st);
+        if (run == TB_ERR_OOM && opts->panel == 0 && sh.panel > 64) {   // as run_solve
+            sh.panel = 64;
+            run = run_shaped(h, q, &oc, sh, stats ? &ts : nullptr, st);
+        }
         if (run == TB_ERR_NOT_CONVERGED) unconverged = true;
         else if (run != TB_OK) return run;
         if (ob.host) {
@@ -2556,8 +2682,15 @@ tb_status tb_mulliken_vjp(tb_handle* h, int32_t K, const double* z, const double
     // chunks of shifts, each solved again from its own seed sequence
     const double per_cs = 64.0 * (double)N;
     const double budget = (double)state_budget(opts);
-    const int Rc = (int)std::max<double>(1.0, std::min<double>(std::max<int64_t>(ns, 1), std::floor(budget / (per_cs * K))));
-    const int Kc = (int)std::max<double>(1.0, std::min<double>(K, std::floor(budget / (per_cs * Rc))));
+    // the slices' blocks of steps, where they are small beside the budget
+    auto blocks = [&](int64_t cols_, int k) {
+        const int P = std::min(opts->panel ? opts->panel : 64, next_pow2((int)std::max<int64_t>(cols_, 1)));
+        return block_bytes(std::max(P, 2), k, h->ds.npad, false, SLICE_STEPS);
+    };
+    const bool sliced = slices_on() && h->sys_ds.empty() && slice_system(h);
+    const double reserve = sliced && blocks(ns, K) <= budget / 8 ? blocks(ns, K) : 0.0;
+    const int Rc = (int)std::max<double>(1.0, std::min<double>(std::max<int64_t>(ns, 1), std::floor((budget - reserve) / (per_cs * K))));
+    const int Kc = (int)std::max<double>(1.0, std::min<double>(K, std::floor((budget - reserve) / (per_cs * Rc))));
     Cleanup cl;
     cl.st = st;
     int32_t *ead, *ebd, *cpos;
@@ -2618,6 +2751,7 @@ tb_status tb_mulliken_vjp(tb_handle* h, int32_t K, const double* z, const double
                 q.K = kc; q.z = z + 2 * (size_t)k0; q.R = rc; q.cols = cols.data(); q.proj = PROJ_NONE;
                 q.x_out = pass == 0 ? X : Y;
                 if (pass == 1) q.rhs = Sc;
+                q.block_scale = std::max(0.0, budget - per_cs * Rc * Kc) / blocks(rc, kc);
                 tb_stats ts{};
                 const tb_status run = run_view(vw, q, &oc, &ts, st);
                 if (run == TB_ERR_NOT_CONVERGED) unconverged = true;

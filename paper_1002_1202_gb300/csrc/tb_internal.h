@@ -175,6 +175,7 @@ struct InnerState {
 struct PanelDev {
     int P = 0;                    // columns (right-hand sides), even
     int C = 0;                    // pairs of columns, P / 2: the unit of the vector kernels
+    int XP = 0;                   // columns of X and Pk: P, or 1 for a single column (whose partner has no solutions)
     int K = 0, npad = 0, M = 0, proj = PROJ_NONE;
     int grid = 0;                 // CTAs of the grid-stride kernels
     int mixed = 0;                // 1: inner S^-1 by FP32 corrections inside FP64 refinement
@@ -205,7 +206,7 @@ struct PanelDev {
     int deriv = 0;                               // 1: also d/dz_k of the projections (PROJ_ROWS)
     double2 *dzeta = nullptr, *dpinv = nullptr;  // [P][K] d/dz_k of zeta and pinv
     double2 *dt = nullptr, *du = nullptr;        // [P][K][M] d/dz_k of t, u
-    double2 *X = nullptr, *Pk = nullptr;         // [K][npad][P] full mode x, p
+    double2 *X = nullptr, *Pk = nullptr;         // [K][npad][XP] full mode x, p
     double* partials = nullptr;    // [grid][4][C] per-CTA sums
     double* partials2 = nullptr;   // [MAX_GROUPS][4][C] per-group sums
     unsigned* counter = nullptr;   // [1 + MAX_GROUPS] arrival tickets of the grid reductions

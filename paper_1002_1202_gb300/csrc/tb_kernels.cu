@@ -1646,14 +1646,19 @@ __global__ void k_shift_init(DevSystem s, PanelDev p) {
     }
 }
 
+// element r = row * XP + column of x^k, p^k in the panel vectors
+__device__ __forceinline__ long long full_elem(const PanelDev& p, long long r) {
+    return p.XP == p.P ? r : r / p.XP * p.P + r % p.XP;
+}
+
 __global__ void k_full_init(PanelDev p) {
-    const long long per = (long long)p.npad * p.P;
+    const long long per = (long long)p.npad * p.XP;
     const long long items = per * p.K;
     const double* Rp = reinterpret_cast<const double*>(p.Rp);
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
         p.X[idx] = cmk(0.0, 0.0);
-        p.Pk[idx] = cmk(Rp[idx % per] * p.col[idx % p.P].inv_nu, 0.0);
+        p.Pk[idx] = cmk(Rp[full_elem(p, idx % per)] * p.col[idx % p.XP].inv_nu, 0.0);
     }
 }
 
@@ -1799,13 +1804,12 @@ __global__ void __launch_bounds__(THREADS) k_shift_step(DevSystem s, PanelDev p)
 
 // Full mode: x^k += alpha^k q^k, q^k = u'_{n+1} / nu_{n+1} + l^k q^k.
 __global__ void k_full_update(PanelDev p) {
-    const int P = p.P;
-    const long long per = (long long)p.npad * P;
+    const long long per = (long long)p.npad * p.XP;
     const long long items = per * p.K;
     const double* Rp = reinterpret_cast<const double*>(p.Rp);
     for (long long idx = blockIdx.x * (long long)THREADS + threadIdx.x; idx < items;
          idx += (long long)gridDim.x * THREADS) {
-        const int c = (int)(idx % P);
+        const int c = (int)(idx % p.XP);
         const int k = (int)(idx / per);
         const size_t o = (size_t)c * p.K + k;
         const double2 al = p.ak[o];
@@ -1813,7 +1817,7 @@ __global__ void k_full_update(PanelDev p) {
         const double2 q = p.Pk[idx];
         const double2 qn = cmul(p.bk[o], q);
         p.X[idx] = cadd(p.X[idx], cmul(al, q));
-        p.Pk[idx] = cmk(Rp[idx % per] * p.col[c].inv_nu + qn.x, qn.y);
+        p.Pk[idx] = cmk(Rp[full_elem(p, idx % per)] * p.col[c].inv_nu + qn.x, qn.y);
     }
 }
 
@@ -1825,7 +1829,7 @@ __global__ void k_full_output(PanelDev p, const int32_t* __restrict__ orb2pad, i
         const int o = (int)(idx % n_orb);
         const int c = (int)((idx / n_orb) % ncols);
         const int k = (int)(idx / ((long long)n_orb * ncols));
-        out[((size_t)k * R + c0 + c) * n_orb + o] = p.X[((size_t)k * p.npad + orb2pad[o]) * p.P + c];
+        out[((size_t)k * R + c0 + c) * n_orb + o] = p.X[((size_t)k * p.npad + orb2pad[o]) * p.XP + c];
     }
 }
 
@@ -2968,7 +2972,7 @@ void launch_shift_init(const DevSystem& s, const PanelDev& p, cudaStream_t st) {
     }
     if (p.proj == PROJ_NONE) {
         LaunchScope ls_(K_OTHER, st);
-        k_full_init<<<grid_for((long long)p.npad * p.P * p.K), THREADS, 0, st>>>(p);
+        k_full_init<<<grid_for((long long)p.npad * p.XP * p.K), THREADS, 0, st>>>(p);
     }
 }
 void launch_shift_step(const DevSystem& s, const PanelDev& p, cudaStream_t st) {
@@ -2983,7 +2987,7 @@ void launch_shift_step(const DevSystem& s, const PanelDev& p, cudaStream_t st) {
 void launch_full_update(const DevSystem&, const PanelDev& p, cudaStream_t st) {
     {
         LaunchScope ls_(K_FULL_UPDATE, st);
-        k_full_update<<<grid_for((long long)p.npad * p.P * p.K), THREADS, 0, st>>>(p);
+        k_full_update<<<grid_for((long long)p.npad * p.XP * p.K), THREADS, 0, st>>>(p);
     }
 }
 void launch_full_output(const PanelDev& p, const int32_t* orb2pad, int n_orb, int R, int ncols, int c0,

@@ -1639,7 +1639,7 @@ __global__ void __launch_bounds__(128) k_block_apply(PanelDev p, SliceBlock b, i
     for (int j = 0; j < BK; ++j) {
         const int k = kb + j;
         if (k >= K) break;
-        const size_t o = full ? ((size_t)k * p.npad + r) * p.P + c : ((size_t)c * K + k) * p.M + r;
+        const size_t o = full ? ((size_t)k * p.npad + r) * p.XP + c : ((size_t)c * K + k) * p.M + r;
         double2* X = full ? p.X : p.t;
         double2* Q = full ? p.Pk : p.u;
         double2 x = acc[j][0], dx = DERIV ? acc[j][1 % NV] : cmk(0.0, 0.0);
@@ -1686,7 +1686,7 @@ void launch_block_flush(const PanelDev& p, const SliceBlock& b, int nsteps, int 
     mark = launch_mark_begin(K_FULL_UPDATE, st);
     const int rows = p.proj == PROJ_NONE ? p.npad : p.M;
     constexpr int BK = 4;
-    const dim3 g((rows + 127) / 128, (p.K + BK - 1) / BK, p.P);
+    const dim3 g((rows + 127) / 128, (p.K + BK - 1) / BK, p.proj == PROJ_NONE ? p.XP : p.P);
     const int first = n0 == 0 ? 1 : 0;
     if (p.deriv && goes_on) k_block_apply<BK, true, true><<<g, 128, 0, st>>>(p, b, first);
     else if (p.deriv) k_block_apply<BK, true, false><<<g, 128, 0, st>>>(p, b, first);
