@@ -532,7 +532,7 @@ tb_status tb_lanczos_green_batch(int32_t R, const double *a, const double *b, co
  *    GPU on which a handle was created holds the array until the process
  *    exits.  Call this entry point with the handle's device current
  *    (otherwise TB_ERR_INVALID_ARG).
- *  - Size limit: the call needs about 160 * 4 * n_atoms + 16 * n_steps bytes
+ *  - Size limit: the call needs about 144 * 4 * n_atoms + 16 * n_steps bytes
  *    (plus ~50 kB); a request that does not fit returns TB_ERR_TOO_LARGE
  *    before any device work (N up to ~100 000 orbitals with a few hundred
  *    steps).

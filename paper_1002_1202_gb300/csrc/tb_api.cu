@@ -3277,16 +3277,14 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     p.inner_tol = inner_tol > 0.0 ? inner_tol : 1e-13;
     // size check before any device work: everything must fit in the fixed array
     ScratchCarver dry(nullptr, TB_NOALLOC_SCRATCH_BYTES);
-    for (int v = 0; v < 10; ++v) dry.take<double2>(npad);
+    for (int v = 0; v < 9; ++v) dry.take<double2>(npad);
     dry.take<ColState>(2);
     dry.take<InnerState>(2);
     dry.take<double>((size_t)p.grid * 4);
     dry.take<double>((size_t)MAX_GROUPS * 4);
     dry.take<unsigned>(1 + MAX_GROUPS);
     dry.take<int>(NFLAGS);
-    dry.take<double>((size_t)2 * n_steps);
-    dry.take<double>((size_t)2 * (n_steps + 1));
-    dry.take<double>(2);
+    dry.take<double>((size_t)2 * n_steps + 5);
     if (!dry.ok) return TB_ERR_TOO_LARGE;
     // the handle's device must be current: the scratch address and the
     // kernels were placed there by tb_create
@@ -3302,16 +3300,18 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     for (double2** v : vecs) *v = sc.take<double2>(npad);
     double2* U = sc.take<double2>(npad);
     double2* Uprev = sc.take<double2>(npad);
-    double2* Wv = sc.take<double2>(npad);
+    double2* Wv = p.Rprev;   // u_{n-1} of the solver, not used here
     p.col = sc.take<ColState>(2);
     p.inner = sc.take<InnerState>(2);
     p.partials = sc.take<double>((size_t)p.grid * 4);
     p.partials2 = sc.take<double>((size_t)MAX_GROUPS * 4);
     p.counter = sc.take<unsigned>(1 + MAX_GROUPS);
     p.flags = sc.take<int>(NFLAGS);
-    double* ad = sc.take<double>((size_t)2 * n_steps);          // [column][n_steps]
-    double* bd = sc.take<double>((size_t)2 * (n_steps + 1));
-    double* nd = sc.take<double>(2);
+    // a_n, b_n and the norm; the inactive partner's zeros go to the element after
+    // the column's, which the next step writes
+    double* ad = sc.take<double>((size_t)2 * n_steps + 5);   // [n_steps + 1]
+    double* bd = ad + n_steps + 1;                            // [n_steps + 2]
+    double* nd = bd + n_steps + 2;                            // [2]
     if (!sc.ok) return TB_ERR_TOO_LARGE;
     // the array keeps the previous call's contents: clear everything that
     // the step loop reads before writing
@@ -3325,8 +3325,7 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     TB_CK(cudaMemsetAsync(p.flags, 0, NFLAGS * sizeof(int), st));
     TB_CK(cudaMemsetAsync(p.counter, 0, sizeof(unsigned) * (1 + MAX_GROUPS), st));
     TB_CK(cudaMemsetAsync(Uprev, 0, sizeof(double2) * npad, st));
-    TB_CK(cudaMemsetAsync(ad, 0, sizeof(double) * 2 * n_steps, st));
-    TB_CK(cudaMemsetAsync(bd, 0, sizeof(double) * 2 * (n_steps + 1), st));
+    TB_CK(cudaMemsetAsync(ad, 0, sizeof(double) * ((size_t)2 * n_steps + 5), st));
     int pred = 64;
     int64_t inner_total = 0;
     const int inner_max = 1000;
@@ -3336,13 +3335,13 @@ tb_status tb_generalized_lanczos_noalloc(tb_handle* h, int32_t j, int32_t n_step
     launch_lz_start(p, p.Rp, U, nd, st);
     for (int n = 0; n < n_steps; ++n) {
         launch_lz_spmv(h->ds, h->ds.H, U, p.W, 1, st);
-        launch_lz_dot(p, U, p.W, ad + n, n_steps, 0, st);
+        launch_lz_dot(p, U, p.W, ad + n, 1, 0, st);
         TB_CK(cudaMemcpyAsync(p.Rin, p.W, sizeof(double2) * npad, cudaMemcpyDeviceToDevice, st));
         if ((s = inner_cg(hv, p, inner_max, pred, inner_total, st)) != TB_OK) return s;
-        launch_lz_combine(p, p.Rp, U, Uprev, Wv, ad + n, bd + n, n_steps, n_steps + 1, st);
+        launch_lz_combine(p, p.Rp, U, Uprev, Wv, ad + n, bd + n, 1, 1, st);
         launch_lz_spmv(h->ds, h->ds.S, Wv, p.W, 1, st);
-        launch_lz_dot(p, Wv, p.W, bd + n + 1, n_steps + 1, 1, st);
-        launch_lz_scale(p, Wv, U, Uprev, bd + n + 1, n_steps + 1, st);
+        launch_lz_dot(p, Wv, p.W, bd + n + 1, 1, 1, st);
+        launch_lz_scale(p, Wv, U, Uprev, bd + n + 1, 1, st);
         TB_CK(cudaGetLastError());
     }
     if (h->flags_host[0] & ERR_NOT_SPD) return TB_ERR_S_NOT_SPD;

@@ -123,3 +123,23 @@ def test_ragged_and_padded_steps_of_a_large_box(P, ran):
     assert np.abs(wide - narrow).max() <= 1e-9 * np.abs(wide).max()
     assert np.abs(wide[:64] - one).max() <= 1e-9 * np.abs(wide).max()
     assert ran()["inner32_cheb"] > 0
+
+
+def test_noalloc_request_of_the_whole_scratch(P):
+    """The allocation-free call takes what fits ten vectors of one column, its two
+    coefficient arrays, the norm and the reductions' sums in its fixed array
+    (its capacity before the vectors were held in pairs): a request that fills it
+    to the last 512 bytes.  Uncoupled atoms: the process ends at its first step."""
+    import torch
+    r256 = lambda b: (b + 255) // 256 * 256
+    grid = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    cap = 16 << 20
+    need = lambda n, k: (10 * r256(64 * n) + 256 + 256 + r256(grid * 32) + 64 * 32 + r256(65 * 4) + 256 + r256(8 * k) +
+                         r256(8 * k + 8) + 256)
+    n = next(n for n in range(cap // 640, 0, -4) if need(n, 32) <= cap)
+    k = next(k for k in range(4000, 0, -1) if need(n, k) <= cap)
+    assert cap - 512 < need(n, k) <= cap
+    h = P.tb_create(np.ones(n), np.arange(n + 1), np.arange(n), np.ones(n), eps=np.linspace(-20.0, -5.0, n))
+    a, b, nrm = (np.asarray(v) for v in P.tb_generalized_lanczos_noalloc(h, 7, k))
+    assert len(a) == k and abs(a[0] - np.linspace(-20.0, -5.0, n)[7]) <= 1e-12 * 20 and nrm[0] == 1.0
+    assert np.all(b == 0.0)
