@@ -893,9 +893,10 @@ const SliceDev* get_slice(tb_handle* h, int sys, int cl, cudaStream_t st) {
     up(&d.H64, nullptr, 2 * sizeof(double2) * ni);
     if (ok) {
         d.n_items = (long long)ni;
-        launch_slice_fill(h->ds.S, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.S64),
+        d.base = 16 * (long long)h->brow_h[a0];
+        launch_slice_fill(h->ds.S + d.base, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.S64),
                           reinterpret_cast<float*>(d.Shi), reinterpret_cast<float*>(d.Slo), st);
-        launch_slice_fill(h->ds.H, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64),
+        launch_slice_fill(h->ds.H + d.base, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64),
                           reinterpret_cast<float*>(d.Hhi), reinterpret_cast<float*>(d.Hlo), st);
         ok = cudaGetLastError() == cudaSuccess;
     }
@@ -1784,7 +1785,7 @@ void refill_slices_H(tb_handle* h, cudaStream_t st) {
     for (auto& list : h->slices)
         for (auto& d : list)
             if (d->noct > 0)
-                launch_slice_fill(h->ds.H, d->src, 4 * d->n_items, reinterpret_cast<double*>(d->H64),
+                launch_slice_fill(h->ds.H + d->base, d->src, 4 * d->n_items, reinterpret_cast<double*>(d->H64),
                                   reinterpret_cast<float*>(d->Hhi), reinterpret_cast<float*>(d->Hlo), st);
 }
 

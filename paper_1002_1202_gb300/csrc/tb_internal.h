@@ -93,7 +93,8 @@ struct SliceDev {
     int* dest = nullptr;
     int* row_slot = nullptr;        // [nrows] padded orbital slot of a row, -1: filling
     ushort4* idx = nullptr;         // [batches][8] places (in the CTA's vector) of the items of steps 1, 2, ...
-    int* src = nullptr;             // [items][4] offsets of the coefficients in S and H, -1: zero
+    int* src = nullptr;             // [items][4] offsets of the coefficients in S and H of the system, -1: zero
+    long long base = 0;             // the system's first value in the handle's S and H
     float4 *Shi = nullptr, *Slo = nullptr, *Hhi = nullptr, *Hlo = nullptr;   // [items]
     double2 *S64 = nullptr, *H64 = nullptr;                                  // [items][2]
     long long n_items = 0;

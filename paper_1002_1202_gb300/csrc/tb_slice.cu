@@ -1526,7 +1526,7 @@ bool with_instance(bool mixed, int nc, bool reg, F&& f) {
     return false;
 }
 
-// values of the items from the 4x4 blocks (src: offset in the block array, -1: zero)
+// values of the items from the 4x4 blocks of the system (src: offset in M, -1: zero)
 __global__ void k_slice_fill(const double* __restrict__ M, const int* __restrict__ src, long long n,
                              double* __restrict__ m64, float* __restrict__ hi, float* __restrict__ lo) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -1727,7 +1727,8 @@ bool launch_slice(const SliceDev& ss, const DevSystem& s, const PanelDev& p, con
 
 // Host: groups, octets and items of one system for clusters of cl CTAs (see
 // the head of the file).  brow, bcol: its block rows, columns local to col0;
-// orb: orbitals per atom.
+// orb: orbitals per atom.  The coefficients' offsets count from the system's
+// first block, brow[0].
 void slice_layout(int n, const int32_t* orb, const int64_t* brow, const int32_t* bcol, int32_t col0, int cl,
                   SliceHost& out) {
     struct Group {
@@ -1872,8 +1873,8 @@ void slice_layout(int n, const int32_t* orb, const int64_t* brow, const int32_t*
                         }
                         Item& it = list[pos[row]];
                         if (G.sp)
-                            for (int q = 0; q < 4; ++q) it.src[q] = (int)(16 * b + 4 * q + e);
-                        else it.src[a] = (int)(16 * b + e);
+                            for (int q = 0; q < 4; ++q) it.src[q] = (int)(16 * (b - brow[0]) + 4 * q + e);
+                        else it.src[a] = (int)(16 * (b - brow[0]) + e);
                     }
                 }
             for (int row : seen) pos[row] = -1;
