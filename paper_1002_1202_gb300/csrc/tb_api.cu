@@ -858,7 +858,9 @@ void free_slice(SliceDev& d) {
 }
 
 // The layout of system `sys` of the handle for clusters of cl CTAs, built on
-// first use on stream st (nullptr: not available, e.g. out of memory).
+// first use on stream st (nullptr: not available; a layout that its indices
+// cannot hold is remembered, one that found no device memory is tried again by
+// the next call).
 const SliceDev* get_slice(tb_handle* h, int sys, int cl, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(h->slice_mu);
     if ((int)h->slices.size() <= sys) h->slices.resize(sys + 1);
@@ -871,7 +873,8 @@ const SliceDev* get_slice(tb_handle* h, int sys, int cl, cudaStream_t st) {
     SliceHost hs;
     slice_layout(n, h->orb_per_atom.data() + a0, h->brow_h.data() + a0, h->bcol_h.data(), a0, cl, hs);
     const size_t ni = (size_t)hs.oct_ptr.back() * 8;
-    bool ok = hs.nloc <= 65535 && ni * 4 < ((size_t)1 << 31);
+    const bool holds = hs.nloc <= 65535 && ni * 4 < ((size_t)1 << 31);
+    bool ok = holds;
     auto up = [&](auto** dst, const void* srcp, size_t bytes) {
         if (!ok) return;
         ok = cudaMalloc(reinterpret_cast<void**>(dst), std::max<size_t>(bytes, 16)) == cudaSuccess &&
@@ -905,7 +908,8 @@ const SliceDev* get_slice(tb_handle* h, int sys, int cl, cudaStream_t st) {
     if (!ok) {
         cudaGetLastError();
         free_slice(d);
-        d.cl = cl;   // remembered: not tried again
+        if (holds) return nullptr;
+        d.cl = cl;
         h->slices[sys].push_back(std::move(dev));
         return nullptr;
     }
