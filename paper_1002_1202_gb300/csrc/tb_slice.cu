@@ -1448,11 +1448,18 @@ struct Instance {
         return false;
     }
 
-    // shared-memory limit raised (never lowered), clusters of 16 allowed
+    // shared-memory limit raised (never lowered), clusters of 16 allowed, on the
+    // current device (both are per device)
     static bool prepare(size_t sm) {
         static std::mutex mu;
-        static size_t cur = 0;
+        static size_t limit[64] = {0};
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+            cudaGetLastError();
+            return false;
+        }
         std::lock_guard<std::mutex> lk(mu);
+        size_t& cur = limit[dev];
         if (sm <= cur) return true;
         const auto k = k_slice<MIXED, NC, CPL, REG>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
