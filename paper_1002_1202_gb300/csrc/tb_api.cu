@@ -896,10 +896,10 @@ const SliceDev* get_slice(tb_handle* h, int sys, int cl, cudaStream_t st) {
     up(&d.H64, nullptr, 2 * sizeof(double2) * ni);
     if (ok) {
         d.n_items = (long long)ni;
-        d.base = 16 * (long long)h->brow_h[a0];
-        launch_slice_fill(h->ds.S + d.base, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.S64),
+        const int64_t base = 16 * h->brow_h[a0];   // the system's first value
+        launch_slice_fill(h->ds.S + base, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.S64),
                           reinterpret_cast<float*>(d.Shi), reinterpret_cast<float*>(d.Slo), st);
-        launch_slice_fill(h->ds.H + d.base, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64),
+        launch_slice_fill(h->ds.H + base, d.src, 4 * d.n_items, reinterpret_cast<double*>(d.H64),
                           reinterpret_cast<float*>(d.Hhi), reinterpret_cast<float*>(d.Hlo), st);
         ok = cudaGetLastError() == cudaSuccess;
     }
@@ -1786,11 +1786,12 @@ namespace {
 // The slices' copies of H after ds.H changed.
 void refill_slices_H(tb_handle* h, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(h->slice_mu);
-    for (auto& list : h->slices)
-        for (auto& d : list)
+    for (size_t sys = 0; sys < h->slices.size(); ++sys)
+        for (auto& d : h->slices[sys])
             if (d->noct > 0)
-                launch_slice_fill(h->ds.H + d->base, d->src, 4 * d->n_items, reinterpret_cast<double*>(d->H64),
-                                  reinterpret_cast<float*>(d->Hhi), reinterpret_cast<float*>(d->Hlo), st);
+                launch_slice_fill(h->ds.H + 16 * h->brow_h[h->sys_atom_off[sys]], d->src, 4 * d->n_items,
+                                  reinterpret_cast<double*>(d->H64), reinterpret_cast<float*>(d->Hhi),
+                                  reinterpret_cast<float*>(d->Hlo), st);
 }
 
 // Keep the Hamiltonian of tb_create before the first charge-dependent one

@@ -94,7 +94,6 @@ struct SliceDev {
     int* row_slot = nullptr;        // [nrows] padded orbital slot of a row, -1: filling
     ushort4* idx = nullptr;         // [batches][8] places (in the CTA's vector) of the items of steps 1, 2, ...
     int* src = nullptr;             // [items][4] offsets of the coefficients in S and H of the system, -1: zero
-    long long base = 0;             // the system's first value in the handle's S and H
     float4 *Shi = nullptr, *Slo = nullptr, *Hhi = nullptr, *Hlo = nullptr;   // [items]
     double2 *S64 = nullptr, *H64 = nullptr;                                  // [items][2]
     long long n_items = 0;
@@ -176,7 +175,6 @@ struct InnerState {
 struct PanelDev {
     int P = 0;                    // columns (right-hand sides), even
     int C = 0;                    // pairs of columns, P / 2: the unit of the vector kernels
-    int XP = 0;                   // columns of X and Pk: P, or 1 for a single column (whose partner has no solutions)
     int K = 0, npad = 0, M = 0, proj = PROJ_NONE;
     int grid = 0;                 // CTAs of the grid-stride kernels
     int mixed = 0;                // 1: inner S^-1 by FP32 corrections inside FP64 refinement
@@ -205,6 +203,7 @@ struct PanelDev {
     int32_t* frow = nullptr;       // [P][M] padded rows (PROJ_ROWS)
     double2 *t = nullptr, *u = nullptr;          // [P][K][M] projected x, p
     int deriv = 0;                               // 1: also d/dz_k of the projections (PROJ_ROWS)
+    int XP = 0;                                  // columns of X and Pk: P, or 1 for a single column (without its partner)
     double2 *dzeta = nullptr, *dpinv = nullptr;  // [P][K] d/dz_k of zeta and pinv
     double2 *dt = nullptr, *du = nullptr;        // [P][K][M] d/dz_k of t, u
     double2 *X = nullptr, *Pk = nullptr;         // [K][npad][XP] full mode x, p
