@@ -524,15 +524,26 @@ CHEB_CPT = None
 
 
 def cheb_kernel_name(panel, n_atoms):
-    """The Chebyshev step's kernel of a panel of ``panel`` column pairs: with
-    two pairs per thread the form with S staged in shared memory for 16 to
-    128 pairs, else the plain one; with four pairs the packed one (from 16
-    pairs on; taken when no run or TB_CHEB_CPT says otherwise)."""
+    """The Chebyshev step's kernel of a panel of ``panel`` column pairs of a
+    system without s-only atoms: with two pairs per thread (the library's
+    default, which a run sets) the form with S staged in shared memory for 16
+    to 128 pairs, else the plain one; with four pairs (the autotuner's choice
+    or TB_CHEB_CPT=4; here also when nothing has run) the packed one."""
     env = os.environ.get("TB_CHEB_CPT")
     cpt = CHEB_CPT if CHEB_CPT else (int(env) if env else (4 if panel >= 16 else 2))
     if cpt == 2 or panel < 4:
         return "k_inner32_chebs" if panel in (16, 32, 64, 128) else "k_inner32_cheb"
     return "k_inner32_cheb4"
+
+
+def algorithmic_bytes(kname, s, panel):
+    """Bytes of one launch of an SpMM-type kernel over ``panel`` pairs of real
+    columns: the matrix and its indices once, every panel vector once.  The
+    SpMVs read x and write y; the Chebyshev step reads d_k, f and d_{k-1} and
+    writes d_{k+1}."""
+    _kern, mb, vb, _fp64 = KERNEL_INFO[kname]
+    vec_io = {"inner_spmv": 2, "inner32_spmv": 2, "inner32_cheb": 4, "refine_residual": 3, "outer_spmm": 5}[kname]
+    return 16 * s.nb * mb + 4 * s.nb + 4 * (s.n_atoms + 1) + vec_io * s.n_orb * panel * vb
 
 
 DF_INSTR_PER_MAC = 12   # FP32 instructions of one double-float multiply-add (exact product + two-sum)
@@ -551,7 +562,7 @@ def roofline_for(kname, ms, launches, s, panel, peaks, mixed=False, busy_ms=None
     double-float FP32 arithmetic, DF_INSTR_PER_MAC FP32 instructions per
     FP64 multiply-add; they are rated against the FP32 issue peak (2 flop per
     FP32 lane-instruction), not against the FP64 units they do not use."""
-    kern, mb, vb, fp64 = KERNEL_INFO[kname]
+    kern, _mb, _vb, fp64 = KERNEL_INFO[kname]
     if kname == "inner32_cheb":
         kern = cheb_kernel_name(panel, s.n_atoms)
     double_float = mixed and kname in ("outer_spmm", "refine_residual")
@@ -559,10 +570,7 @@ def roofline_for(kname, ms, launches, s, panel, peaks, mixed=False, busy_ms=None
     flops = 2.0 * nnz * 2 * panel
     if kname == "inner32_cheb":
         flops += 5.0 * s.n_orb * 2 * panel      # d_{k+1} = d_{k-1} + omega (gamma (f - S d_k) + d_k - d_{k-1})
-    # panel vectors moved once: the SpMVs read x and write y; the Chebyshev
-    # step reads d_k, f and d_{k-1} and writes d_{k+1}
-    vec_io = {"inner_spmv": 2, "inner32_spmv": 2, "inner32_cheb": 4, "refine_residual": 3, "outer_spmm": 5}[kname]
-    nbytes = nnz * mb + 4 * s.nb + 4 * (s.n_atoms + 1) + vec_io * s.n_orb * panel * vb
+    nbytes = algorithmic_bytes(kname, s, panel)
     mean_s = ms / max(launches, 1) / 1e3
     avg_s = busy_ms / max(launches, 1) / 1e3 if busy_ms else mean_s
     if avg_s <= 0:
@@ -899,7 +907,6 @@ def run_large(args):
     z, w = gauss_legendre_grid(128, -20.0, 5.0, 0.01)
     h = P.tb_create_system(s)
     peaks = measured_peaks()
-    nnz = 16 * s.nb
     rows = []
     for panel in (4, 8, 16, 32, 64, 128):
         cols = rank_columns(s.n_orb, panel, 0)
@@ -920,7 +927,7 @@ def run_large(args):
                 n_l, _ms = P.tb_profile_read("inner32_cheb")
                 busy = P.tb_profile_busy("inner32_cheb")
                 us = busy / max(n_l, 1) * 1e3
-                nbytes = nnz * 4 + 4 * s.nb + 4 * (s.n_atoms + 1) + 4 * s.n_orb * panel * 8
+                nbytes = algorithmic_bytes("inner32_cheb", s, max(panel // 2, 1))
                 rec.update({"cheb_launches": n_l, "cheb_us_per_launch": us,
                             "cheb_algorithmic_GBps": nbytes / us / 1e3,
                             "cheb_hbm_frac": nbytes / us / 1e3 / peaks["hbm_gbs"]})
