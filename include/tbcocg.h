@@ -67,10 +67,12 @@ typedef enum {
     TB_ERR_CUDA = 5,           /* a CUDA runtime call failed              */
     TB_ERR_NOT_CONVERGED = 6,  /* max_iter reached; converged shifts valid*/
     TB_ERR_BREAKDOWN = 7,      /* COCG breakdown (rho or mu == 0)         */
-    TB_ERR_TIMEOUT = 8,        /* reserved: no kernel of this library waits
-                                  on another CTA, flag or stream (grid
-                                  reductions take arrival tickets and never
-                                  spin), so no call returns it              */
+    TB_ERR_TIMEOUT = 8,        /* reserved: no kernel of this library spins
+                                  on a flag, a stream or another CTA (grid
+                                  reductions take arrival tickets; the CTAs
+                                  of one thread-block cluster, which run
+                                  together, meet at hardware barriers), so
+                                  no call returns it                        */
     TB_ERR_NO_DEVICE = 9,      /* no usable CUDA device                   */
     TB_ERR_TOO_LARGE = 10      /* request exceeds the fixed scratch of the
                                   allocation-free entry point              */

@@ -29,9 +29,15 @@ namespace tb {
 int max_grid();
 }
 
-// orbitals of the largest system that the column slices take: beyond it S no
-// longer stays in the shared memory of a cluster, and the panel kernels are
-// faster (6912 orbitals, 256 columns: 184 ms against 380-610)
+// orbitals of the largest system that the column slices take.  Up to it they
+// are as fast as the panel kernels or faster for every number of columns (32
+// outer steps, mixed, slices / panels in ms: 8, 256 and all columns of 576
+// silicon atoms 3.3 / 18.2, 13.3 / 23.6 and 121 / 198, 32, 256 and all of 256 water
+// molecules 11.8 / 42.9, 50.6 / 50.2 and 226 / 293; 8 steps in FP64, all columns,
+// 312 / 435 and 320 / 785).  Beyond it they lose at many columns, as S no longer
+// stays on chip (256 and 1024 of 800 atoms 25.9 / 25.2 and 129 / 95, 256 of 1728
+// atoms, whole call, 380-610 / 184), though not at few (8 of 1000 atoms 4.2 /
+// 19.8).
 constexpr int64_t SLICE_MAX_ROWS = 2304;
 constexpr int SLICE_MAX_M = 256;        // projected rows per column that they take
 // outer steps per slice launch: the host looks at the columns after each

@@ -891,7 +891,7 @@ struct Slice {   // CPL: columns per lane
                         sh.gprev[(it + 1) & 1][c] = q;
                     }
                 }
-                __syncwarp(3 * NC == 32 ? 0xffffffffu : (1u << (3 * NC)) - 1u);
+                __syncwarp((1u << (3 * NC)) - 1u);
                 if (role == 0 && done) sh.skip[c] = 1;
             }
             __syncthreads();
