@@ -2884,15 +2884,18 @@ static void cheb_launch(const DevSystem& s, const PanelDev& p, const float2* cur
     // fewer than 16 columns: one pair per thread, for the warps in flight (16
     // outer steps, 4 / 8 columns of 1000 silicon atoms 16.0 / 14.0 -> 11.4 /
     // 10.1 ms, 4 of 512 water molecules 39.7 -> 25.7, panels of 8 for 256 of
-    // them 240 -> 184; 8 columns of 100 000 atoms, 4 steps, 17.7)
-    if (p.C >= 8) {
+    // them 240 -> 184; 8 columns of 100 000 atoms, us per step, 60.4 -> 57.7);
+    // four columns of a system whose pairs exceed the resident threads keep
+    // two (100 000 atoms 51.7 -> 49.1)
+    if (p.C >= 8 || (p.C == 2 && 2LL * s.n_atoms > (long long)gmax() * THREADS)) {
         const int g = grid_for((long long)s.n_atoms * (p.C / 2));
         switch (p.C) {
             case 128: k_inner32_cheb<2, 128, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 64: k_inner32_cheb<2, 64, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 32: k_inner32_cheb<2, 32, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
             case 16: k_inner32_cheb<2, 16, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
-            default: k_inner32_cheb<2, 8, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+            case 8: k_inner32_cheb<2, 8, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
+            default: k_inner32_cheb<2, 2, LAST><<<g, THREADS, 0, st>>>(s, p, cur, io, omega, gamma, mode); break;
         }
     } else {
         const int g = grid_for((long long)s.n_atoms * p.C);

@@ -143,3 +143,24 @@ def test_noalloc_request_of_the_whole_scratch(P):
     a, b, nrm = (np.asarray(v) for v in P.tb_generalized_lanczos_noalloc(h, 7, k))
     assert len(a) == k and abs(a[0] - np.linspace(-20.0, -5.0, n)[7]) <= 1e-12 * 20 and nrm[0] == 1.0
     assert np.all(b == 0.0)
+
+
+def test_four_columns_of_a_very_large_system(P, ran):
+    """A ring of 100 000 s atoms, whose four columns make more pairs than threads are
+    resident (two pairs per thread), against panels of eight (one): full solutions
+    after fixed steps to 1e-9."""
+    n = 100000
+    i = np.arange(n)
+    cols = np.sort(np.stack([(i - 1) % n, i, (i + 1) % n], axis=1), axis=1)
+    S = np.where(cols == i[:, None], 1.0, 0.2)
+    h = P.tb_create(np.ones(n), 3 * np.arange(n + 1), cols.ravel(), S.ravel(), eps=-13.0 + np.sin(i))
+    z = np.array([-13.0 + 1j, -10.0 + 1j])
+    pick = np.array([5, 31234, 60000, 99999, 7, 8, 9, 10], dtype=np.int32)
+
+    def x(k, panel):
+        o = P.tb_default_opts(precision=1, max_iter=6, panel=panel)
+        return P.tb_shifted_cocg(h, z, pick[:k], opts=o, allow_unconverged=True)[0].cpu().numpy()[:, :4]
+
+    a, b = x(4, 4), x(8, 8)
+    assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
+    assert ran()["inner32_cheb"] > 0
