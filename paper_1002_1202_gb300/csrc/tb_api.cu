@@ -1610,17 +1610,16 @@ std::vector<int> system_columns(const tb_handle* h, int R, const int32_t* cols) 
     return n;
 }
 
-// The most that f(columns of a panel, padded orbitals of its system) sums to
-// over the panels that can be in flight at once.
+// The most that f(columns of a panel, its system) sums to over the panels that
+// can be in flight at once.
 template <class F>
 double in_flight(const tb_handle* h, const std::vector<int>& ncols, int panel, int streams, F&& f) {
     std::vector<double> v;
     for (size_t s = 0; s < ncols.size(); ++s) {
         if (ncols[s] == 0) continue;
         const int P = std::min(panel, next_pow2(ncols[s]));
-        const int npad = 4 * (int)(h->sys_atom_off[s + 1] - h->sys_atom_off[s]);
         const int jobs = std::min((ncols[s] + P - 1) / P, streams);
-        v.insert(v.end(), jobs, f(P, npad));
+        v.insert(v.end(), jobs, f(P, (int)s));
     }
     std::sort(v.rbegin(), v.rend());
     double sum = 0.0;
@@ -2491,16 +2490,19 @@ tb_status tb_shifted_cocg(tb_handle* h, int32_t K, const double* z, int32_t R, c
     const int64_t N = h->n_orb;
     const bool host_out = !is_device_ptr(x_out);
     const double budget = (double)state_budget(opts), out_shift = host_out ? 16.0 * (double)R * N : 0.0;
-    const bool sliced = slices_on() && slice_system(h);
     const std::vector<int> ncols = system_columns(h, R, cols);
+    auto npad = [&](int s) { return 4 * (int)(h->sys_atom_off[s + 1] - h->sys_atom_off[s]); };
     auto state = [&](int panel, int streams) {   // of one shift
-        return in_flight(h, ncols, panel, streams, [](int P, int npad) { return 32.0 * npad * P; });
+        return in_flight(h, ncols, panel, streams, [&](int P, int s) { return 32.0 * npad(s) * P; });
     };
     auto blocks = [&](int panel, int streams, int k) {
-        if (!sliced) return 0.0;
-        return in_flight(h, ncols, panel, streams,
-                         [&](int P, int npad) { return block_bytes(std::max(P, 2), k, npad, false, SLICE_STEPS); });
+        if (!slices_on()) return 0.0;
+        return in_flight(h, ncols, panel, streams, [&](int P, int s) {
+            const bool small = h->sys_orb_off[s + 1] - h->sys_orb_off[s] <= SLICE_MAX_ROWS;
+            return small ? block_bytes(std::max(P, 2), k, npad(s), false, SLICE_STEPS) : 0.0;
+        });
     };
+    const bool sliced = blocks(64, 1, 1) > 0.0;   // some system of the call
     Solve qs;
     qs.K = K;
     Shape sh = call_shape(h, qs, opts, budget, [&](int panel, int streams) {

@@ -6,7 +6,7 @@ import ctypes
 import numpy as np
 import pytest
 
-from tbinputs import gauss_legendre_grid, si_system
+from tbinputs import gauss_legendre_grid, si_system, water_system
 
 pytestmark = pytest.mark.gpu
 
@@ -131,3 +131,15 @@ def test_wide_calls_stay_on_the_slices(P, which):
         P.tb_green_elements_dz(h, z, np.arange(256), ptr, rows, opts=P.tb_default_opts(precision=1, max_iter=4),
                                allow_unconverged=True)
     assert launches(P)["slice"] > n0
+
+
+def test_small_systems_beside_a_large_one_stay_on_the_slices(P):
+    """A batch of a system that the slices take and one that they do not."""
+    s, _ = system(P, 2, 2, 2)
+    hb = P.tb_create_batch([s, water_system(400, seed=4, excess_proton=False)])
+    hb_cols = [3, int(hb.orb_off[1]) + 5]
+    z, _ = gauss_legendre_grid(8, -40.0, 0.0, 1.0)
+    n0 = launches(P)
+    P.tb_shifted_cocg(hb, z, hb_cols, opts=P.tb_default_opts(precision=1, max_iter=4), allow_unconverged=True)
+    n1 = launches(P)
+    assert n1["slice"] > n0["slice"] and n1["inner32_cheb"] > n0["inner32_cheb"]
